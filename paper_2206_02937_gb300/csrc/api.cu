@@ -118,7 +118,7 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
     ctx->accepted_cap = P > ((int64_t)1 << 20) ? P : ((int64_t)1 << 20);
     size_t o_acc = cv.take<compton::AcceptedPair>(ctx->accepted_cap);
     size_t o_nacc = cv.take<uint32_t>(1);
-    size_t o_wacc = cv.take<uint32_t>(compton::kMaxProbWarps);
+    size_t o_wacc = cv.take<uint32_t>(compton::max_prob_warps(ctx->n_sm));
     size_t o_cand = cv.take<compton::CandPair>(ctx->accepted_cap);
     size_t o_ncand = cv.take<uint32_t>(1);
     size_t o_st = cv.take<compton::DeviceStats>(1);
@@ -136,7 +136,7 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
     }
     size_t o_tr = cv.take<uint8_t>(cfg->max_train_batch > 0 ? compton::train_scratch_bytes(cfg->max_train_batch) : 1);
     size_t o_rb = cv.take<float>(P > 0 ? P : 1);
-    size_t o_pn = cv.take<float>(4 * compton::kPnetParams + 2);
+    size_t o_pn = cv.take<float>(4 * compton::kPnetParams + 2 + compton::kPnetParams + 2 + 1);
     const size_t total = align_up(cv.used, 256);
     if (cfg->mem_budget_bytes && total > cfg->mem_budget_bytes) {
         delete ctx;
@@ -196,6 +196,8 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
         pn.adam_m = pb + 2 * compton::kPnetParams;
         pn.adam_v = pb + 3 * compton::kPnetParams;
         pn.loss = pb + 4 * compton::kPnetParams;
+        pn.acc = pn.loss + 2;
+        pn.ticket = reinterpret_cast<uint32_t*>(pn.acc + compton::kPnetParams + 2);
         pn.fs[0] = 1.0f;
         pn.fs[1] = 7.0f;
         pn.fs[2] = 1e-4f;

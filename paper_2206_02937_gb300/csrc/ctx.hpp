@@ -19,7 +19,12 @@ constexpr int kSortTile = 512;        // particles per sort tile (by cell start 
 constexpr int kSortCap = 640;         // particles a sort CTA holds in shared memory
 constexpr int kPairsPerTile = 1024;   // pairs per scatter CTA (256 threads x 4)
 constexpr int kCellWindow = 512;      // cells of a scatter tile staged in shared memory
-constexpr int kMaxProbWarps = 8192;   // warps of the probability kernel (their accepted counts)
+constexpr int kMaxProbWarps = 8192;   // warps of the probability kernel (their accepted counts) at most:
+inline int max_prob_warps(int n_sm)   // four CTAs of eight warps per SM
+{
+    const int64_t w = (int64_t)n_sm * 32;
+    return w < kMaxProbWarps ? (int)w : kMaxProbWarps;
+}
 
 // Per-cell record written by the scan and read by the scatter kernel.
 struct __align__(16) CellInfo {
@@ -137,6 +142,8 @@ struct PnetDev {
     float* adam_m;  // [kPnetParams]
     float* adam_v;  // [kPnetParams]
     float* loss;    // [2] weighted |error| sum, weight sum of the last step
+    float* acc;     // [kPnetParams + 2] sums of the step in flight (gradient, then loss), zero between steps
+    uint32_t* ticket;  // blocks of the step in flight that have added their sums, zero between steps
     float fs[4];    // feature scales s_u, n_u, s_k, n_k
     float range[3]; // training range: gamma^2 max, eps^2 min, eps^2 max
     int64_t step;   // Adam steps taken
@@ -175,7 +182,7 @@ struct compton_ctx {
     int64_t* n_pairs = nullptr;                  // device scalar
     compton::AcceptedPair* accepted = nullptr;   // [accepted_cap] pairs that passed their trial
     uint32_t* n_accepted = nullptr;              // device scalar
-    uint32_t* warp_acc = nullptr;                // [kMaxProbWarps] accepted pairs per probability region
+    uint32_t* warp_acc = nullptr;                // [max_prob_warps] accepted pairs per probability region
     int64_t accepted_cap = 0;                    // max(max_particles, 2^20)
     compton::CandPair* cand = nullptr;           // [accepted_cap] candidates of the surrogate modes
     uint32_t* n_cand = nullptr;                  // device scalar

@@ -17,11 +17,9 @@
 //                  particles, P_max = 2 n_p dt of the pair) with the decision
 //                  made in the same thread (analytic probability outside the
 //                  training range) and accepted pairs appended to the list;
-//   k_pnet_train   forward and backward per sample; each parameter's
-//                  gradient is summed over the warp by shuffles, then over
-//                  the block in shared memory, then once per block in global
-//                  memory;
-//   k_pnet_adam    Adam over the 337 parameters.
+//   k_pnet_train   one training step: forward and backward per sample, the
+//                  parameters' gradients as products of rows staged in shared
+//                  memory, and Adam by the block that finishes last.
 #include "ctx.hpp"
 #include "device_math.cuh"
 #include "features.cuh"
@@ -55,7 +53,6 @@ struct PnetArgs {
     // training
     const float* y;
     const float* wts;
-    float* loss;  // [2] weighted |error| sum, weight sum
 };
 
 __device__ __forceinline__ void pnet_features(const PnetDev& p, const float* q, float lwe, float lwg, float lpm,
@@ -199,110 +196,162 @@ __global__ void __launch_bounds__(kPnetThreads, 3) k_pnet_infer(PnetArgs a)
     }
 }
 
-// Adds v summed over the warp to acc (lane 0 does the add).
-__device__ __forceinline__ void warp_add(float* acc, float v)
+// Training step: gradient, loss and Adam in one launch.
+//
+// A tile of kS samples per pass: one thread per sample runs the forward and
+// backward passes and leaves the sample's 70 vector components (inputs, hidden
+// activations, deltas) as rows of shared memory; then every parameter's
+// gradient is a dot product of two of those rows over the tile, one thread per
+// parameter (the loss and the weight sum are two more such sums), so nothing
+// is reduced by shuffles and no two threads add to the same word.  The rows
+// are kS + 4 words apart: the eight lanes of a 16-byte shared load read
+// neighbouring rows, which then lie in different banks.  A tile's sums are
+// added to the thread's running sums once (two levels, as short as the tile).
+// Each block adds its sums to acc; the block that finishes last (a ticket)
+// takes them as the step's gradient, runs Adam and clears acc and the ticket
+// for the next step, so a step needs no memset and no second launch.
+//
+// What bounds it: at a minibatch of 8192 the latency of one tile's chain (about
+// 600 dependent multiply-adds, then 16 steps of the row products).
+constexpr int kTrainSums = kPnetParams + 2;  // gradients, weighted |error| sum, weight sum
+constexpr int kTrainThreads = 352;           // a thread per sum, whole warps
+constexpr int kRowF = 0, kRowH1 = 9, kRowH2 = 18, kRowH3 = 30, kRowD0 = 39, kRowD1 = 48, kRowD2 = 60, kRowD3 = 69,
+              kRowLoss = 70, kRowW = 71, kRowOne = 72, kTrainRows = 73;
+static_assert(kTrainSums <= kTrainThreads, "a thread per sum");
+
+// The two rows whose product sums to entry p of acc.
+__device__ __forceinline__ void train_rows(int p, int& ra, int& rb)
 {
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) v += __shfl_xor_sync(0xffffffffu, v, d);
-    if ((threadIdx.x & 31u) == 0) atomicAdd(acc, v);
+    rb = kRowOne;
+    if (p < kP_B0) { ra = kRowD0 + p / 9; rb = kRowF + p % 9; }
+    else if (p < kP_W1) ra = kRowD0 + (p - kP_B0);
+    else if (p < kP_B1) { ra = kRowD1 + (p - kP_W1) / 9; rb = kRowH1 + (p - kP_W1) % 9; }
+    else if (p < kP_W2) ra = kRowD1 + (p - kP_B1);
+    else if (p < kP_B2) { ra = kRowD2 + (p - kP_W2) / 12; rb = kRowH2 + (p - kP_W2) % 12; }
+    else if (p < kP_W3) ra = kRowD2 + (p - kP_B2);
+    else if (p < kP_B3) { ra = kRowD3; rb = kRowH3 + (p - kP_W3); }
+    else if (p == kP_B3) ra = kRowD3;
+    else ra = p == kPnetParams ? kRowLoss : kRowW;
 }
 
-__global__ void __launch_bounds__(kPnetThreads, 2) k_pnet_train(PnetArgs a)
+template <int kS>
+__global__ void __launch_bounds__(kTrainThreads, 1) k_pnet_train(PnetArgs a, float lr, float b1t, float b2t)
 {
+    constexpr int kStride = kS + 4;
+    extern __shared__ __align__(16) float rows[];  // [kTrainRows][kStride]
     __shared__ float th[kPnetParams];
-    __shared__ float g[kPnetParams];
-    for (int i = threadIdx.x; i < kPnetParams; i += blockDim.x) g[i] = 0.0f;
+    __shared__ bool last;
+    const int tid = threadIdx.x;
+    for (int i = tid; i < kS; i += kTrainThreads) rows[kRowOne * kStride + i] = 1.0f;
     stage_params(a.p, th);
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t first = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31u);
-    const unsigned lane = threadIdx.x & 31u;
-    float loss_num = 0.0f, wsum = 0.0f;
-    for (int64_t base = first; base < a.n; base += stride) {
-        const int64_t s = base + lane;
-        const bool live = s < a.n;
-        float q[6] = {0, 0, 0, 0, 0, 0};
-        float y = 0.0f, wt = 0.0f;
-        if (live) {
-            q[0] = a.u[0][s];
-            q[1] = a.u[1][s];
-            q[2] = a.u[2][s];
-            q[3] = a.k[0][s];
-            q[4] = a.k[1][s];
-            q[5] = a.k[2][s];
-            y = a.y[s];
-            wt = a.wts ? a.wts[s] : 1.0f;
+    int ra = 0, rb = 0;
+    if (tid < kTrainSums) train_rows(tid, ra, rb);
+    const float4* va = reinterpret_cast<const float4*>(rows + ra * kStride);
+    const float4* vb = reinterpret_cast<const float4*>(rows + rb * kStride);
+    float sum = 0.0f;
+    for (int64_t base = (int64_t)blockIdx.x * kS; base < a.n; base += (int64_t)gridDim.x * kS) {
+        if (tid < kS) {
+            const int64_t s = base + tid;
+            float q[6] = {0, 0, 0, 0, 0, 0};
+            float y = 0.0f, wt = 0.0f;
+            if (s < a.n) {
+                q[0] = a.u[0][s];
+                q[1] = a.u[1][s];
+                q[2] = a.u[2][s];
+                q[3] = a.k[0][s];
+                q[4] = a.k[1][s];
+                q[5] = a.k[2][s];
+                y = a.y[s];
+                wt = a.wts ? a.wts[s] : 1.0f;
+            }
+            float* col = rows + tid;
+            auto put = [&](int r, float v) { col[r * kStride] = v; };
+            float f[9], h1[9], h2[12], h3[9];
+            pnet_features(a.p, q, a.ln_we, a.ln_wg, a.ln_pmax, f);
+            const float yp = pnet_forward(th, f, h1, h2, h3);
+            // the weights are read from shared memory again in the backward
+            // pass (kept in registers they spill)
+            asm volatile("" ::: "memory");
+            const float err = yp - y;
+            put(kRowLoss, wt * fabsf(err));
+            put(kRowW, wt);
+            // d loss / d z of the output times sum w: w sign(err) sigma'(z)
+            // (Adam divides by the weight sum)
+            const float sgn = err > 0.0f ? 1.0f : (err < 0.0f ? -1.0f : 0.0f);
+            const float dz3 = wt * sgn * yp * (1.0f - yp);
+            put(kRowD3, dz3);
+            float dz2[9], dz1[12];
+#pragma unroll
+            for (int o = 0; o < 9; ++o) {
+                dz2[o] = h3[o] > 0.0f ? dz3 * th[kP_W3 + o] : 0.0f;
+                put(kRowF + o, f[o]);
+                put(kRowH1 + o, h1[o]);
+                put(kRowH3 + o, h3[o]);
+                put(kRowD2 + o, dz2[o]);
+            }
+#pragma unroll
+            for (int i = 0; i < 12; ++i) {
+                float d = 0.0f;
+#pragma unroll
+                for (int o = 0; o < 9; ++o) d = fmaf(th[kP_W2 + 12 * o + i], dz2[o], d);
+                dz1[i] = h2[i] > 0.0f ? d : 0.0f;
+                put(kRowH2 + i, h2[i]);
+                put(kRowD1 + i, dz1[i]);
+            }
+#pragma unroll
+            for (int i = 0; i < 9; ++i) {
+                float d = 0.0f;
+#pragma unroll
+                for (int o = 0; o < 12; ++o) d = fmaf(th[kP_W1 + 9 * o + i], dz1[o], d);
+                put(kRowD0 + i, h1[i] > 0.0f ? d : 0.0f);
+            }
         }
-        float f[9], h1[9], h2[12], h3[9];
-        pnet_features(a.p, q, a.ln_we, a.ln_wg, a.ln_pmax, f);
-        const float yp = pnet_forward(th, f, h1, h2, h3);
-        const float err = yp - y;
-        loss_num += wt * fabsf(err);
-        wsum += wt;
-        // d loss / d z of the output times sum w: w sign(err) sigma'(z) (the
-        // Adam kernel divides by the weight sum)
-        const float sgn = err > 0.0f ? 1.0f : (err < 0.0f ? -1.0f : 0.0f);
-        const float dz3 = wt * sgn * yp * (1.0f - yp);
-        // output layer
-#pragma unroll
-        for (int i = 0; i < 9; ++i) warp_add(&g[kP_W3 + i], dz3 * h3[i]);
-        warp_add(&g[kP_B3], dz3);
-        float dz2[9];
-#pragma unroll
-        for (int o = 0; o < 9; ++o) dz2[o] = h3[o] > 0.0f ? dz3 * th[kP_W3 + o] : 0.0f;
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-#pragma unroll
-            for (int i = 0; i < 12; ++i) warp_add(&g[kP_W2 + 12 * o + i], dz2[o] * h2[i]);
-            warp_add(&g[kP_B2 + o], dz2[o]);
+        __syncthreads();
+        if (tid < kTrainSums) {
+            float t0 = 0.0f, t1 = 0.0f, t2 = 0.0f, t3 = 0.0f;
+#pragma unroll 8
+            for (int i = 0; i < kS / 4; ++i) {
+                const float4 x = va[i], z = vb[i];
+                t0 = fmaf(x.x, z.x, t0);
+                t1 = fmaf(x.y, z.y, t1);
+                t2 = fmaf(x.z, z.z, t2);
+                t3 = fmaf(x.w, z.w, t3);
+            }
+            sum += (t0 + t1) + (t2 + t3);
         }
-        float dz1[12];
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-            float d = 0.0f;
-#pragma unroll
-            for (int o = 0; o < 9; ++o) d = fmaf(th[kP_W2 + 12 * o + i], dz2[o], d);
-            dz1[i] = h2[i] > 0.0f ? d : 0.0f;
-        }
-#pragma unroll
-        for (int o = 0; o < 12; ++o) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) warp_add(&g[kP_W1 + 9 * o + i], dz1[o] * h1[i]);
-            warp_add(&g[kP_B1 + o], dz1[o]);
-        }
-        float dz0[9];
-#pragma unroll
-        for (int i = 0; i < 9; ++i) {
-            float d = 0.0f;
-#pragma unroll
-            for (int o = 0; o < 12; ++o) d = fmaf(th[kP_W1 + 9 * o + i], dz1[o], d);
-            dz0[i] = h1[i] > 0.0f ? d : 0.0f;
-        }
-#pragma unroll
-        for (int o = 0; o < 9; ++o) {
-#pragma unroll
-            for (int i = 0; i < 9; ++i) warp_add(&g[kP_W0 + 9 * o + i], dz0[o] * f[i]);
-            warp_add(&g[kP_B0 + o], dz0[o]);
-        }
+        __syncthreads();
     }
-    warp_add(&a.loss[0], loss_num);
-    warp_add(&a.loss[1], wsum);
+    if (tid < kTrainSums) atomicAdd(&a.p.acc[tid], sum);
+    __threadfence();
     __syncthreads();
-    for (int i = threadIdx.x; i < kPnetParams; i += blockDim.x) atomicAdd(&a.p.grad[i], g[i]);
+    if (tid == 0) last = atomicAdd(a.p.ticket, 1u) == gridDim.x - 1;
+    __syncthreads();
+    if (!last) return;
+    // the sums of every block are in acc: Adam (beta 0.9, 0.999) on the mean over the weights
+    __threadfence();
+    const float wsum = __ldcg(&a.p.acc[kPnetParams + 1]);
+    if (tid < kPnetParams) {
+        const float gr = __ldcg(&a.p.acc[tid]) / wsum;
+        a.p.grad[tid] = gr;
+        const float m = 0.9f * a.p.adam_m[tid] + 0.1f * gr;
+        const float v = 0.999f * a.p.adam_v[tid] + 0.001f * gr * gr;
+        a.p.adam_m[tid] = m;
+        a.p.adam_v[tid] = v;
+        const float mh = m / (1.0f - b1t), vh = v / (1.0f - b2t);
+        a.p.theta[tid] -= lr * mh / (sqrtf(vh) + 1e-7f);
+    } else if (tid < kTrainSums) {
+        a.p.loss[tid - kPnetParams] = __ldcg(&a.p.acc[tid]);
+    }
+    __syncthreads();
+    if (tid < kTrainSums) a.p.acc[tid] = 0.0f;
+    if (tid == 0) *a.p.ticket = 0u;
 }
 
-__global__ void k_pnet_adam(PnetDev p, float lr, float b1t, float b2t)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kPnetParams) return;
-    const float gr = p.grad[i] / p.loss[1];  // mean over the weights
-    p.grad[i] = gr;
-    const float m = 0.9f * p.adam_m[i] + 0.1f * gr;
-    const float v = 0.999f * p.adam_v[i] + 0.001f * gr * gr;
-    p.adam_m[i] = m;
-    p.adam_v[i] = v;
-    const float mh = m / (1.0f - b1t), vh = v / (1.0f - b2t);
-    p.theta[i] -= lr * mh / (sqrtf(vh) + 1e-7f);
-}
+// Samples per tile: 64, so that a minibatch of 8192 reaches 128 SMs, while
+// every block has at most two tiles; beyond that 320 (ten of a block's eleven
+// warps in the per-sample pass).
+constexpr int kTrainTile = 64, kTrainTileBig = 320;
+constexpr size_t train_smem(int s) { return sizeof(float) * kTrainRows * (s + 4); }
 
 int pnet_grid(int64_t rows)
 {
@@ -378,8 +427,6 @@ compton_status launch_pnet_train_step(compton_ctx* ctx, const float* ux, const f
 {
     if (n <= 0) return COMPTON_EINVAL;
     PnetDev& P = ctx->pnet;
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(P.grad, 0, sizeof(float) * kPnetParams, stream));
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(P.loss, 0, sizeof(float) * 2, stream));
     PnetArgs a{};
     a.p = P;
     a.u[0] = ux;
@@ -394,13 +441,23 @@ compton_status launch_pnet_train_step(compton_ctx* ctx, const float* ux, const f
     a.ln_pmax = logf(p_max);
     a.y = y;
     a.wts = w;
-    a.loss = P.loss;
-    k_pnet_train<<<pnet_grid(n), kPnetThreads, 0, stream>>>(a);
-    COMPTON_LAUNCH_CHECK(ctx, "k_pnet_train");
-    ++P.step;
-    const float b1t = powf(0.9f, (float)P.step), b2t = powf(0.999f, (float)P.step);
-    k_pnet_adam<<<(kPnetParams + 127) / 128, 128, 0, stream>>>(P, lr, b1t, b2t);
-    COMPTON_LAUNCH_CHECK(ctx, "k_pnet_adam");
+    const int64_t step = P.step + 1;
+    const float b1t = powf(0.9f, (float)step), b2t = powf(0.999f, (float)step);
+    const bool big = n > (int64_t)2 * ctx->n_sm * kTrainTile;
+    const int tile = big ? kTrainTileBig : kTrainTile;
+    const int64_t tiles = (n + tile - 1) / tile;
+    const unsigned grid = (unsigned)(tiles < ctx->n_sm ? tiles : ctx->n_sm);
+    const int smem = (int)train_smem(tile);
+    if (big)
+        COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_pnet_train<kTrainTileBig>,
+                                                   cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+    // the launch is the whole step: an injected failure comes before it, so that no failed call has updated anything
+    if (inject_fault()) return set_injected_error(ctx, "k_pnet_train");
+    if (big) k_pnet_train<kTrainTileBig><<<grid, kTrainThreads, smem, stream>>>(a, lr, b1t, b2t);
+    else k_pnet_train<kTrainTile><<<grid, kTrainThreads, smem, stream>>>(a, lr, b1t, b2t);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "k_pnet_train");
+    P.step = step;
     return COMPTON_OK;
 }
 

@@ -804,13 +804,9 @@ __global__ void k_sample_angle(const float* __restrict__ x, const uint32_t* __re
 
 // Persistent probability kernel: at most the CTAs resident at once (four
 // per SM).
-unsigned prob_grid(unsigned tiles)
+unsigned prob_grid(const compton_ctx* ctx, unsigned tiles)
 {
-    int dev = 0, n_sm = 1;
-    cudaGetDevice(&dev);
-    if (cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm < 1) n_sm = 1;
-    if (n_sm > kMaxProbWarps / (4 * kProbWarps)) n_sm = kMaxProbWarps / (4 * kProbWarps);
-    const unsigned cap = (unsigned)n_sm * 4u;
+    const unsigned cap = (unsigned)(max_prob_warps(ctx->n_sm) / kProbWarps);
     return tiles < 1u ? 1u : (tiles < cap ? tiles : cap);
 }
 
@@ -873,7 +869,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
 {
     COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->n_accepted, 0, sizeof(uint32_t), stream));
     if (mode == COMPTON_MODE_PLAIN) {
-        const unsigned grid = prob_grid(tiles);
+        const unsigned grid = prob_grid(ctx, tiles);
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
             k_pair_prob<kBinned, kWeighted><<<grid, kProbThreads, 0, stream>>>(a);
@@ -892,7 +888,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
             // the candidate filter of the plain kernel, candidates to the list
-            k_pair_prob<kBinned, kWeighted, true><<<prob_grid(tiles), kProbThreads, 0, stream>>>(a);
+            k_pair_prob<kBinned, kWeighted, true><<<prob_grid(ctx, tiles), kProbThreads, 0, stream>>>(a);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob<cand>");
         // tensor-core modes and the paper's network decide inside the network

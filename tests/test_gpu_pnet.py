@@ -86,6 +86,38 @@ def test_gradient_and_adam_match_oracle(n, weighted):
     assert np.all(np.abs(step_gpu) <= lr * (1.0 + 1e-5) + 1e-7 * np.abs(th64))
 
 
+@pytest.mark.parametrize("n,weighted", [(1, False), (64, True), (65, False), (19456, True), (19457, True), (50001, False)])
+def test_training_step_at_tile_edges(n, weighted):
+    """Two consecutive steps at the edges of the sample tiles (64; 320 above
+    two tiles of 64 per SM of 152): each step's gradient and loss against the
+    oracle at the parameters the step started from."""
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    cg.build()
+    u, k = wl.c3(n, seed=75)
+    rng = np.random.default_rng(76)
+    y = rng.uniform(0.02, 0.98, n)
+    w = rng.uniform(0.5, 2.0, n) if weighted else None
+    ctx = _ctx(cg, n)
+    try:
+        cg.compton_pnet_set_params(ctx, opn.init_params(9).astype(np.float32))
+        ut, kt, yt, wt = _cuda(torch, u, k, y, w)
+        f = opn.features(u.astype(np.float64), k.astype(np.float64), W_E, W_G, P_MAX)
+        y64 = y.astype(np.float32).astype(np.float64)
+        w64 = None if w is None else w.astype(np.float32).astype(np.float64)
+        for _ in range(2):
+            th = cg.compton_pnet_get_params(ctx)[0].astype(np.float64)
+            loss = cg.compton_pnet_train_step(ctx, ut, kt, yt, wt, W_E, W_G, P_MAX, lr=1e-3)
+            g_gpu = cg.compton_pnet_get_params(ctx)[1].astype(np.float64)
+            loss_ref, g_ref = opn.backward(th, f, y64, w64)
+            assert loss == pytest.approx(loss_ref, rel=1e-5)
+            for (Wg, bg), (Wr, br) in zip(opn.unpack(g_gpu), opn.unpack(g_ref)):
+                assert np.linalg.norm(Wg - Wr) <= 1e-4 * np.linalg.norm(Wr) + 1e-9
+                assert np.linalg.norm(bg - br) <= 1e-4 * np.linalg.norm(br) + 1e-9
+    finally:
+        cg.compton_destroy(ctx)
+
+
 def test_training_learns_the_analytic_ratio():
     import paper_2206_02937_gb300 as cg
     torch = torch_cuda()
