@@ -96,15 +96,35 @@ def strerror(status: int) -> str:
     return lib().compton_strerror(int(status)).decode()
 
 
-def _stream_ptr(stream):
-    if stream is None:
-        import torch
-        stream = torch.cuda.current_stream()
-    return c_p(stream.cuda_stream)
+# A call's marshalling runs on the caller's thread before every launch, and a
+# training or inference call's kernels take 10 to 30 us: pointers go to ctypes
+# as plain integers (no c_void_p objects), the rows of a (3, n) tensor are
+# addressed from its base and stride instead of three indexed views (1.2 us
+# each), and the current stream's handle is read without building a Stream
+# object.  A compton_pnet_train_step call: 23 -> 7 us on the host.
+def _stream_ptr(stream) -> int:
+    if stream is not None:
+        return stream.cuda_stream
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
 
 
-def _ptr(t):
-    return c_p(0) if t is None else c_p(t.data_ptr())
+def _ptr(t) -> int:
+    return 0 if t is None else t.data_ptr()
+
+
+def _rows(t) -> tuple:
+    """Addresses of t[0], t[1], t[2]."""
+    try:
+        rows, base, stride = t.shape[0], t.data_ptr(), t.stride(0) * t.element_size()
+    except AttributeError:  # three tensors in a list
+        return _ptr(t[0]), _ptr(t[1]), _ptr(t[2])
+    if rows < 3:
+        t[2]  # raises IndexError
+    return base, base + stride, base + 2 * stride
 
 
 def _check(st: int, what: str, ctx=None):
@@ -155,17 +175,17 @@ def compton_init(n_cells: int, max_particles: int, w_over_v: float, dt: float, s
 
 
 def compton_destroy(ctx: int) -> None:
-    _check(lib().compton_destroy(c_p(ctx)), "compton_destroy")
+    _check(lib().compton_destroy(ctx), "compton_destroy")
 
 
 def compton_check(ctx: int, stream=None) -> int:
     """Returns the status (does not raise on ERANGE)."""
-    return lib().compton_check(c_p(ctx), _stream_ptr(stream))
+    return lib().compton_check(ctx, _stream_ptr(stream))
 
 
 def compton_get_stats(ctx: int, reset: bool = False, stream=None) -> dict:
     s = compton_stats()
-    _check(lib().compton_get_stats(c_p(ctx), ctypes.byref(s), int(reset), _stream_ptr(stream)),
+    _check(lib().compton_get_stats(ctx, ctypes.byref(s), int(reset), _stream_ptr(stream)),
            "compton_get_stats", ctx)
     return dict(pairs_tested=s.pairs_tested, scatters=s.scatters, mlp_fallbacks=s.mlp_fallbacks,
                 error_flags=s.error_flags)
@@ -175,7 +195,7 @@ def compton_bin_pairs(ctx: int, e_in: Species, g_in: Species, e_out: Species, g_
                       stream=None) -> compton_pairs:
     pairs = compton_pairs()
     ei, gi, eo, go = e_in.c(), g_in.c(), e_out.c(), g_out.c()
-    _check(lib().compton_bin_pairs(c_p(ctx), ctypes.byref(ei), ctypes.byref(gi), ctypes.byref(eo),
+    _check(lib().compton_bin_pairs(ctx, ctypes.byref(ei), ctypes.byref(gi), ctypes.byref(eo),
                                    ctypes.byref(go), int(step), ctypes.byref(pairs), _stream_ptr(stream)),
            "compton_bin_pairs", ctx)
     return pairs
@@ -184,7 +204,7 @@ def compton_bin_pairs(ctx: int, e_in: Species, g_in: Species, e_out: Species, g_
 def compton_scatter_step(ctx: int, e: Species, g: Species, pairs: compton_pairs, mode: int, step: int,
                          prob_out=None, flag_out=None, stream=None) -> None:
     ec, gc = e.c(), g.c()
-    _check(lib().compton_scatter_step(c_p(ctx), ctypes.byref(ec), ctypes.byref(gc), ctypes.byref(pairs),
+    _check(lib().compton_scatter_step(ctx, ctypes.byref(ec), ctypes.byref(gc), ctypes.byref(pairs),
                                       int(mode), int(step), _ptr(prob_out), _ptr(flag_out),
                                       _stream_ptr(stream)), "compton_scatter_step", ctx)
 
@@ -198,7 +218,7 @@ def compton_scatter_step_ntc(ctx: int, e: Species, g: Species, pairs: compton_pa
                              stream=None) -> None:
     """No-Time-Counter collisions of the binned species, in place."""
     ec, gc = e.c(), g.c()
-    _check(lib().compton_scatter_step_ntc(c_p(ctx), ctypes.byref(ec), ctypes.byref(gc), ctypes.byref(pairs),
+    _check(lib().compton_scatter_step_ntc(ctx, ctypes.byref(ec), ctypes.byref(gc), ctypes.byref(pairs),
                                           int(step), _stream_ptr(stream)), "compton_scatter_step_ntc", ctx)
 
 
@@ -206,21 +226,20 @@ def compton_scatter_pairs(ctx: int, u, k, n_dens, seed: int, step: int, mode: in
                           prob_out=None, flag_out=None, stream=None) -> None:
     """u, k: (3, n) float32 CUDA tensors (rows contiguous), updated in place."""
     n = int(u.shape[1])
-    _check(lib().compton_scatter_pairs(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                       _ptr(k[2]), _ptr(n_dens), n, int(seed), int(step), int(mode),
+    _check(lib().compton_scatter_pairs(ctx, *_rows(u), *_rows(k), _ptr(n_dens), n, int(seed), int(step), int(mode),
                                        _ptr(prob_out), _ptr(flag_out), _stream_ptr(stream)),
            "compton_scatter_pairs", ctx)
 
 
 def compton_kn_ratio(ctx: int, u, k, r_out, stream=None) -> None:
     n = int(u.shape[1])
-    _check(lib().compton_kn_ratio(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                  _ptr(k[2]), n, _ptr(r_out), _stream_ptr(stream)), "compton_kn_ratio", ctx)
+    _check(lib().compton_kn_ratio(ctx, *_rows(u), *_rows(k), n, _ptr(r_out), _stream_ptr(stream)),
+           "compton_kn_ratio", ctx)
 
 
 def compton_kn_sample_angle(ctx: int, x, r, cth_out, sth_out, ratio_out, stream=None) -> None:
     n = int(x.shape[0])
-    _check(lib().compton_kn_sample_angle(c_p(ctx), _ptr(x), _ptr(r), n, _ptr(cth_out), _ptr(sth_out),
+    _check(lib().compton_kn_sample_angle(ctx, _ptr(x), _ptr(r), n, _ptr(cth_out), _ptr(sth_out),
                                          _ptr(ratio_out), _stream_ptr(stream)), "compton_kn_sample_angle", ctx)
 
 
@@ -246,7 +265,7 @@ def _host_f32(a):
 def compton_mlp_set_params(ctx: int, theta, feature_scales=None) -> None:
     th = _host_f32(theta)
     fs = None if feature_scales is None else _host_f32(feature_scales)
-    _check(lib().compton_mlp_set_params(c_p(ctx), c_p(th.ctypes.data), int(th.shape[0]),
+    _check(lib().compton_mlp_set_params(ctx, c_p(th.ctypes.data), int(th.shape[0]),
                                         c_p(0) if fs is None else c_p(fs.ctypes.data)),
            "compton_mlp_set_params", ctx)
 
@@ -254,42 +273,40 @@ def compton_mlp_set_params(ctx: int, theta, feature_scales=None) -> None:
 def compton_mlp_get_params(ctx: int):
     import numpy as np
     th = np.zeros(N_MLP_PARAMS, dtype=np.float32)
-    _check(lib().compton_mlp_get_params(c_p(ctx), c_p(th.ctypes.data), N_MLP_PARAMS), "compton_mlp_get_params", ctx)
+    _check(lib().compton_mlp_get_params(ctx, c_p(th.ctypes.data), N_MLP_PARAMS), "compton_mlp_get_params", ctx)
     return th
 
 
 def compton_mlp_calibrate(ctx: int, u, k, stream=None) -> None:
     n = int(u.shape[1])
-    _check(lib().compton_mlp_calibrate(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                       _ptr(k[2]), n, _stream_ptr(stream)), "compton_mlp_calibrate", ctx)
+    _check(lib().compton_mlp_calibrate(ctx, *_rows(u), *_rows(k), n, _stream_ptr(stream)),
+           "compton_mlp_calibrate", ctx)
 
 
 def compton_mlp_infer(ctx: int, u, k, mode: int, r_out, stream=None) -> None:
     n = int(u.shape[1])
-    _check(lib().compton_mlp_infer(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                   _ptr(k[2]), n, int(mode), _ptr(r_out), _stream_ptr(stream)),
+    _check(lib().compton_mlp_infer(ctx, *_rows(u), *_rows(k), n, int(mode), _ptr(r_out), _stream_ptr(stream)),
            "compton_mlp_infer", ctx)
 
 
 def compton_mlp_save(ctx: int) -> bytes:
     n = ctypes.c_size_t(0)
-    _check(lib().compton_mlp_save(c_p(ctx), c_p(0), ctypes.byref(n)), "compton_mlp_save", ctx)
+    _check(lib().compton_mlp_save(ctx, c_p(0), ctypes.byref(n)), "compton_mlp_save", ctx)
     buf = ctypes.create_string_buffer(n.value)
-    _check(lib().compton_mlp_save(c_p(ctx), ctypes.cast(buf, c_p), ctypes.byref(n)), "compton_mlp_save", ctx)
+    _check(lib().compton_mlp_save(ctx, ctypes.cast(buf, c_p), ctypes.byref(n)), "compton_mlp_save", ctx)
     return buf.raw[:n.value]
 
 
 def compton_mlp_load(ctx: int, blob: bytes) -> None:
     buf = ctypes.create_string_buffer(blob, len(blob))
-    _check(lib().compton_mlp_load(c_p(ctx), ctypes.cast(buf, c_p), len(blob)), "compton_mlp_load", ctx)
+    _check(lib().compton_mlp_load(ctx, ctypes.cast(buf, c_p), len(blob)), "compton_mlp_load", ctx)
 
 
 def compton_mlp_train_step(ctx: int, u, k, y, w, lr: float = 1e-3, want_loss: bool = True, stream=None):
     """One Adam step on a minibatch; returns the minibatch loss (synchronising) or None."""
     n = int(u.shape[1])
     loss = c_f32(0.0)
-    _check(lib().compton_mlp_train_step(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                        _ptr(k[2]), _ptr(y), _ptr(w), n, float(lr),
+    _check(lib().compton_mlp_train_step(ctx, *_rows(u), *_rows(k), _ptr(y), _ptr(w), n, float(lr),
                                         ctypes.byref(loss) if want_loss else None, _stream_ptr(stream)),
            "compton_mlp_train_step", ctx)
     return float(loss.value) if want_loss else None
@@ -301,7 +318,7 @@ SIGNATURES["compton_mlp_get_grad"] = (c_i32, [c_p, c_p, c_i64])
 def compton_mlp_get_grad(ctx: int):
     import numpy as np
     g = np.zeros(N_MLP_PARAMS, dtype=np.float32)
-    _check(lib().compton_mlp_get_grad(c_p(ctx), c_p(g.ctypes.data), N_MLP_PARAMS), "compton_mlp_get_grad", ctx)
+    _check(lib().compton_mlp_get_grad(ctx, c_p(g.ctypes.data), N_MLP_PARAMS), "compton_mlp_get_grad", ctx)
     return g
 
 
@@ -326,11 +343,11 @@ SIGNATURES.update({
 
 
 def compton_serve_start(ctx: int, pool_bytes: int, max_active: int = 1024) -> None:
-    _check(lib().compton_serve_start(c_p(ctx), int(pool_bytes), int(max_active)), "compton_serve_start", ctx)
+    _check(lib().compton_serve_start(ctx, int(pool_bytes), int(max_active)), "compton_serve_start", ctx)
 
 
 def compton_serve_stop(ctx: int) -> None:
-    _check(lib().compton_serve_stop(c_p(ctx)), "compton_serve_stop", ctx)
+    _check(lib().compton_serve_stop(ctx), "compton_serve_stop", ctx)
 
 
 def compton_submit(ctx: int, u_in, k_in, u_out, k_out, n_dens, seed: int, step: int = 0,
@@ -339,18 +356,17 @@ def compton_submit(ctx: int, u_in, k_in, u_out, k_out, n_dens, seed: int, step: 
     n_dens: a float or an (n,) float32 CUDA tensor.  Returns the ticket."""
     n = int(u_in.shape[1])
     dens_ptr, dens_val = (c_p(0), float(n_dens)) if isinstance(n_dens, (int, float)) else (_ptr(n_dens), 0.0)
-    r = compton_request(*[_ptr(t) for t in (u_in[0], u_in[1], u_in[2], k_in[0], k_in[1], k_in[2],
-                                            u_out[0], u_out[1], u_out[2], k_out[0], k_out[1], k_out[2])],
-                        dens_ptr, dens_val, n, int(seed), int(step), int(mode))
+    r = compton_request(*_rows(u_in), *_rows(k_in), *_rows(u_out), *_rows(k_out), dens_ptr, dens_val, n, int(seed),
+                        int(step), int(mode))
     t = c_u64(0)
-    _check(lib().compton_submit(c_p(ctx), ctypes.byref(r), ctypes.byref(t)), "compton_submit", ctx)
+    _check(lib().compton_submit(ctx, ctypes.byref(r), ctypes.byref(t)), "compton_submit", ctx)
     return int(t.value)
 
 
 def compton_poll(ctx: int, ticket: int):
     """None while the request is running, else a dict with its result."""
     res = compton_result()
-    st = lib().compton_poll(c_p(ctx), int(ticket), ctypes.byref(res))
+    st = lib().compton_poll(ctx, int(ticket), ctypes.byref(res))
     if st == COMPTON_ENOTREADY:
         return None
     _check(st, "compton_poll", ctx)
@@ -359,7 +375,7 @@ def compton_poll(ctx: int, ticket: int):
 
 def compton_serve_info(ctx: int) -> dict:
     a, b, c = c_u64(0), c_u64(0), c_u64(0)
-    _check(lib().compton_serve_info(c_p(ctx), ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
+    _check(lib().compton_serve_info(ctx, ctypes.byref(a), ctypes.byref(b), ctypes.byref(c)),
            "compton_serve_info", ctx)
     return dict(in_use=a.value, peak=b.value, pool=c.value)
 
@@ -388,7 +404,7 @@ def compton_mlp_balance_weights(ctx: int, r, edges, w_out, stream=None) -> None:
     """r: float32 CUDA tensor; edges: n_bins + 1 increasing host floats."""
     import numpy as np
     e = np.ascontiguousarray(edges, dtype=np.float32)
-    _check(lib().compton_mlp_balance_weights(c_p(ctx), _ptr(r), int(r.shape[0]), c_p(e.ctypes.data),
+    _check(lib().compton_mlp_balance_weights(ctx, _ptr(r), int(r.shape[0]), c_p(e.ctypes.data),
                                              int(e.shape[0] - 1), _ptr(w_out), _stream_ptr(stream)),
            "compton_mlp_balance_weights", ctx)
 
@@ -399,7 +415,7 @@ SIGNATURES["compton_mlp_set_train_precision"] = (c_i32, [c_p, c_i32])
 def compton_mlp_set_train_precision(ctx: int, mode: int) -> None:
     """Training arithmetic: MODE_MLP_FP32 (CUDA cores, the default) or
     MODE_MLP_BF16 (tcgen05 tensor cores, BF16 operands, FP32 accumulation)."""
-    _check(lib().compton_mlp_set_train_precision(c_p(ctx), int(mode)), "compton_mlp_set_train_precision", ctx)
+    _check(lib().compton_mlp_set_train_precision(ctx, int(mode)), "compton_mlp_set_train_precision", ctx)
 
 
 SIGNATURES["compton_mlp_set_features"] = (c_i32, [c_p, c_i32])
@@ -408,13 +424,13 @@ SIGNATURES["compton_mlp_set_range"] = (c_i32, [c_p, c_f64, c_f64, c_f64])
 
 def compton_mlp_set_range(ctx: int, gamma_max: float, eps_min: float, eps_max: float) -> None:
     """Training range of the network (outside it: analytic probability)."""
-    _check(lib().compton_mlp_set_range(c_p(ctx), float(gamma_max), float(eps_min), float(eps_max)),
+    _check(lib().compton_mlp_set_range(ctx, float(gamma_max), float(eps_min), float(eps_max)),
            "compton_mlp_set_range", ctx)
 
 
 def compton_mlp_set_features(ctx: int, features: int) -> None:
     """Network inputs: FEATURES_MOMENTA (default) or FEATURES_INVARIANTS."""
-    _check(lib().compton_mlp_set_features(c_p(ctx), int(features)), "compton_mlp_set_features", ctx)
+    _check(lib().compton_mlp_set_features(ctx, int(features)), "compton_mlp_set_features", ctx)
 
 
 SIGNATURES["compton_pnet_set_params"] = (c_i32, [c_p, c_p, c_i64, c_p, c_f64, c_f64, c_f64])
@@ -430,7 +446,7 @@ def compton_pnet_set_params(ctx: int, theta, feature_scales=None, gamma_max: flo
     import numpy as np
     t = np.ascontiguousarray(theta, dtype=np.float32)
     fs = None if feature_scales is None else np.ascontiguousarray(feature_scales, dtype=np.float32)
-    _check(lib().compton_pnet_set_params(c_p(ctx), c_p(t.ctypes.data), int(t.shape[0]),
+    _check(lib().compton_pnet_set_params(ctx, c_p(t.ctypes.data), int(t.shape[0]),
                                          None if fs is None else c_p(fs.ctypes.data), float(gamma_max),
                                          float(eps_min), float(eps_max)), "compton_pnet_set_params", ctx)
 
@@ -440,15 +456,14 @@ def compton_pnet_get_params(ctx: int):
     import numpy as np
     t = np.zeros(PNET_PARAMS, np.float32)
     g = np.zeros(PNET_PARAMS, np.float32)
-    _check(lib().compton_pnet_get_params(c_p(ctx), c_p(t.ctypes.data), c_p(g.ctypes.data), PNET_PARAMS),
+    _check(lib().compton_pnet_get_params(ctx, c_p(t.ctypes.data), c_p(g.ctypes.data), PNET_PARAMS),
            "compton_pnet_get_params", ctx)
     return t, g
 
 
 def compton_pnet_infer(ctx: int, u, k, w_e: float, w_g: float, p_max: float, r_out, stream=None) -> None:
     """u, k: (3, n) float32 CUDA tensors; r_out: (n,) float32."""
-    _check(lib().compton_pnet_infer(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                    _ptr(k[2]), int(u.shape[1]), float(w_e), float(w_g), float(p_max),
+    _check(lib().compton_pnet_infer(ctx, *_rows(u), *_rows(k), int(u.shape[1]), float(w_e), float(w_g), float(p_max),
                                     _ptr(r_out), _stream_ptr(stream)), "compton_pnet_infer", ctx)
 
 
@@ -457,8 +472,7 @@ def compton_pnet_train_step(ctx: int, u, k, y, w, w_e: float, w_g: float, p_max:
     """One Adam step on the weighted MAE; returns the loss before the update
     (synchronising) when want_loss, else None."""
     loss = ctypes.c_float(0.0)
-    _check(lib().compton_pnet_train_step(c_p(ctx), _ptr(u[0]), _ptr(u[1]), _ptr(u[2]), _ptr(k[0]), _ptr(k[1]),
-                                         _ptr(k[2]), _ptr(y), None if w is None else _ptr(w), int(u.shape[1]),
+    _check(lib().compton_pnet_train_step(ctx, *_rows(u), *_rows(k), _ptr(y), _ptr(w), int(u.shape[1]),
                                          float(w_e), float(w_g), float(p_max), float(lr),
                                          ctypes.byref(loss) if want_loss else None, _stream_ptr(stream)),
            "compton_pnet_train_step", ctx)
@@ -473,7 +487,7 @@ SIGNATURES["compton_kernel_times"] = (c_i32, [c_p, c_p, c_p])
 
 def compton_kernel_timing(ctx: int, enable: bool) -> None:
     """Start (restarting the counts) or stop per-kernel event timing."""
-    _check(lib().compton_kernel_timing(c_p(ctx), 1 if enable else 0), "compton_kernel_timing", ctx)
+    _check(lib().compton_kernel_timing(ctx, 1 if enable else 0), "compton_kernel_timing", ctx)
 
 
 def compton_kernel_times(ctx: int) -> dict:
@@ -481,7 +495,7 @@ def compton_kernel_times(ctx: int) -> dict:
     was enabled (the last 64 launches of each slot)."""
     ms = (ctypes.c_double * len(KERNEL_SLOTS))()
     n = (ctypes.c_int64 * len(KERNEL_SLOTS))()
-    _check(lib().compton_kernel_times(c_p(ctx), ms, n), "compton_kernel_times", ctx)
+    _check(lib().compton_kernel_times(ctx, ms, n), "compton_kernel_times", ctx)
     return {name: {"ms": ms[i], "launches": n[i]} for i, name in enumerate(KERNEL_SLOTS)}
 
 
@@ -501,4 +515,4 @@ SIGNATURES["compton_selftest_wait"] = (c_i32, [c_p, c_u64, c_p])
 
 
 def compton_selftest_wait(ctx: int, timeout_ns: int, stream=None) -> None:
-    _check(lib().compton_selftest_wait(c_p(ctx), int(timeout_ns), _stream_ptr(stream)), "compton_selftest_wait", ctx)
+    _check(lib().compton_selftest_wait(ctx, int(timeout_ns), _stream_ptr(stream)), "compton_selftest_wait", ctx)
