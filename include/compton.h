@@ -82,8 +82,8 @@ typedef struct compton_config {
                                     relative to gamma + eps stays below 2e-6 up to 8);
                                     0 = always FP64                                            */
     uint64_t mem_budget_bytes;   /* cap on library-owned device memory (0 = no cap)            */
-    int64_t max_train_batch;     /* largest minibatch of compton_mlp_train_step (sizes its
-                                    scratch: 2060 bytes per sample); 0 = no training           */
+    int64_t max_train_batch;     /* largest minibatch of compton_mlp_train_step (its scratch is
+                                    52 KB, whatever the minibatch); 0 = no training            */
 } compton_config;
 
 /* One species in structure-of-arrays form (all device pointers, length n).

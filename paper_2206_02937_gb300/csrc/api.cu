@@ -134,7 +134,7 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
         delete ctx;
         return COMPTON_EINVAL;
     }
-    size_t o_tr = cv.take<uint8_t>(cfg->max_train_batch > 0 ? compton::train_scratch_bytes(cfg->max_train_batch) : 1);
+    const size_t o_ac = cv.take<float>(cfg->max_train_batch > 0 ? NP + 3 : 1);
     size_t o_rb = cv.take<float>(P > 0 ? P : 1);
     size_t o_pn = cv.take<float>(4 * compton::kPnetParams + 2 + compton::kPnetParams + 2 + 1);
     const size_t total = align_up(cv.used, 256);
@@ -186,7 +186,10 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
     m.amax = reinterpret_cast<float*>(base + o_ax);
     m.edges = reinterpret_cast<float*>(base + o_ed);
     m.hist = reinterpret_cast<int*>(base + o_hi);
-    ctx->train_scratch = base + o_tr;
+    if (cfg->max_train_batch > 0) {
+        m.acc = reinterpret_cast<float*>(base + o_ac);
+        m.ticket = reinterpret_cast<uint32_t*>(m.acc + NP + 2);
+    }
     ctx->r_buf = reinterpret_cast<float*>(base + o_rb);
     {
         float* pb = reinterpret_cast<float*>(base + o_pn);

@@ -101,9 +101,12 @@ __host__ __device__ constexpr int mlp_off_b(int l)
 // Device-side network state (all pointers into one context allocation).
 struct MlpDev {
     float* theta;        // [kMlpParams] FP32 master parameters
-    float* grad;         // [kMlpParams]
+    float* grad;         // [kMlpParams] gradient sums of the last step
     float* adam_m;       // [kMlpParams]
     float* adam_v;       // [kMlpParams]
+    float* acc;          // [kMlpParams + 2] sums of the step in flight (gradient, weighted |error|,
+                         // weights), zero between steps; nullptr without training
+    uint32_t* ticket;    // blocks of k_mlp_finish that have read the weight sum, zero between steps
     void* wbf16;         // 4 x 8 KB BF16 tiles, 128-byte swizzled K-major
     void* whalf;         // inference image: 4 x 8 KB BF16 tiles of W / 2 (layer 0 with b / 2 as
                          // hi + lo in K columns 6, 7), then 3 x 2 KB blocks of b / 2 (hi, lo in K
@@ -192,7 +195,7 @@ struct compton_ctx {
     compton::MlpDev mlp{};
     bool mlp_loaded = false;
     int64_t adam_step = 0;
-    void* train_scratch = nullptr;  // inside the arena, sized by cfg.max_train_batch
+    bool train_dirty = false;       // mlp.acc may hold the sums of a step that failed half-way
     float* r_buf = nullptr;         // [max_particles] network output per pair (surrogate modes)
     compton::ServeEngine* serve = nullptr;  // continuous-batching engine (compton_serve_start)
     compton::KernelTiming* timing = nullptr;  // per-kernel event pairs (compton_kernel_timing)
@@ -294,7 +297,7 @@ compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* 
                                 const float* kx, const float* ky, const float* kz, int64_t n, compton_mode mode,
                                 float* r_out, cudaStream_t stream, bool binned = false, bool candidates = false,
                                 const MlpDecide* decide = nullptr);
-size_t train_scratch_bytes(int64_t max_batch);
+compton_status mlp_adam(compton_ctx* ctx, float lr, cudaStream_t stream);
 compton_status launch_balance_weights(compton_ctx* ctx, const float* r, int64_t n, const float* edges_host,
                                       int n_bins, float* w_out, cudaStream_t stream);
 compton_status launch_mlp_train_step(compton_ctx* ctx, const float* ux, const float* uy, const float* uz,

@@ -9,7 +9,7 @@
 // f = [sgnlog(u/s_u)/n_u, sgnlog(k/s_k)/n_k] with sgnlog(z) = sign(z) ln(1+|z|).
 //
 // Kernels:
-//   k_mlp_pack   FP32 parameter vector -> BF16 weight tiles in the 128-byte
+//   k_mlp_finish (Adam on) the FP32 parameter vector -> BF16 weight tiles in the 128-byte
 //                swizzled K-major layout the tensor core reads (layer 0's six
 //                inputs zero-padded to K = 64), FP8 E4M3 tiles (K padded to 128)
 //                with per-tensor scales, transposed FP32 copies for the CUDA
@@ -24,6 +24,8 @@
 //   k_mlp_fp32   FP32 forward on the CUDA cores (reference precision).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>
+
+#include <cmath>
 
 #include "act_math.cuh"
 #include "ctx.hpp"
@@ -91,78 +93,175 @@ __device__ __forceinline__ uint32_t pack_e4m3x4(float a, float b, float c, float
 // Packing.  theta layout (float, 12993): W0 (64x6), b0, W1 (64x64), b1, W2, b2,
 // W3, b3, W4 (1x64), b4; W stored (out, in) row-major.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float theta_w(const float* th, int l, int n, int k)
+// Adam (kAdam) and the images the kernels read, one CTA per layer (CTA 4: the
+// output layer).  A training step's gradient sums come from MlpDev::acc, which
+// is cleared here for the next step (the weight sum by the CTA that reads it
+// last).  The layer's new weights stay in shared memory, where the amax of the
+// FP8 scale and the images are taken from, so that Adam, the scales and the
+// packing are one launch (three before: 4.5, 5 and 4.5 us); images are written
+// 16 bytes at a time.  Without kAdam the parameters are packed as they are.
+struct AdamArgs {
+    float lr, b1, b2, eps, bc1, bc2;
+};
+
+// Adam on one parameter from its loaded state: returns the new parameter.
+__device__ __forceinline__ float adam_value(const AdamArgs& ad, float sum, float ws, float& am, float& av, float th)
 {
-    if (l == 0) return k < 6 ? th[n * 6 + k] : 0.0f;
-    return th[mlp_off_w(l) + n * 64 + k];
+    const float g = ws > 0.0f ? sum / ws : 0.0f;
+    am = ad.b1 * am + (1.0f - ad.b1) * g;
+    av = ad.b2 * av + (1.0f - ad.b2) * g * g;
+    const float mh = am / ad.bc1;
+    const float vh = av / ad.bc2;
+    return th - ad.lr * mh / (sqrtf(vh) + ad.eps);
 }
 
-__global__ void k_mlp_pack(MlpDev m)
+// Parameter i, and four from i on (i % 4 == 0): updated and stored with
+// kAdam, the accumulators cleared; as they are without it.
+template <bool kAdam>
+__device__ __forceinline__ float finish_param(const MlpDev& m, const AdamArgs& ad, int i, float ws)
 {
-    const float* th = m.theta;
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    // BF16 tiles: 4 x 64 x 64
-    if (i < 4 * 64 * 64) {
-        const int l = i / 4096, n = (i / 64) % 64, k = i % 64;
-        uint8_t* base = reinterpret_cast<uint8_t*>(m.wbf16) + l * kWTileBytes;
-        const __nv_bfloat16 v = __float2bfloat16_rn(theta_w(th, l, n, k));
-        *reinterpret_cast<__nv_bfloat16*>(base + tc::sw128_offset(n, k >> 3) + (k & 7) * 2) = v;
-        // transposed FP32 copy for the CUDA-core path: wt[l][k][n]
-        m.wt32[l * 4096 + k * 64 + n] = theta_w(th, l, n, k);
-        // inference image: W / 2 (exact), and in layer 0's padding columns
-        // 6, 7 the half bias as hi + lo (the A rows carry 1, 1 there)
-        uint8_t* hbase = reinterpret_cast<uint8_t*>(m.whalf) + l * kWTileBytes;
-        float hv = 0.5f * theta_w(th, l, n, k);
-        if (l == 0 && (k == 6 || k == 7)) {
-            const float hb = 0.5f * th[mlp_off_b(0) + n];
-            const float hi = __bfloat162float(__float2bfloat16_rn(hb));
-            hv = k == 6 ? hi : hb - hi;
-        }
-        *reinterpret_cast<__nv_bfloat16*>(hbase + tc::sw128_offset(n, k >> 3) + (k & 7) * 2) =
-            __float2bfloat16_rn(hv);
+    float th = m.theta[i];
+    if (kAdam) {
+        const float sum = m.acc[i];
+        float am = m.adam_m[i], av = m.adam_v[i];
+        th = adam_value(ad, sum, ws, am, av, th);
+        m.acc[i] = 0.0f;
+        m.grad[i] = sum;
+        m.adam_m[i] = am;
+        m.adam_v[i] = av;
+        m.theta[i] = th;
     }
-    // half-bias blocks of layers 1-3: row n, K columns 0 (hi) and 1 (lo), zeros to 15
-    if (i < 3 * 64 * 16) {
-        const int l = 1 + i / 1024, n = (i / 16) % 64, k = i % 16;
-        uint8_t* bb = reinterpret_cast<uint8_t*>(m.whalf) + 4 * kWTileBytes + (l - 1) * 2048;
-        const float hb = 0.5f * th[mlp_off_b(l) + n];
-        const float hi = __bfloat162float(__float2bfloat16_rn(hb));
-        const float v = k == 0 ? hi : (k == 1 ? hb - hi : 0.0f);
-        *reinterpret_cast<__nv_bfloat16*>(bb + tc::sw32_offset(n, k >> 3) + (k & 7) * 2) = __float2bfloat16_rn(v);
+    return th;
+}
+template <bool kAdam>
+__device__ __forceinline__ float4 finish_param4(const MlpDev& m, const AdamArgs& ad, int i, float ws)
+{
+    float4 th = *reinterpret_cast<const float4*>(m.theta + i);
+    if (kAdam) {
+        const float4 sum = *reinterpret_cast<const float4*>(m.acc + i);
+        float4 am = *reinterpret_cast<const float4*>(m.adam_m + i), av = *reinterpret_cast<const float4*>(m.adam_v + i);
+        th.x = adam_value(ad, sum.x, ws, am.x, av.x, th.x);
+        th.y = adam_value(ad, sum.y, ws, am.y, av.y, th.y);
+        th.z = adam_value(ad, sum.z, ws, am.z, av.z, th.z);
+        th.w = adam_value(ad, sum.w, ws, am.w, av.w, th.w);
+        *reinterpret_cast<float4*>(m.acc + i) = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        *reinterpret_cast<float4*>(m.grad + i) = sum;
+        *reinterpret_cast<float4*>(m.adam_m + i) = am;
+        *reinterpret_cast<float4*>(m.adam_v + i) = av;
+        *reinterpret_cast<float4*>(m.theta + i) = th;
     }
-    // FP8 tiles: 4 x 64 rows x 128 B (K = 64 real + 64 zero)
-    if (i < 4 * 64 * 128) {
-        const int l = i / 8192, n = (i / 128) % 64, k = i % 128;
-        uint8_t* base = reinterpret_cast<uint8_t*>(m.wfp8) + l * kWTileBytes;
-        const float w = k < 64 ? theta_w(th, l, n, k) * m.scale_w_inv[l] : 0.0f;
-        base[tc::sw128_offset(n, k >> 4) + (k & 15)] = __nv_cvt_float_to_fp8(w, __NV_SATFINITE, __NV_E4M3);
-    }
-    if (i < 4 * 64) {
-        const int l = i / 64, n = i % 64;
-        m.bias[i] = th[mlp_off_b(l) + n];
-    }
-    if (i < 64) m.w4[i] = th[mlp_off_w(4) + i];
-    if (i == 0) m.b4[0] = th[mlp_off_b(4)];
+    return th;
 }
 
-// Per-tensor amax of each layer's weights (for the FP8 scales): one block per layer.
-__global__ void k_mlp_weight_amax(MlpDev m)
+constexpr int kFinishThreads = 1024;
+
+template <bool kAdam>
+__global__ void __launch_bounds__(kFinishThreads) k_mlp_finish(MlpDev m, AdamArgs ad)
 {
+    __shared__ float w[64][65];  // the layer's weights [out][in], layer 0 zero-padded to 64 inputs
+    __shared__ float hb[64];     // half biases
     __shared__ float red[32];
-    const int l = blockIdx.x;
-    const int n_el = l == 0 ? 64 * 6 : 64 * 64;
-    const float* w = m.theta + mlp_off_w(l);
-    float a = 0.0f;
-    for (int i = threadIdx.x; i < n_el; i += blockDim.x) a = fmaxf(a, fabsf(w[i]));
-    for (int d = 16; d > 0; d >>= 1) a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, d));
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = a;
+    const int l = blockIdx.x, tid = threadIdx.x;
+    float ws = 0.0f;
+    if (kAdam) ws = m.acc[kMlpParams + 1];
+    if (l == 4) {
+        if (tid < 64) m.w4[tid] = finish_param<kAdam>(m, ad, mlp_off_w(4) + tid, ws);
+        if (tid == 64) m.b4[0] = finish_param<kAdam>(m, ad, mlp_off_b(4), ws);
+        if (kAdam && tid == 65) {
+            m.loss[0] = m.acc[kMlpParams];
+            m.loss[1] = ws;
+            m.acc[kMlpParams] = 0.0f;
+        }
+    } else {
+        float amax = 0.0f;
+        if (l > 0) {
+            const float4 v = finish_param4<kAdam>(m, ad, mlp_off_w(l) + 4 * tid, ws);
+            float* row = &w[tid >> 4][4 * (tid & 15)];
+            row[0] = v.x;
+            row[1] = v.y;
+            row[2] = v.z;
+            row[3] = v.w;
+            amax = fmaxf(fmaxf(fabsf(v.x), fabsf(v.y)), fmaxf(fabsf(v.z), fabsf(v.w)));
+        } else {
+            for (int e = tid; e < 64 * 64; e += kFinishThreads) {
+                const int n = e >> 6, k = e & 63;
+                if (k >= 6) w[n][k] = 0.0f;
+            }
+            if (tid < 64 * 6) {
+                const float v = finish_param<kAdam>(m, ad, tid, ws);
+                w[tid / 6][tid % 6] = v;
+                amax = fabsf(v);
+            }
+        }
+        if (tid >= kFinishThreads - 64) {  // layer 0: warps without weights
+            const int i = tid - (kFinishThreads - 64);
+            const float b = finish_param<kAdam>(m, ad, mlp_off_b(l) + i, ws);
+            m.bias[l * 64 + i] = b;
+            hb[i] = 0.5f * b;
+        }
+        for (int d = 16; d > 0; d >>= 1) amax = fmaxf(amax, __shfl_xor_sync(0xffffffffu, amax, d));
+        if ((tid & 31) == 0) red[tid >> 5] = amax;
+    }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        float t = 0.0f;
-        for (int i = 0; i < (int)(blockDim.x >> 5); ++i) t = fmaxf(t, red[i]);
-        const float s = t > 0.0f ? t / 448.0f : 1.0f;  // 448 = largest finite E4M3
-        m.scale_w[l] = s;
-        m.scale_w_inv[l] = 1.0f / s;
+    if (kAdam && tid == 0) {
+        // every thread of this CTA has read the weight sum
+        __threadfence();
+        if (atomicAdd(m.ticket, 1u) == gridDim.x - 1) {
+            m.acc[kMlpParams + 1] = 0.0f;
+            *m.ticket = 0u;
+        }
+    }
+    if (l == 4) return;
+    float amax = 0.0f;
+#pragma unroll
+    for (int i = 0; i < kFinishThreads / 32; ++i) amax = fmaxf(amax, red[i]);
+    const float scale = amax > 0.0f ? amax / 448.0f : 1.0f;  // 448 = largest finite E4M3
+    const float scale_inv = 1.0f / scale;
+    if (tid == 0) {
+        m.scale_w[l] = scale;
+        m.scale_w_inv[l] = scale_inv;
+    }
+    // transposed FP32 copy for the CUDA-core path: wt[l][k][n]
+    {
+        const int k = tid >> 4, n = 4 * (tid & 15);
+        reinterpret_cast<float4*>(m.wt32 + l * 4096)[tid] = make_float4(w[n][k], w[n + 1][k], w[n + 2][k], w[n + 3][k]);
+    }
+    const int n = tid >> 3, c = tid & 7;  // row, 16-byte chunk (eight BF16 values)
+    if (tid < 512) {
+        uint32_t v[4], h[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float x = w[n][8 * c + 2 * q], y = w[n][8 * c + 2 * q + 1];
+            v[q] = pack_bf16x2(x, y);
+            h[q] = pack_bf16x2(0.5f * x, 0.5f * y);  // the inference image: W / 2 (exact)
+        }
+        if (l == 0 && c == 0) {
+            // layer 0's padding columns 6, 7: the half bias as hi + lo (the A rows carry 1, 1 there)
+            const float hi = __bfloat162float(__float2bfloat16_rn(hb[n]));
+            h[3] = pack_bf16x2(hi, hb[n] - hi);
+        }
+        uint8_t* base = reinterpret_cast<uint8_t*>(m.wbf16) + l * kWTileBytes;
+        uint8_t* hbase = reinterpret_cast<uint8_t*>(m.whalf) + l * kWTileBytes;
+        *reinterpret_cast<uint4*>(base + tc::sw128_offset(n, c)) = make_uint4(v[0], v[1], v[2], v[3]);
+        *reinterpret_cast<uint4*>(hbase + tc::sw128_offset(n, c)) = make_uint4(h[0], h[1], h[2], h[3]);
+    } else if (tid < 768) {
+        // FP8 tile: the 64 real bytes of each 128-byte row (the upper half stays zero)
+        const int r = (tid - 512) >> 2, c8 = tid & 3;
+        uint32_t v[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const float* x = &w[r][16 * c8 + 4 * q];
+            v[q] = pack_e4m3x4(x[0] * scale_inv, x[1] * scale_inv, x[2] * scale_inv, x[3] * scale_inv);
+        }
+        *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(m.wfp8) + l * kWTileBytes + tc::sw128_offset(r, c8)) =
+            make_uint4(v[0], v[1], v[2], v[3]);
+    } else if (l > 0 && tid < 896) {
+        // half-bias block of layers 1-3: row r, K columns 0 (hi) and 1 (lo), zeros to 15
+        const int r = (tid - 768) >> 1, c2 = tid & 1;
+        const float hi = __bfloat162float(__float2bfloat16_rn(hb[r]));
+        *reinterpret_cast<uint4*>(reinterpret_cast<uint8_t*>(m.whalf) + 4 * kWTileBytes + (l - 1) * 2048 +
+                                  tc::sw32_offset(r, c2)) =
+            make_uint4(c2 == 0 ? pack_bf16x2(hi, hb[r] - hi) : 0u, 0u, 0u, 0u);
     }
 }
 
@@ -833,11 +932,21 @@ int grid_persistent(const void* kernel, int threads, int smem, int64_t work_item
 
 compton_status mlp_repack(compton_ctx* ctx, cudaStream_t stream)
 {
-    MlpDev m = ctx->mlp;
-    k_mlp_weight_amax<<<4, 256, 0, stream>>>(m);
-    COMPTON_LAUNCH_CHECK(ctx, "k_mlp_weight_amax");
-    k_mlp_pack<<<(4 * 64 * 128 + 255) / 256, 256, 0, stream>>>(m);
-    COMPTON_LAUNCH_CHECK(ctx, "k_mlp_pack");
+    k_mlp_finish<false><<<5, kFinishThreads, 0, stream>>>(ctx->mlp, AdamArgs{});
+    COMPTON_LAUNCH_CHECK(ctx, "k_mlp_finish");
+    return COMPTON_OK;
+}
+
+// Adam on the gradient sums of the step in flight, then the images.
+compton_status mlp_adam(compton_ctx* ctx, float lr, cudaStream_t stream)
+{
+    if (inject_fault()) return set_injected_error(ctx, "k_mlp_finish");  // before the update, not after it
+    const double step = (double)(ctx->adam_step + 1);
+    AdamArgs ad{lr, 0.9f, 0.999f, 1e-7f, 1.0f - (float)std::pow(0.9, step), 1.0f - (float)std::pow(0.999, step)};
+    k_mlp_finish<true><<<5, kFinishThreads, 0, stream>>>(ctx->mlp, ad);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return set_cuda_error(ctx, e, "k_mlp_finish");
+    ctx->adam_step += 1;
     return COMPTON_OK;
 }
 

@@ -5,32 +5,20 @@
 // the simulation).
 //
 // One training step over a minibatch of n samples (inputs u, k; targets y;
-// per-sample weights w from the data balancing):
-//   k_train_fwd_bwd  one sample per thread, FP32: forward through the four
-//                    SiLU layers and the sigmoid output, storing each hidden
-//                    pre-activation z_l; the weighted MAE subgradient
-//                    w sign(y' - y) (0 at equality); backward through the
-//                    sigmoid and each layer, storing each layer's delta
-//                    (dL/dz_l); loss numerator and weight sum accumulated.
-//   k_train_dw       dW_l = sum_s delta_l(s) h_{l-1}(s)^T and db_l = sum_s
-//                    delta_l(s) over the batch: each CTA reduces a chunk of
-//                    samples for one layer into registers and adds its
-//                    partial sums to the gradient.
-//   k_train_adam     Adam (Kingma and Ba 2014, Algorithm 1) on the FP32 master
-//                    parameters with the gradient divided by sum w, then the
-//                    inference images are rebuilt (k_mlp_pack).
-// With the tensor-core training precision selected (compton_mlp_set_train_
-// precision), the gradient comes from k_train_tc (mlp_train_tc.cu) instead of
-// the first two kernels; Adam and the repacking are shared.
-// Scratch: z and delta for 4 layers x 64 units x n samples, laid out
-// [layer][unit][sample] so that consecutive threads touch consecutive words.
+// per-sample weights w from the data balancing) is two launches:
+//   k_train_f32 or (tensor-core precision) k_train_tc of mlp_train_tc.cu
+//                    forward and backward over tiles of samples; the gradient
+//                    sums, the loss numerator and the weight sum are added to
+//                    MlpDev::acc;
+//   k_mlp_finish     (mlp.cu) Adam (Kingma and Ba 2014, Algorithm 1) on the
+//                    FP32 master parameters with the gradient divided by sum
+//                    w, the inference images rebuilt, acc cleared for the
+//                    next step.
 #include "ctx.hpp"
 #include "features.cuh"
 
 namespace compton {
 namespace {
-
-constexpr int kTrThreads = 128;
 
 __device__ __forceinline__ float sigm(float z) { return 1.0f / (1.0f + expf(-z)); }
 
@@ -41,195 +29,269 @@ struct TrainArgs {
     const float* y;
     const float* w;  // nullable: all ones
     int64_t n;
-    float* z;        // [4][64][n]
-    float* delta;    // [4][64][n]
-    float* dout;     // [n] delta of the output unit
-    float* feat;     // [6][n]
 };
 
-__global__ void __launch_bounds__(kTrThreads) k_train_fwd_bwd(TrainArgs a)
+// ---------------------------------------------------------------------------
+// FP32 gradient on the CUDA cores.  One CTA per SM takes tiles of 64 samples;
+// every contraction of the tile (z = a W^T, dX = delta W, dW = delta^T a, each
+// 64 x 64 x 64) is a register tile of 4 x 4 outputs per thread over operands in
+// shared memory: two 16-byte shared loads per 16 multiply-adds, where one
+// sample per thread took 16 such loads for 64 and left an SM eight warps.
+// Activations and deltas lie as [unit][sample] rows 68 words apart, so that the
+// 16-byte loads along the samples of neighbouring rows (dW) fall into different
+// banks; the weights lie in both orders.  Pre-activations never leave the
+// thread: the backward pass uses the same thread-to-output map as the forward
+// pass, so the derivative of SiLU stays in 16 registers per layer, and dW is
+// accumulated over the CTA's tiles in registers (a tile's sums first, then
+// added, so that no FP32 sum is longer than a tile plus the tiles).
+//
+// What bounds it: the FP32 pipe (9.2 contractions of 1.1 us each per tile) and
+// the SiLU's exact exponentials and divisions.
+// ---------------------------------------------------------------------------
+constexpr int kTrThreads = 256;
+constexpr int kTrTile = 64;              // samples per tile
+constexpr int kTrStride = kTrTile + 4;   // words between rows of activations and deltas
+constexpr int kTrMat = 64 * kTrStride;   // one 64-row block of activations
+struct TrainSmem {
+    static constexpr int wt = 0;                       // W_1..W_3 as [in][out]
+    static constexpr int wj = wt + 3 * 4096;           // W_1..W_3 as [out][in]
+    static constexpr int wt0 = wj + 3 * 4096;          // W_0 as [in][out], 6 rows
+    static constexpr int bias = wt0 + 6 * 64;          // 4 x 64
+    static constexpr int w4 = bias + 256;              // 64
+    static constexpr int feat = w4 + 64;               // 6 rows
+    static constexpr int act = feat + 6 * kTrStride;   // a_0..a_3
+    static constexpr int delta = act + 4 * kTrMat;     // two blocks of deltas
+    static constexpr int dout = delta + 2 * kTrMat;    // delta of the output unit per sample
+    static constexpr int words = dout + kTrTile;
+};
+
+__device__ __forceinline__ void cp_async16(float* smem_dst, const float* gmem_src)
 {
-    extern __shared__ float sm[];
-    float* wt = sm;                          // 4 x 64 x 64: wt[l][i][j] = W_l[j][i]
-    float* hs = wt + 4 * 4096;               // 64 x kTrThreads activations / deltas
-    float* bias = hs + 64 * kTrThreads;      // 256
-    float* w4 = bias + 256;                  // 64
+    const uint32_t d = (uint32_t)__cvta_generic_to_shared(smem_dst);
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n" ::"r"(d), "l"(gmem_src) : "memory");
+}
+
+// acc[p][q] += x[p] y[q]
+__device__ __forceinline__ void outer4(float (&acc)[4][4], float4 x, float4 y)
+{
+    const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+    for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(xv[p], yv[q], acc[p][q]);
+}
+
+__device__ __forceinline__ float dot4(float4 x, float4 y, float t)
+{
+    return fmaf(x.w, y.w, fmaf(x.z, y.z, fmaf(x.y, y.y, fmaf(x.x, y.x, t))));
+}
+
+__global__ void __launch_bounds__(kTrThreads, 1) k_train_f32(TrainArgs a)
+{
+    extern __shared__ __align__(16) float sm[];
+    using S = TrainSmem;
     const int tid = threadIdx.x;
     const MlpDev& m = a.m;
-    for (int i = tid; i < 4096; i += kTrThreads) reinterpret_cast<float4*>(wt)[i] = reinterpret_cast<const float4*>(m.wt32)[i];
-    for (int i = tid; i < 256; i += kTrThreads) bias[i] = m.bias[i];
-    if (tid < 64) w4[tid] = m.w4[tid];
+    // forward operands first, the backward pass's weight order behind them
+    for (int i = tid; i < 3 * 1024; i += kTrThreads) cp_async16(sm + S::wt + 4 * i, m.wt32 + 4096 + 4 * i);
+    if (tid < 6 * 16) cp_async16(sm + S::wt0 + 4 * tid, m.wt32 + 4 * tid);
+    if (tid < 64) cp_async16(sm + S::bias + 4 * tid, m.bias + 4 * tid);
+    if (tid < 16) cp_async16(sm + S::w4 + 4 * tid, m.w4 + 4 * tid);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    for (int l = 1; l < 4; ++l)
+        for (int i = tid; i < 1024; i += kTrThreads)
+            cp_async16(sm + S::wj + (l - 1) * 4096 + 4 * i, m.theta + mlp_off_w(l) + 4 * i);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
     const float b4 = m.b4[0];
-    __syncthreads();
-    const int64_t n = a.n;
+
+    const int s0 = 4 * (tid & 15), j0 = 4 * (tid >> 4);  // forward and dX: samples s0.., units j0..
+    const int di = tid & 15, dj = tid >> 4;              // dW: inputs di + 16 q, outputs dj + 16 p
+    const int bj = tid >> 2, bp = tid & 3;               // bias sums: unit bj, a quarter of the samples
+    float dw[3][4][4], db[4] = {0, 0, 0, 0}, dw0[3] = {0, 0, 0}, dw4 = 0.0f, db4 = 0.0f;
+#pragma unroll
+    for (int l = 0; l < 3; ++l)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q) dw[l][p][q] = 0.0f;
     float loss_num = 0.0f, wsum = 0.0f;
-    for (int64_t s = (int64_t)blockIdx.x * kTrThreads + tid; s < n; s += (int64_t)gridDim.x * kTrThreads) {
+
+    for (int64_t base = (int64_t)blockIdx.x * kTrTile; base < a.n; base += (int64_t)gridDim.x * kTrTile) {
+        const int ns = a.n - base < kTrTile ? (int)(a.n - base) : kTrTile;
+        // ---- features ----
+        if (tid < kTrTile) {
+            float f[6] = {0, 0, 0, 0, 0, 0};
+            if (tid < ns) {
+                const int64_t s = base + tid;
+                features(m, a.u[0][s], a.u[1][s], a.u[2][s], a.k[0][s], a.k[1][s], a.k[2][s], f);
+            }
+#pragma unroll
+            for (int i = 0; i < 6; ++i) sm[S::feat + i * kTrStride + tid] = f[i];
+        }
+        asm volatile("cp.async.wait_group 1;\n" ::: "memory");
+        __syncthreads();
         // ---- forward ----
-        float f[6];
-        features(m, a.u[0][s], a.u[1][s], a.u[2][s], a.k[0][s], a.k[1][s], a.k[2][s], f);
+        float ds[4][4][4];  // SiLU'(z_l) of units j0.., samples s0..
 #pragma unroll
-        for (int i = 0; i < 6; ++i) {
-            hs[i * kTrThreads + tid] = f[i];
-            a.feat[i * n + s] = f[i];
-        }
-        float acc[64];
         for (int l = 0; l < 4; ++l) {
+            float z[4][4];
 #pragma unroll
-            for (int j = 0; j < 64; ++j) acc[j] = bias[l * 64 + j];
-            const int n_in = l == 0 ? 6 : 64;
-            for (int i = 0; i < n_in; ++i) {
-                const float hi = hs[i * kTrThreads + tid];
-                const float4* wr = reinterpret_cast<const float4*>(wt + l * 4096 + i * 64);
+            for (int p = 0; p < 4; ++p)
 #pragma unroll
-                for (int j4 = 0; j4 < 16; ++j4) {
-                    const float4 wv = wr[j4];
-                    acc[4 * j4 + 0] = fmaf(wv.x, hi, acc[4 * j4 + 0]);
-                    acc[4 * j4 + 1] = fmaf(wv.y, hi, acc[4 * j4 + 1]);
-                    acc[4 * j4 + 2] = fmaf(wv.z, hi, acc[4 * j4 + 2]);
-                    acc[4 * j4 + 3] = fmaf(wv.w, hi, acc[4 * j4 + 3]);
+                for (int q = 0; q < 4; ++q) z[p][q] = sm[S::bias + 64 * l + j0 + p];
+            const float* in = l == 0 ? sm + S::feat : sm + S::act + (l - 1) * kTrMat;
+            const float* w = l == 0 ? sm + S::wt0 : sm + S::wt + (l - 1) * 4096;
+#pragma unroll 8
+            for (int i = 0; i < (l == 0 ? 6 : 64); ++i)
+                outer4(z, *reinterpret_cast<const float4*>(w + 64 * i + j0),
+                       *reinterpret_cast<const float4*>(in + kTrStride * i + s0));
+#pragma unroll
+            for (int p = 0; p < 4; ++p) {
+                float h[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q) {
+                    const float zz = z[p][q], sg = sigm(zz);
+                    ds[l][p][q] = sg * (1.0f + zz * (1.0f - sg));
+                    h[q] = zz * sg;
+                    if (s0 + q >= ns) h[q] = ds[l][p][q] = 0.0f;
                 }
+                *reinterpret_cast<float4*>(sm + S::act + l * kTrMat + (j0 + p) * kTrStride + s0) =
+                    make_float4(h[0], h[1], h[2], h[3]);
             }
-#pragma unroll
-            for (int j = 0; j < 64; ++j) {
-                a.z[((int64_t)l * 64 + j) * n + s] = acc[j];
-                hs[j * kTrThreads + tid] = acc[j] * sigm(acc[j]);
+            __syncthreads();
+        }
+        // ---- output, loss and the output unit's delta: one thread per sample ----
+        if (tid < kTrTile) {
+            float d_out = 0.0f;
+            if (tid < ns) {
+                float zo = b4;
+#pragma unroll 16
+                for (int j = 0; j < 64; ++j) zo = fmaf(sm[S::act + 3 * kTrMat + j * kTrStride + tid], sm[S::w4 + j], zo);
+                const float yp = sigm(zo);
+                const float wi = a.w ? a.w[base + tid] : 1.0f;
+                const float diff = yp - a.y[base + tid];
+                loss_num += wi * fabsf(diff);
+                wsum += wi;
+                // unnormalised: the 1 / sum w factor is applied in Adam
+                const float g = diff > 0.0f ? wi : (diff < 0.0f ? -wi : 0.0f);
+                d_out = g * yp * (1.0f - yp);
             }
+            sm[S::dout + tid] = d_out;
+            db4 += d_out;
         }
-        float zo = b4;
+        asm volatile("cp.async.wait_group 0;\n" ::: "memory");
+        __syncthreads();
+        // ---- backward ----
+        {
+            const float4 d4 = *reinterpret_cast<const float4*>(sm + S::dout + s0);
+            const float d[4] = {d4.x, d4.y, d4.z, d4.w};
 #pragma unroll
-        for (int j = 0; j < 64; ++j) zo = fmaf(hs[j * kTrThreads + tid], w4[j], zo);
-        const float yp = sigm(zo);
-        const float wi = a.w ? a.w[s] : 1.0f;
-        const float diff = yp - a.y[s];
-        loss_num += wi * fabsf(diff);
-        wsum += wi;
-        // ---- backward ----  (unnormalised: the 1/sum w factor is applied in Adam)
-        const float g = diff > 0.0f ? wi : (diff < 0.0f ? -wi : 0.0f);
-        const float d_out = g * yp * (1.0f - yp);
-        a.dout[s] = d_out;
-        // delta of the last hidden layer: W4^T d_out times silu'(z_3); acc holds z_3
+            for (int p = 0; p < 4; ++p) {
+                const float w = sm[S::w4 + j0 + p];
+                *reinterpret_cast<float4*>(sm + S::delta + (j0 + p) * kTrStride + s0) =
+                    make_float4(w * d[0] * ds[3][p][0], w * d[1] * ds[3][p][1], w * d[2] * ds[3][p][2],
+                                w * d[3] * ds[3][p][3]);
+            }
+            // dw_4
+            const float4* av = reinterpret_cast<const float4*>(sm + S::act + 3 * kTrMat + bj * kTrStride + 16 * bp);
+            const float4* dv = reinterpret_cast<const float4*>(sm + S::dout + 16 * bp);
+            float t = 0.0f;
 #pragma unroll
-        for (int j = 0; j < 64; ++j) {
-            const float sg = sigm(acc[j]);
-            const float ds = sg * (1.0f + acc[j] * (1.0f - sg));
-            acc[j] = w4[j] * d_out * ds;
+            for (int i = 0; i < 4; ++i) t = dot4(av[i], dv[i], t);
+            dw4 += t;
         }
+        __syncthreads();
+#pragma unroll
         for (int l = 3; l >= 0; --l) {
+            const float* dl = sm + S::delta + ((3 - l) & 1) * kTrMat;
+            if (l > 0) {
+                // delta_{l-1} = (delta_l W_l) SiLU'(z_{l-1}), units j0.. of layer l - 1
+                float t[4][4] = {};
+#pragma unroll 8
+                for (int j = 0; j < 64; ++j)
+                    outer4(t, *reinterpret_cast<const float4*>(sm + S::wj + (l - 1) * 4096 + 64 * j + j0),
+                           *reinterpret_cast<const float4*>(dl + kTrStride * j + s0));
+                float* dn = sm + S::delta + ((4 - l) & 1) * kTrMat;
 #pragma unroll
-            for (int j = 0; j < 64; ++j) a.delta[((int64_t)l * 64 + j) * n + s] = acc[j];
-            if (l == 0) break;
-            // dh_{l-1}[i] = sum_j W_l[j][i] delta_l[j] = sum_j wt[l][i][j] delta_l[j]
-            for (int i = 0; i < 64; ++i) {
-                const float4* wr = reinterpret_cast<const float4*>(wt + l * 4096 + i * 64);
+                for (int p = 0; p < 4; ++p)
+                    *reinterpret_cast<float4*>(dn + (j0 + p) * kTrStride + s0) =
+                        make_float4(t[p][0] * ds[l - 1][p][0], t[p][1] * ds[l - 1][p][1], t[p][2] * ds[l - 1][p][2],
+                                    t[p][3] * ds[l - 1][p][3]);
+                // dW_l
+                const float* in = sm + S::act + (l - 1) * kTrMat;
+                float g[4][4] = {};
+#pragma unroll 2
+                for (int s = 0; s < kTrTile; s += 4) {
+                    float4 dv[4], av[4];
+#pragma unroll
+                    for (int p = 0; p < 4; ++p) {
+                        dv[p] = *reinterpret_cast<const float4*>(dl + (dj + 16 * p) * kTrStride + s);
+                        av[p] = *reinterpret_cast<const float4*>(in + (di + 16 * p) * kTrStride + s);
+                    }
+#pragma unroll
+                    for (int p = 0; p < 4; ++p)
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) g[p][q] = dot4(dv[p], av[q], g[p][q]);
+                }
+#pragma unroll
+                for (int p = 0; p < 4; ++p)
+#pragma unroll
+                    for (int q = 0; q < 4; ++q) dw[l - 1][p][q] += g[p][q];
+            } else if (tid < 128) {
+                // dW_0: output tid / 2, three of the six inputs
+                float g[3] = {0, 0, 0};
+                for (int s = 0; s < kTrTile; s += 4) {
+                    const float4 dv = *reinterpret_cast<const float4*>(dl + (tid >> 1) * kTrStride + s);
+#pragma unroll
+                    for (int q = 0; q < 3; ++q)
+                        g[q] = dot4(dv, *reinterpret_cast<const float4*>(sm + S::feat + (3 * (tid & 1) + q) * kTrStride + s),
+                                    g[q]);
+                }
+#pragma unroll
+                for (int q = 0; q < 3; ++q) dw0[q] += g[q];
+            }
+            {
+                const float4* dv = reinterpret_cast<const float4*>(dl + bj * kTrStride + 16 * bp);
                 float t = 0.0f;
 #pragma unroll
-                for (int j4 = 0; j4 < 16; ++j4) {
-                    const float4 wv = wr[j4];
-                    t = fmaf(wv.x, acc[4 * j4 + 0], t);
-                    t = fmaf(wv.y, acc[4 * j4 + 1], t);
-                    t = fmaf(wv.z, acc[4 * j4 + 2], t);
-                    t = fmaf(wv.w, acc[4 * j4 + 3], t);
-                }
-                hs[i * kTrThreads + tid] = t;
+                for (int i = 0; i < 4; ++i) t += (dv[i].x + dv[i].y) + (dv[i].z + dv[i].w);
+                db[l] += t;
             }
-            // delta_{l-1} = dh_{l-1} * silu'(z_{l-1}), silu' = s (1 + z (1 - s))
-#pragma unroll
-            for (int i = 0; i < 64; ++i) {
-                const float zz = a.z[((int64_t)(l - 1) * 64 + i) * n + s];
-                const float sg = sigm(zz);
-                acc[i] = hs[i * kTrThreads + tid] * sg * (1.0f + zz * (1.0f - sg));
-            }
+            __syncthreads();
         }
     }
-    // loss and weight sums
-    for (int d = 16; d > 0; d >>= 1) {
-        loss_num += __shfl_xor_sync(0xffffffffu, loss_num, d);
-        wsum += __shfl_xor_sync(0xffffffffu, wsum, d);
-    }
-    if ((tid & 31) == 0) {
-        atomicAdd(&m.loss[0], loss_num);
-        atomicAdd(&m.loss[1], wsum);
-    }
-}
 
-// Weight gradient of one layer over a chunk of samples.  256 threads, each
-// owning 16 consecutive entries (j, i..i+15) of the 64 x 64 block (layer 0:
-// 64 x 6, the output layer: 1 x 64 plus its bias).  Inputs h_{l-1} are the
-// features (l = 0) or silu(z_{l-1}); deltas are stored per layer.
-constexpr int kDwThreads = 256;
-constexpr int kDwChunk = 256;
-
-__global__ void __launch_bounds__(kDwThreads) k_train_dw(TrainArgs a, int64_t chunk)
-{
-    __shared__ float hsh[64][kDwChunk / 8 + 1];   // 64 inputs x 32 samples (+1: no bank conflicts)
-    __shared__ float dsh[64][kDwChunk / 8 + 1];   // 64 deltas x 32 samples
-    const int l = blockIdx.y;                  // 0..4 (4 = output layer)
-    const int tid = threadIdx.x;
-    const int64_t n = a.n;
-    const int64_t s0 = (int64_t)blockIdx.x * chunk;
-    const int64_t s1 = s0 + chunk < n ? s0 + chunk : n;
-    const int n_in = l == 0 ? 6 : 64;
-    const int n_out = l == 4 ? 1 : 64;
-    const int j = tid / 4;                     // output unit
-    const int i0 = (tid % 4) * 16;             // first input of this thread
-    float acc[16];
+    // ---- the CTA's sums into the step's accumulators ----
+    float* acc = m.acc;
 #pragma unroll
-    for (int q = 0; q < 16; ++q) acc[q] = 0.0f;
-    float accb = 0.0f;
-    constexpr int S = kDwChunk / 8;
-    for (int64_t sb = s0; sb < s1; sb += S) {
-        const int ns = (int)(s1 - sb < S ? s1 - sb : S);
-        __syncthreads();
-        for (int e = tid; e < 64 * S; e += kDwThreads) {
-            const int unit = e / S, ss = e % S;
-            float h = 0.0f, d = 0.0f;
-            if (ss < ns) {
-                const int64_t s = sb + ss;
-                if (unit < n_in) {
-                    if (l == 0) {
-                        h = a.feat[unit * n + s];
-                    } else {
-                        const float zz = a.z[((int64_t)(l - 1) * 64 + unit) * n + s];
-                        h = zz / (1.0f + expf(-zz));
-                    }
-                }
-                if (unit < n_out) d = l == 4 ? a.dout[s] : a.delta[((int64_t)l * 64 + unit) * n + s];
-            }
-            hsh[unit][ss] = h;
-            dsh[unit][ss] = d;
+    for (int l = 1; l < 4; ++l)
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+                atomicAdd(&acc[mlp_off_w(l) + (dj + 16 * p) * 64 + di + 16 * q], dw[l - 1][p][q]);
+    if (tid < 128)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) atomicAdd(&acc[(tid >> 1) * 6 + 3 * (tid & 1) + q], dw0[q]);
+#pragma unroll
+    for (int l = 0; l < 5; ++l) {
+        float t = l < 4 ? db[l] : dw4;
+        t += __shfl_xor_sync(0xffffffffu, t, 1);
+        t += __shfl_xor_sync(0xffffffffu, t, 2);
+        if (bp == 0) atomicAdd(&acc[(l < 4 ? mlp_off_b(l) : mlp_off_w(4)) + bj], t);
+    }
+    if (tid < kTrTile) {
+        for (int d = 16; d > 0; d >>= 1) {
+            loss_num += __shfl_xor_sync(0xffffffffu, loss_num, d);
+            wsum += __shfl_xor_sync(0xffffffffu, wsum, d);
+            db4 += __shfl_xor_sync(0xffffffffu, db4, d);
         }
-        __syncthreads();
-        if (j < n_out) {
-            for (int ss = 0; ss < ns; ++ss) {
-                const float d = dsh[j][ss];
-                accb += (i0 == 0) ? d : 0.0f;
-#pragma unroll
-                for (int q = 0; q < 16; ++q) acc[q] = fmaf(d, hsh[i0 + q][ss], acc[q]);
-            }
+        if ((tid & 31) == 0) {
+            atomicAdd(&acc[mlp_off_b(4)], db4);
+            atomicAdd(&acc[kMlpParams], loss_num);
+            atomicAdd(&acc[kMlpParams + 1], wsum);
         }
     }
-    if (j < n_out) {
-        float* gw = a.m.grad + mlp_off_w(l);
-#pragma unroll
-        for (int q = 0; q < 16; ++q)
-            if (i0 + q < n_in) atomicAdd(&gw[j * n_in + i0 + q], acc[q]);
-        if (i0 == 0) atomicAdd(&a.m.grad[mlp_off_b(l) + j], accb);
-    }
-}
-
-__global__ void k_train_adam(MlpDev m, float lr, float b1, float b2, float eps, float bc1, float bc2)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= kMlpParams) return;
-    const float ws = m.loss[1];
-    const float g = ws > 0.0f ? m.grad[i] / ws : 0.0f;
-    const float mm = b1 * m.adam_m[i] + (1.0f - b1) * g;
-    const float vv = b2 * m.adam_v[i] + (1.0f - b2) * g * g;
-    m.adam_m[i] = mm;
-    m.adam_v[i] = vv;
-    const float mh = mm / bc1;
-    const float vh = vv / bc2;
-    m.theta[i] -= lr * mh / (sqrtf(vh) + eps);
 }
 
 // Data balancing (Sec. 3.2: events of every probability range should appear
@@ -303,67 +365,41 @@ compton_status launch_balance_weights(compton_ctx* ctx, const float* r, int64_t 
     return COMPTON_OK;
 }
 
-size_t train_scratch_bytes(int64_t max_batch)
-{
-    return (size_t)max_batch * sizeof(float) * (2 * 4 * 64 + 1 + 6);
-}
-
-compton_status adam_and_repack(compton_ctx* ctx, float lr, cudaStream_t stream);
-
 compton_status launch_mlp_train_step(compton_ctx* ctx, const float* ux, const float* uy, const float* uz,
                                      const float* kx, const float* ky, const float* kz, const float* y,
                                      const float* w, int64_t n, float lr, cudaStream_t stream)
 {
-    TrainArgs a;
-    a.m = ctx->mlp;
-    a.u[0] = ux;
-    a.u[1] = uy;
-    a.u[2] = uz;
-    a.k[0] = kx;
-    a.k[1] = ky;
-    a.k[2] = kz;
-    a.y = y;
-    a.w = w;
-    a.n = n;
-    float* base = reinterpret_cast<float*>(ctx->train_scratch);
-    a.z = base;
-    a.delta = base + (size_t)4 * 64 * n;
-    a.dout = a.delta + (size_t)4 * 64 * n;
-    a.feat = a.dout + n;
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.grad, 0, sizeof(float) * kMlpParams, stream));
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.loss, 0, 2 * sizeof(float), stream));
+    // the accumulators are zero between steps (k_mlp_finish clears them); after
+    // a step that failed between its two launches they are cleared here
+    if (ctx->train_dirty)
+        COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.acc, 0, sizeof(float) * (kMlpParams + 2), stream));
+    ctx->train_dirty = true;
+    compton_status st;
     if (ctx->train_tc) {
-        const compton_status st = launch_mlp_grad_tc(ctx, ux, uy, uz, kx, ky, kz, y, w, n, stream);
+        st = launch_mlp_grad_tc(ctx, ux, uy, uz, kx, ky, kz, y, w, n, stream);
         if (st != COMPTON_OK) return st;
-        return adam_and_repack(ctx, lr, stream);
+    } else {
+        TrainArgs a;
+        a.m = ctx->mlp;
+        a.u[0] = ux;
+        a.u[1] = uy;
+        a.u[2] = uz;
+        a.k[0] = kx;
+        a.k[1] = ky;
+        a.k[2] = kz;
+        a.y = y;
+        a.w = w;
+        a.n = n;
+        const int smem = TrainSmem::words * (int)sizeof(float);
+        COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_train_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
+        const int64_t tiles = (n + kTrTile - 1) / kTrTile;
+        const unsigned grid = (unsigned)(tiles < ctx->n_sm ? tiles : ctx->n_sm);
+        k_train_f32<<<grid, kTrThreads, smem, stream>>>(a);
+        COMPTON_LAUNCH_CHECK(ctx, "k_train_f32");
     }
-    const int smem = (4 * 4096 + 64 * kTrThreads + 256 + 64) * 4;
-    COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_train_fwd_bwd, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
-    int n_sm = 0, dev = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
-    int64_t blocks = (n + kTrThreads - 1) / kTrThreads;
-    if (blocks > (int64_t)n_sm * 2) blocks = (int64_t)n_sm * 2;
-    k_train_fwd_bwd<<<(unsigned)blocks, kTrThreads, smem, stream>>>(a);
-    COMPTON_LAUNCH_CHECK(ctx, "k_train_fwd_bwd");
-    int64_t chunk = (n + 4 * n_sm - 1) / (4 * n_sm);
-    if (chunk < kDwChunk) chunk = kDwChunk;
-    const dim3 grid((unsigned)((n + chunk - 1) / chunk), 5);
-    k_train_dw<<<grid, kDwThreads, 0, stream>>>(a, chunk);
-    COMPTON_LAUNCH_CHECK(ctx, "k_train_dw");
-    return adam_and_repack(ctx, lr, stream);
-}
-
-// Adam on the gradient sums of the step, then the inference images.
-compton_status adam_and_repack(compton_ctx* ctx, float lr, cudaStream_t stream)
-{
-    ctx->adam_step += 1;
-    const float b1 = 0.9f, b2 = 0.999f, eps = 1e-7f;
-    const float bc1 = 1.0f - (float)std::pow(0.9, (double)ctx->adam_step);
-    const float bc2 = 1.0f - (float)std::pow(0.999, (double)ctx->adam_step);
-    k_train_adam<<<(kMlpParams + 255) / 256, 256, 0, stream>>>(ctx->mlp, lr, b1, b2, eps, bc1, bc2);
-    COMPTON_LAUNCH_CHECK(ctx, "k_train_adam");
-    return mlp_repack(ctx, stream);
+    st = mlp_adam(ctx, lr, stream);
+    if (st == COMPTON_OK) ctx->train_dirty = false;
+    return st;
 }
 
 }  // namespace compton

@@ -32,8 +32,8 @@
 //                 read a padding region and are never used.
 // Bias gradients, the output layer and the loss run on the CUDA cores (warp
 // reduce-scatters of the per-row values).  At the end each CTA adds its
-// gradient sums to the context's gradient with one atomic per entry; Adam and
-// the repacking of the inference images follow as in the FP32 path.
+// gradient sums to MlpDev::acc with one atomic per entry; Adam and the repacking
+// of the inference images follow as in the FP32 path.
 // Every wait is bounded by %globaltimer (ETIMEOUT recorded, TMEM freed).
 #include <cuda_bf16.h>
 
@@ -314,7 +314,7 @@ __global__ void __launch_bounds__(kTT, 1) k_train_tc(TrainTcArgs a)
     }
     if (failed && tid == 0) atomicOr(&a.stats->error_flags, (unsigned long long)kErrTimeout);
 
-    // ---------------- the CTA's sums into the context's gradient ----------------
+    // ---------------- the CTA's sums into the step's accumulators ----------------
     tc::fence_before_sync();
     __syncthreads();
     tc::fence_after_sync();
@@ -322,7 +322,7 @@ __global__ void __launch_bounds__(kTT, 1) k_train_tc(TrainTcArgs a)
         // rows 0..63 of each dW block (TMEM lanes of warps 0 and 1)
         const int j = tid;  // output unit
         for (int l = 0; l < 4; ++l) {
-            float* gw = m.grad + mlp_off_w(l);
+            float* gw = m.acc + mlp_off_w(l);
             const int n_in = l == 0 ? 6 : 64;
 #pragma unroll
             for (int h = 0; h < 2; ++h) {
@@ -336,8 +336,8 @@ __global__ void __launch_bounds__(kTT, 1) k_train_tc(TrainTcArgs a)
     }
     if (!failed) {
         for (int l = 0; l < 4; ++l)
-            for (int h = 0; h < 2; ++h) atomicAdd(&m.grad[mlp_off_b(l) + 32 * h + (int)lane], db[l][h]);
-        for (int h = 0; h < 2; ++h) atomicAdd(&m.grad[mlp_off_w(4) + 32 * h + (int)lane], dw4[h]);
+            for (int h = 0; h < 2; ++h) atomicAdd(&m.acc[mlp_off_b(l) + 32 * h + (int)lane], db[l][h]);
+        for (int h = 0; h < 2; ++h) atomicAdd(&m.acc[mlp_off_w(4) + 32 * h + (int)lane], dw4[h]);
 #pragma unroll
         for (int d = 16; d > 0; d >>= 1) {
             db4 += __shfl_xor_sync(0xffffffffu, db4, d);
@@ -345,9 +345,9 @@ __global__ void __launch_bounds__(kTT, 1) k_train_tc(TrainTcArgs a)
             wsum += __shfl_xor_sync(0xffffffffu, wsum, d);
         }
         if (lane == 0) {
-            atomicAdd(&m.grad[mlp_off_b(4)], db4);
-            atomicAdd(&m.loss[0], loss_num);
-            atomicAdd(&m.loss[1], wsum);
+            atomicAdd(&m.acc[mlp_off_b(4)], db4);
+            atomicAdd(&m.acc[kMlpParams], loss_num);
+            atomicAdd(&m.acc[kMlpParams + 1], wsum);
         }
     }
     tc::fence_before_sync();
@@ -358,8 +358,8 @@ __global__ void __launch_bounds__(kTT, 1) k_train_tc(TrainTcArgs a)
 
 }  // namespace
 
-// The gradient of one minibatch on the tensor cores (the caller zeroes the
-// gradient and loss sums before, and runs Adam after).
+// The gradient of one minibatch on the tensor cores, added to MlpDev::acc
+// (zero before; the caller runs Adam after).
 compton_status launch_mlp_grad_tc(compton_ctx* ctx, const float* ux, const float* uy, const float* uz,
                                   const float* kx, const float* ky, const float* kz, const float* y, const float* w,
                                   int64_t n, cudaStream_t stream)
