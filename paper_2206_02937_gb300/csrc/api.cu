@@ -156,7 +156,7 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
         ctx->rec[s] = reinterpret_cast<compton::SortRec*>(base + o_rec[s]);
         ctx->stile[s] = reinterpret_cast<int32_t*>(base + o_stile[s]);
     }
-    ctx->unsorted = reinterpret_cast<int32_t*>(base + o_count) + 2 * C_pad;
+    ctx->unsorted = reinterpret_cast<uint32_t*>(base + o_count) + 2 * C_pad;
     ctx->block_sums = reinterpret_cast<int64_t*>(base + o_bs);
     ctx->cinfo = reinterpret_cast<CellInfo*>(base + o_ci);
     ctx->tile_cell = reinterpret_cast<int32_t*>(base + o_tc);

@@ -8,9 +8,9 @@
 //   k_scan_reduce  per-tile sums of N_e,c, N_g,c and M_c = min(N_e,c, N_g,c)
 //   k_scan_blocks  exclusive scan of the tile sums (one CTA)
 //   k_scan_final   per-cell offsets, CellInfo, tile maps; resets the cursors
-//   k_place        input not in cell order only: Philox key per particle,
-//                  (key, id, momentum) record placed in its cell's segment
-//                  (arbitrary order inside the segment)
+//   k_place        input not in cell order only: each particle's index (input
+//                  nearly in order) or its record (key, id, momentum) placed
+//                  in its cell's segment (arbitrary order inside the segment)
 //   k_sort_gather  per-cell sort by (key, id) in shared memory (a bucket
 //                  sort of each tile of whole cells), each particle written
 //                  to its sorted position
@@ -24,7 +24,12 @@ namespace compton {
 namespace {
 
 constexpr int kSortThreads = 128;
-constexpr int kPlaceThreads = 1024;  // threads per placement CTA
+constexpr int kPlaceThreads = 512;   // threads per placement CTA
+constexpr int kPlaceCtasPerSm = 16;  // placement CTAs per SM and species
+constexpr int kPlaceAloneCells = 4096;  // cells from which records are placed one atomic each (with a search for
+                                        // peers in the warp, 301 x 257 cells of 40 + 40 in no order: 361 against
+                                        // 348 us for the step; with few cells one address would serialise them)
+constexpr int kPlaceUnroll = 4;      // particles whose indices a thread places at once
 constexpr int kCountThreads = 1024;  // threads per histogram CTA (256, 512: 1 us slower)
 
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
@@ -37,8 +42,9 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // cancels), costs one atomic per element of shuffled input and two per run
 // of input in cell order.  Each thread takes four consecutive positions with
 // one vector load; the neighbours across threads come by shuffle.
-// unsorted[s] is set if a cell index descends or lies outside [0, C): only
-// then does the placement run.
+// unsorted[s] counts the positions at which the cell index descends, plus one
+// per warp that saw an index outside [0, C): only if it is not zero does the
+// placement run, and by its size the placement takes its form (sort_source).
 // ---------------------------------------------------------------------------
 template <typename Idx>
 __device__ __forceinline__ int4 load_cells4(const int32_t* __restrict__ cell, Idx i, Idx n, bool vec)
@@ -58,7 +64,7 @@ template <typename Idx>
 __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restrict__ cell_e, int64_t n_e,
                                                         const int32_t* __restrict__ cell_g, int64_t n_g, int64_t C,
                                                         int32_t* __restrict__ count_e, int32_t* __restrict__ count_g,
-                                                        int32_t* __restrict__ unsorted, DeviceStats* stats)
+                                                        uint32_t* __restrict__ unsorted, DeviceStats* stats)
 {
     const int s = blockIdx.y;
     const int32_t* __restrict__ cell = s == 0 ? cell_e : cell_g;
@@ -70,7 +76,8 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
     const bool vec = (reinterpret_cast<uintptr_t>(cell) & 15u) == 0;
     // cell indices are int32, so C above 2^31 admits every non-negative one
     const uint32_t C32 = C > 0x80000000ll ? 0x80000000u : (uint32_t)C;
-    bool disorder = false, bad = false;
+    uint32_t descents = 0;
+    bool bad = false;
     // the next group's loads are issued before this group is processed, so
     // two groups per thread are in flight
     auto edge = [&](Idx j0) -> int32_t {
@@ -110,7 +117,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
                 const int32_t nc = j == 3 ? next : v[j + 1];
                 const bool ok = (uint32_t)c < C32;
                 bad |= !ok;
-                disorder |= pc > c;
+                descents += pc > c;
                 const bool first = pc != c, last = nc != c;
                 if (ok && (first || last))
                     atomicAdd(&count[c], (last ? base + j + 1 : 0) - (first ? base + j : 0));
@@ -126,15 +133,35 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
             const int32_t nc = j == 3 ? next : v[j + 1];
             const bool ok = c >= 0 && (int64_t)c < C;
             bad |= !ok;
-            disorder |= i > 0 && pc > c;
+            descents += i > 0 && pc > c;
             const bool first = ok && (i == 0 || pc != c);
             const bool last = ok && (i + 1 == n || nc != c);
             if (first || last)
                 atomicAdd(&count[c], (last ? (int32_t)(i + 1) : 0) - (first ? (int32_t)i : 0));
         }
     }
-    if (__any_sync(0xffffffffu, bad) && lane == 0) atomicOr(&stats->error_flags, (unsigned long long)kErrCellRange);
-    if (__any_sync(0xffffffffu, disorder || bad) && lane == 0) atomicOr(&unsorted[s], 1);
+    const bool any_bad = __any_sync(0xffffffffu, bad);
+    descents = __reduce_add_sync(0xffffffffu, descents);
+    if (lane == 0) {
+        if (any_bad) atomicOr(&stats->error_flags, (unsigned long long)kErrCellRange);
+        if (descents + any_bad) atomicAdd(&unsorted[s], descents + any_bad);
+    }
+}
+
+// Where the sort reads a species from.  In cell order: the input arrays in
+// place.  With fewer descents than a quarter of the particles (a plasma after
+// a push, where some crossed into a neighbouring cell; a few ordered runs one
+// after another) most of a cell's particles are neighbours in the input: the
+// placement writes each particle's index (4 bytes) and the sort gathers
+// through it.  Above that (particles in no order: half the positions descend)
+// a gather would fetch a 32-byte sector per word, and whole records are placed.
+// 512^2 cells, 64 + 64 per cell, a tenth of them moved: the placement takes
+// 0.087 ms by index and 0.368 ms by record, the sort after it 0.34 ms each.
+enum SortSource : int { kInPlace = 0, kByIndex = 1, kRecords = 2 };
+__device__ __forceinline__ SortSource sort_source(uint32_t unsorted, int64_t n)
+{
+    if (unsorted == 0) return kInPlace;
+    return (int64_t)unsorted * 4 < n ? kByIndex : kRecords;
 }
 
 // ---------------------------------------------------------------------------
@@ -330,12 +357,13 @@ __global__ void __launch_bounds__(256) k_scan_final(ScanFinalArgs a)
 }
 
 // ---------------------------------------------------------------------------
-// Keyed placement of input not yet in cell order: each particle's record
-// (Philox key, id, momentum, weight if any) goes to off[c] + cursor.  A record fills one
-// aligned 32-byte sector, written as two 16-byte stores, so the scattered
-// writes never leave partly written sectors behind.  Input already in cell
-// order (k_count found no descent and no bad index) skips this kernel: the
-// sort then reads the input arrays in place.
+// Placement of input not in cell order: each particle takes the next place of
+// its cell's segment (off[c] + cursor), where its index or its record (Philox
+// key, id, momentum, weight if any) is written.  A record fills one aligned
+// 32-byte sector, written as two 16-byte stores, so the scattered writes never
+// leave partly written sectors behind.  Input already in cell order skips
+// this kernel.  The kernel is bound by the latency of each particle's chain
+// (cell index, cursor atomic, write).
 // ---------------------------------------------------------------------------
 struct PlaceArgs {
     const int32_t* cell[2];
@@ -345,10 +373,10 @@ struct PlaceArgs {
     int64_t n[2];
     const int32_t* off[2];
     int32_t* cursor[2];
-    const int32_t* unsorted;
-    SortRec* rec[2];
+    const uint32_t* unsorted;
+    SortRec* rec[2];  // records, or (kByIndex) the indices as int32
     int64_t C;
-    uint64_t seed, step;
+    KeyDraw draw;
 };
 
 __device__ __forceinline__ void store_rec(SortRec* r, uint32_t key, uint32_t pid, float ux, float uy, float uz,
@@ -362,43 +390,76 @@ __device__ __forceinline__ void store_rec(SortRec* r, uint32_t key, uint32_t pid
 // The weight a record carries (its first padding word).
 __device__ __forceinline__ float rec_weight(const SortRec* r) { return __uint_as_float(r->pad[0]); }
 
-__global__ void __launch_bounds__(kPlaceThreads) k_place(PlaceArgs a)
+// The next places of the cells of the warp's 32 particles, one cursor atomic
+// per distinct cell: the group's first place in its leader, and this lane's
+// leader and rank in its group.
+__device__ __forceinline__ void claim_places(const int32_t* __restrict__ off, int32_t* __restrict__ cursor, int c,
+                                             int& first_place, int& leader, int& rank)
+{
+    const unsigned lane = lane_id();
+    const unsigned peers = __match_any_sync(0xffffffffu, c);
+    leader = __ffs(peers) - 1;
+    rank = __popc(peers & ((1u << lane) - 1u));
+    first_place = 0;
+    if (c >= 0 && lane == (unsigned)leader) first_place = off[c] + atomicAdd(&cursor[c], __popc(peers));
+}
+
+__global__ void __launch_bounds__(kPlaceThreads, 2048 / kPlaceThreads) k_place(const __grid_constant__ PlaceArgs a)
 {
     const int s = blockIdx.y;
-    if (a.unsorted[s] == 0) return;
     const int64_t n = a.n[s];
+    const SortSource source = sort_source(a.unsorted[s], n);
+    if (source == kInPlace) return;
     const int32_t* __restrict__ cell = a.cell[s];
-    const uint32_t* __restrict__ id = a.id[s];
-    const float* __restrict__ u0 = a.u[s][0];
-    const float* __restrict__ u1 = a.u[s][1];
-    const float* __restrict__ u2 = a.u[s][2];
-    const float* __restrict__ wt = a.w[s];
     const int32_t* __restrict__ off = a.off[s];
     int32_t* __restrict__ cursor = a.cursor[s];
-    SortRec* __restrict__ rec = a.rec[s];
-    const uint32_t stream = s == 0 ? kStreamPairE : kStreamPairG;
-    const int64_t stride = (int64_t)gridDim.x * blockDim.x;
-    const int64_t n_round = (n + 31) / 32 * 32;
     const unsigned lane = lane_id();
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n_round; i += stride) {
-        int c = -1;
-        uint32_t key = 0, pid = 0;
-        if (i < n) {
-            const int32_t ci = cell[i];
-            if (ci >= 0 && (int64_t)ci < a.C) {
-                c = ci;
-                pid = id[i];
-                key = draw(a.seed, a.step, stream, pid).r0;
+    const int64_t warp = (int64_t)blockIdx.x * (kPlaceThreads / 32) + (threadIdx.x >> 5);
+    const int64_t n_warps = (int64_t)gridDim.x * (kPlaceThreads / 32);
+    auto load_cell = [&](int64_t i) {
+        const int32_t ci = i < n ? cell[i] : -1;
+        return ci >= 0 && (int64_t)ci < a.C ? ci : -1;
+    };
+    if (source == kByIndex) {
+        // a warp takes runs of kPlaceUnroll * 32 consecutive particles, their
+        // chains (cell, cursor atomic, index) in flight together
+        int32_t* __restrict__ idx = reinterpret_cast<int32_t*>(a.rec[s]);
+        constexpr int kRun = 32 * kPlaceUnroll;
+        for (int64_t r0 = warp * kRun; r0 < n; r0 += n_warps * kRun) {
+            int c[kPlaceUnroll], place[kPlaceUnroll], rank[kPlaceUnroll], leader[kPlaceUnroll];
+#pragma unroll
+            for (int k = 0; k < kPlaceUnroll; ++k) c[k] = load_cell(r0 + 32 * k + lane);
+#pragma unroll
+            for (int k = 0; k < kPlaceUnroll; ++k) claim_places(off, cursor, c[k], place[k], leader[k], rank[k]);
+#pragma unroll
+            for (int k = 0; k < kPlaceUnroll; ++k) {
+                const int base = __shfl_sync(0xffffffffu, place[k], leader[k]);
+                if (c[k] >= 0) idx[(int64_t)base + rank[k]] = (int32_t)(r0 + 32 * k + lane);
             }
         }
-        const unsigned peers = __match_any_sync(0xffffffffu, c);
-        const int leader = __ffs(peers) - 1;
-        int base = 0;
-        if (c >= 0 && lane == (unsigned)leader) base = atomicAdd(&cursor[c], __popc(peers));
-        base = __shfl_sync(peers, base, leader);
+        return;
+    }
+    // whole records.  Particles in no order among many cells seldom share one
+    // within a warp: each takes its own place, with no search for peers
+    const uint32_t* __restrict__ id = a.id[s];
+    const float* __restrict__ wt = a.w[s];
+    SortRec* __restrict__ rec = a.rec[s];
+    const bool alone = a.C >= kPlaceAloneCells;
+    for (int64_t r0 = warp * 32; r0 < n; r0 += n_warps * 32) {
+        const int64_t i = r0 + lane;
+        const int c = load_cell(i);
+        int64_t slot = 0;
+        if (alone) {
+            if (c >= 0) slot = (int64_t)off[c] + atomicAdd(&cursor[c], 1);
+        } else {
+            int place, leader, rank;
+            claim_places(off, cursor, c, place, leader, rank);
+            slot = (int64_t)__shfl_sync(0xffffffffu, place, leader) + rank;
+        }
         if (c >= 0) {
-            const int64_t slot = (int64_t)off[c] + base + __popc(peers & ((1u << lane) - 1u));
-            store_rec(rec + slot, key, pid, u0[i], u1[i], u2[i], wt ? wt[i] : 0.0f);
+            const uint32_t pid = id[i];
+            const float u0 = a.u[s][0][i], u1 = a.u[s][1][i], u2 = a.u[s][2][i], w = wt ? wt[i] : 0.0f;
+            store_rec(rec + slot, a.draw.word0(s, pid), pid, u0, u1, u2, w);
         }
     }
 }
@@ -426,23 +487,26 @@ struct SortGatherArgs {
     float* out_u[2][3];
     int32_t* out_cell[2];
     uint32_t* out_id[2];
-    SortRec* rec[2];
+    SortRec* rec[2];  // placed records, or (kByIndex) indices
     const int32_t* off[2];
     const int32_t* stile[2];
-    const int32_t* unsorted;
+    const uint32_t* unsorted;
+    int64_t n[2];
     int64_t nb_e;
-    uint64_t seed, step;
+    KeyDraw draw;
 };
 
-// Where a species' particles are read from: the placed records, or (input in
-// cell order) the input arrays, with keys drawn from the ids.
+// Where a species' particles are read from: the placed records, or the input
+// arrays (in place or through the placed indices), with keys drawn from the ids.
 struct SortSrc {
-    const SortRec* rec;  // nullptr: read the input arrays in place
+    const SortRec* rec;  // kRecords, else nullptr
+    const int32_t* idx;  // kByIndex, else nullptr
     const uint32_t* id;
     const float* u[3];
-    const float* w;      // weights (in place), or nullptr
-    uint64_t seed, step;
-    uint32_t stream;
+    const float* w;      // weights, or nullptr
+
+    // the input index of position p (no records)
+    __device__ __forceinline__ int64_t input(int64_t p) const { return idx ? (int64_t)idx[p] : p; }
 };
 
 // The order inside a cell is by (key, id), with the tile slot breaking ties
@@ -532,21 +596,22 @@ __device__ __forceinline__ void block_scan_counts(int32_t* cnt, int R)
 __device__ __forceinline__ void sort_tile_block(const SortGatherArgs& g, int s, const SortSrc& t, const SortSmem& m,
                                                 int64_t c0, int64_t c1, int64_t o0, int R)
 {
-    const int tid = threadIdx.x, lane = (int)lane_id(), w = tid >> 5;
+    const int tid = threadIdx.x;
     const int32_t* __restrict__ off = g.off[s];
     constexpr int kPer = (kSortCap + kSortThreads - 1) / kSortThreads;
     uint32_t key[kPer], pid[kPer];
-    // input in cell order: issue the tile's loads first, so they are in
+    // from the input arrays: issue the tile's loads first, so they are in
     // flight while the cell map is built
     if (!t.rec) {
 #pragma unroll
         for (int k = 0; k < kPer; ++k) {
             const int i = tid + k * kSortThreads;
             if (i < R) {
-                cp_async4(&m.us[0][i], t.u[0] + o0 + i);
-                cp_async4(&m.us[1][i], t.u[1] + o0 + i);
-                cp_async4(&m.us[2][i], t.u[2] + o0 + i);
-                pid[k] = t.id[o0 + i];
+                const int64_t q = t.input(o0 + i);
+                cp_async4(&m.us[0][i], t.u[0] + q);
+                cp_async4(&m.us[1][i], t.u[1] + q);
+                cp_async4(&m.us[2][i], t.u[2] + q);
+                pid[k] = t.id[q];
             }
         }
     }
@@ -559,13 +624,15 @@ __device__ __forceinline__ void sort_tile_block(const SortGatherArgs& g, int s, 
         for (int i = tid; i <= n_cells; i += kSortThreads) offs[i] = off[c0 + i] - (int32_t)o0;
     for (int i = tid; i < kBucketsPerSlot * R; i += kSortThreads) m.cnt[i] = 0;
     __syncthreads();
-    // cell of every position (warp per cell) and the output cell indices
-    for (int64_t c = c0 + w; c < c1; c += kSortThreads / 32) {
-        const int a = staged ? offs[c - c0] : off[c] - (int32_t)o0;
-        const int n = (staged ? offs[c - c0 + 1] : off[c + 1] - (int32_t)o0) - a;
-        for (int j = lane; j < n; j += 32) {
+    // cell of every position and the output cell indices: a group of lanes per
+    // cell, 32, or 16 or 8 where the tile's cells hold that few on average
+    const int gs = R > 16 * n_cells ? 5 : (R > 8 * n_cells ? 4 : 3);
+    for (int ci = tid >> gs; ci < n_cells; ci += kSortThreads >> gs) {
+        const int a = staged ? offs[ci] : off[c0 + ci] - (int32_t)o0;
+        const int n = (staged ? offs[ci + 1] : off[c0 + ci + 1] - (int32_t)o0) - a;
+        for (int j = tid & ((1 << gs) - 1); j < n; j += 1 << gs) {
             m.cmap[a + j] = (uint32_t)a | ((uint32_t)n << 16);
-            g.out_cell[s][o0 + a + j] = (int32_t)c;
+            g.out_cell[s][o0 + a + j] = (int32_t)(c0 + ci);
         }
     }
     // keys (and, from placed records, momenta)
@@ -580,7 +647,7 @@ __device__ __forceinline__ void sort_tile_block(const SortGatherArgs& g, int s, 
         for (int k = 0; k < kPer; ++k) {
             const int i = tid + k * kSortThreads;
             if (i < R) {
-                key[k] = draw(t.seed, t.step, t.stream, pid[k]).r0;
+                key[k] = g.draw.word0(s, pid[k]);
                 m.id[i] = pid[k];
             }
         }
@@ -674,45 +741,65 @@ __device__ __forceinline__ void sort_tile_block(const SortGatherArgs& g, int s, 
         g.out_id[s][go] = m.id[i];
         // the weight is not staged: read once more where the tile came from
         // (a sector this block has just read)
-        if (g.out_w[s]) g.out_w[s][go] = t.rec ? rec_weight(t.rec + o0 + i) : t.w[o0 + i];
+        if (g.out_w[s]) g.out_w[s][go] = t.rec ? rec_weight(t.rec + o0 + i) : t.w[t.input(o0 + i)];
     }
 }
 
-// A cell larger than the shared-memory capacity: records in global memory
-// (materialised from the input first when the placement was skipped), each
-// particle ranked against the whole cell by the block.
+// A cell larger than the shared-memory capacity, ranked in global memory by
+// the block: the cell's own part of the output arrays is the scratch, first
+// for the keys and ids, then for the source position of every sorted place.
 __device__ void sort_giant_cell(const SortGatherArgs& g, int s, const SortSrc& t, int64_t o, int64_t n, int32_t c)
 {
-    SortRec* rec = g.rec[s];
-    if (!t.rec) {
-        for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-            const uint32_t pid = t.id[o + i];
-            store_rec(rec + o + i, draw(t.seed, t.step, t.stream, pid).r0, pid, t.u[0][o + i], t.u[1][o + i],
-                      t.u[2][o + i], t.w ? t.w[o + i] : 0.0f);
-        }
-        __syncthreads();
-    }
+    uint32_t* key = reinterpret_cast<uint32_t*>(g.out_u[s][0]) + o;
+    uint32_t* id = g.out_id[s] + o;
+    int32_t* src = g.out_cell[s] + o;
     for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
-        const SortRec ri = rec[o + i];
+        if (t.rec) {
+            key[i] = t.rec[o + i].key;
+            id[i] = t.rec[o + i].id;
+        } else {
+            const uint32_t pid = t.id[t.input(o + i)];
+            key[i] = g.draw.word0(s, pid);
+            id[i] = pid;
+        }
+    }
+    __syncthreads();
+    for (int64_t i = threadIdx.x; i < n; i += blockDim.x) {
+        const uint32_t ki = key[i], di = id[i];
         int64_t rank = 0;
         for (int64_t j = 0; j < n; ++j) {
-            const uint32_t kj = rec[o + j].key, dj = rec[o + j].id;
-            rank += (kj < ri.key) | ((kj == ri.key) & ((dj < ri.id) | ((dj == ri.id) & (j < i))));
+            const uint32_t kj = key[j], dj = id[j];
+            rank += (kj < ki) | ((kj == ki) & ((dj < di) | ((dj == di) & (j < i))));
         }
-        const int64_t p = o + rank;
-        g.out_u[s][0][p] = ri.ux;
-        g.out_u[s][1][p] = ri.uy;
-        g.out_u[s][2][p] = ri.uz;
-        g.out_cell[s][p] = c;
-        g.out_id[s][p] = ri.id;
-        if (g.out_w[s]) g.out_w[s][p] = rec_weight(&ri);
+        src[rank] = (int32_t)i;
+    }
+    __syncthreads();
+    for (int64_t p = threadIdx.x; p < n; p += blockDim.x) {
+        const int64_t q = o + src[p];
+        float x, y, z, wt = 0.0f;
+        if (t.rec) {
+            const SortRec r = t.rec[q];
+            x = r.ux, y = r.uy, z = r.uz;
+            id[p] = r.id;
+            wt = rec_weight(&r);
+        } else {
+            const int64_t i = t.input(q);
+            x = t.u[0][i], y = t.u[1][i], z = t.u[2][i];
+            id[p] = t.id[i];
+            if (g.out_w[s]) wt = t.w[i];
+        }
+        g.out_u[s][0][o + p] = x;
+        g.out_u[s][1][o + p] = y;
+        g.out_u[s][2][o + p] = z;
+        if (g.out_w[s]) g.out_w[s][o + p] = wt;
+        src[p] = c;
     }
     __syncthreads();
 }
 
 constexpr size_t kSortSmem = (size_t)kSortCap * (4 + 4 * kBucketsPerSlot + 4 + 12 + 2 + 2);
 
-__global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(SortGatherArgs g)
+__global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(const __grid_constant__ SortGatherArgs g)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem m;
@@ -736,14 +823,12 @@ __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(SortGatherArgs
     if (R <= 0) return;
 
     SortSrc t;
-    const bool placed = g.unsorted[s] != 0;
-    t.rec = placed ? g.rec[s] : nullptr;
+    const SortSource source = sort_source(g.unsorted[s], g.n[s]);
+    t.rec = source == kRecords ? g.rec[s] : nullptr;
+    t.idx = source == kByIndex ? reinterpret_cast<const int32_t*>(g.rec[s]) : nullptr;
     t.id = g.in_id[s];
     for (int k = 0; k < 3; ++k) t.u[k] = g.in_u[s][k];
     t.w = g.in_w[s];
-    t.seed = g.seed;
-    t.step = g.step;
-    t.stream = s == 0 ? kStreamPairE : kStreamPairG;
 
     if (R <= kSortCap) {
         sort_tile_block(g, s, t, m, c0, c1, o0, (int)R);
@@ -768,13 +853,10 @@ __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(SortGatherArgs
     }
 }
 
-// CTAs per SM and species of the grid-stride histogram and placement (the
-// launches' second grid dimension takes the two species).  The histogram
-// runs in one wave of 1024-thread CTAs: 0.0394 ms on the 512^2 step against
-// 0.0404 with four and 0.0435 with eight.  The placement keeps four: with
-// two, binning shuffled input took 1.46 against 1.28 ms.
+// CTAs per SM and species of the grid-stride histogram (the launch's second
+// grid dimension takes the two species), which runs in one wave of 1024-thread CTAs: 0.0394 ms on the 512^2 step against
+// 0.0404 with four and 0.0435 with eight.
 constexpr int kCountCtasPerSm = 2;
-constexpr int kPlaceCtasPerSm = 4;
 
 int grid_for(int64_t n, int threads, int max_blocks)
 {
@@ -794,15 +876,12 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
     const int64_t ne = e_in->n, ng = g_in->n;
     const int64_t n_tiles = (C + kScanTile - 1) / kScanTile;
     // count[0], count[1] and unsorted lie in one block of the workspace
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->count[0], 0, sizeof(int32_t) * (ctx->unsorted + 2 - ctx->count[0]),
+    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->count[0], 0,
+                                          reinterpret_cast<char*>(ctx->unsorted + 2) -
+                                              reinterpret_cast<char*>(ctx->count[0]),
                                           stream));
 
     const int64_t nmax = ne > ng ? ne : ng;
-    // grid-stride kernels: CTAs per SM of the histogram and the placement,
-    // both in 1024-thread CTAs (the placement: as many threads as sixteen
-    // 256-thread CTAs per SM, whose placement of shuffled input one wave of
-    // fewer threads made 0.3 ms longer, in a quarter of the CTAs, so its
-    // early exit for input in cell order is shorter)
     const dim3 cgrid(grid_for((nmax + 3) / 4, kCountThreads, ctx->n_sm * kCountCtasPerSm), 2);  // four per thread
     {
         TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
@@ -870,8 +949,7 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
     }
     pa.unsorted = ctx->unsorted;
     pa.C = C;
-    pa.seed = ctx->cfg.seed;
-    pa.step = step;
+    pa.draw = KeyDraw(ctx->cfg.seed, step, kStreamPairE, kStreamPairG);
     {
         TimedScope ts_(ctx, COMPTON_K_PLACE, stream);
         k_place<<<pgrid, kPlaceThreads, 0, stream>>>(pa);
@@ -895,10 +973,10 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
             sg.rec[s] = ctx->rec[s];
             sg.off[s] = ctx->off[s];
             sg.stile[s] = ctx->stile[s];
+            sg.n[s] = ins[s]->n;
         }
+        sg.draw = pa.draw;
         sg.unsorted = ctx->unsorted;
-        sg.seed = ctx->cfg.seed;
-        sg.step = step;
         sg.nb_e = nb_e;
         const int smem = (int)kSortSmem;
         COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_sort_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
