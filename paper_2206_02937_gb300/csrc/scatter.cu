@@ -563,7 +563,7 @@ __global__ void __launch_bounds__(256) k_collide(ScatterArgs a)
 }
 
 // No-Time-Counter candidate selection (Sec. 3.1, second step; Bird 1989),
-// one thread per cell: the cell draws N = floor(E + U) candidates with
+// per cell: the cell draws N = floor(E + U) candidates with
 // E = N_e N_g (w/V) 2 dt (sigma_max v_max = 2 sigma_T c) and U from
 // Philox(c, step, 5); candidate j takes the block (c, step, 6 | j << 8):
 // word 0 picks the electron, word 1 the photon, the pair collides iff the
@@ -598,8 +598,10 @@ __device__ __forceinline__ int32_t ntc_count(const NtcArgs& a, int32_t c, int ne
     return (int32_t)floor(__dadd_rn(expect, uc));
 }
 
-// Cells with at least this many candidates are taken by a whole warp.
-constexpr int kNtcBig = 32;
+// Cells with at least this many candidates are listed and taken first, one at
+// a time; the others in runs of kNtcCells.
+constexpr int kNtcBig = 64;
+constexpr int kNtcCells = 8;
 
 __device__ __forceinline__ int pick_index(uint32_t w, int n) { return (int)(((uint64_t)w * (uint64_t)n) >> 32); }
 
@@ -623,154 +625,247 @@ __global__ void __launch_bounds__(256) k_ntc_scan(NtcArgs a)
     if ((threadIdx.x & 31u) == 0 && n_cand) atomicAdd(&a.stats->pairs_tested, n_cand);
 }
 
-// The candidates of cell c from candidate j0 on, by the whole warp, exact
-// and in order: the warp evaluates the next 32 candidates at once on the
-// momenta as they are; candidate k's evaluation is what the sequence would
-// give unless an earlier candidate of the batch was accepted and shares its
-// electron or photon.  The candidates before the first such k are final:
-// their accepted ones (which share no particle) collide and write back, and
-// the next batch starts at k with the updated momenta.
-__device__ __forceinline__ unsigned long long ntc_cell_warp(const NtcArgs& a, int32_t c)
+// NTC, second pass.  Each warp runs a stream of candidates, cell after cell and
+// in order within a cell, 32 at a time: it evaluates the 32 next candidates at
+// once on the momenta as they are, and queues the accepted ones; 32 queued
+// collisions are resolved at once, so that both the evaluation and the far
+// longer collision run with every lane busy (one candidate of a cell after
+// another, the collision code ran at the acceptance rate, a fifth of the
+// lanes).  Exactly the in-order result: a candidate is held back, and presented
+// again ahead of all later ones, if one of its particles takes part in a queued
+// collision, or in an earlier candidate of the 32 that was accepted or is held
+// back itself; held candidates keep their order, so whatever is evaluated has
+// every earlier collision of its particles behind it.  The particles of queued
+// collisions are marked in two per-warp bit sets by their index modulo the
+// set's size (a false hit only holds a candidate back once more); the warp's
+// 32 candidates are compared by match.any.
+//
+// What bounds it: the latency of a batch's chain (draw, scattered loads,
+// evaluation).  256^2 cells of 64 + 64, half a million candidates: 142 us with
+// a lane per cell (a warp per long cell), 64 us so.
+constexpr int kNtcWarps = 8;
+constexpr uint32_t kNtcBits = 4096;  // bits per set
+struct NtcWarp {
+    uint32_t busy_e[kNtcBits / 32], busy_g[kNtcBits / 32];
+    float u[3][64], k[3][64], x[64], F2[64];  // queued collisions (at most 31 + 32)
+    int32_t ie[64], ig[64], c[64], j[64];
+    uint32_t r3[64];
+    int32_t lane[32];  // the lanes of the held candidates, in order
+};
+
+__device__ __forceinline__ void ntc_mark(NtcWarp& W, int ie, int ig)
 {
-    const unsigned lane = threadIdx.x & 31u;
+    const uint32_t be = (uint32_t)ie % kNtcBits, bg = (uint32_t)ig % kNtcBits;
+    atomicOr(&W.busy_e[be >> 5], 1u << (be & 31u));
+    atomicOr(&W.busy_g[bg >> 5], 1u << (bg & 31u));
+}
+
+// Resolve the first min(n, 32) queued collisions and write their momenta back;
+// the rest move to the front and stay marked.  Returns how many are left.
+__device__ __forceinline__ int ntc_resolve(const NtcArgs& a, NtcWarp& W, int n)
+{
+    const int lane = (int)(threadIdx.x & 31u);
+    __syncwarp();
+    const int done = n < 32 ? n : 32;
+    if (lane < done) {
+        float ux = W.u[0][lane], uy = W.u[1][lane], uz = W.u[2][lane];
+        float kx = W.k[0][lane], ky = W.k[1][lane], kz = W.k[2][lane];
+        const float x = W.x[lane];
+        const int ie = W.ie[lane], ig = W.ig[lane];
+        const Philox4 z = draw(a.seed, a.step, 7u | ((uint32_t)W.j[lane] << 8), (uint32_t)W.c[lane]);
+        const Angle ang = kn_sample_angle(x, W.r3[lane] >> 8, W.F2[lane]);
+        collide_pair(ux, uy, uz, kx, ky, kz, x, ang, u24_closed0(z.r0), a.collide64_sq);
+        a.u[0][ie] = ux;
+        a.u[1][ie] = uy;
+        a.u[2][ie] = uz;
+        a.k[0][ig] = kx;
+        a.k[1][ig] = ky;
+        a.k[2][ig] = kz;
+        W.busy_e[((uint32_t)ie % kNtcBits) >> 5] = 0u;
+        W.busy_g[((uint32_t)ig % kNtcBits) >> 5] = 0u;
+    }
+    __syncwarp();
+    const int left = n - done;
+    if (lane < left) {
+        const int q = 32 + lane;
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            W.u[i][lane] = W.u[i][q];
+            W.k[i][lane] = W.k[i][q];
+        }
+        W.x[lane] = W.x[q];
+        W.F2[lane] = W.F2[q];
+        W.ie[lane] = W.ie[q];
+        W.ig[lane] = W.ig[q];
+        W.c[lane] = W.c[q];
+        W.j[lane] = W.j[q];
+        W.r3[lane] = W.r3[q];
+        ntc_mark(W, W.ie[lane], W.ig[lane]);  // (a cleared word may have held its bit)
+    }
+    __syncwarp();
+    return left;
+}
+
+__global__ void __launch_bounds__(32 * kNtcWarps, 3) k_ntc(NtcArgs a)
+{
+    __shared__ NtcWarp s_warp[kNtcWarps];
+    NtcWarp& W = s_warp[threadIdx.x >> 5];
+    const int lane = (int)(threadIdx.x & 31u);
+    const unsigned lt_mask = (1u << lane) - 1u;
+    for (uint32_t i = (uint32_t)lane; i < kNtcBits / 32; i += 32) W.busy_e[i] = W.busy_g[i] = 0u;
+    __syncwarp();
+    const uint32_t n_big = *a.n_big;
+    const uint32_t n_runs = (uint32_t)((a.n_cells + kNtcCells - 1) / kNtcCells);
     unsigned long long n_coll = 0;
-    const int e0 = a.off_e[c], ne = a.off_e[c + 1] - e0;
-    const int g0 = a.off_g[c], ng = a.off_g[c + 1] - g0;
-    const int32_t nc = ntc_count(a, c, ne, ng);
-    for (int32_t j0 = 0; j0 < nc;) {
-        const int32_t j = j0 + (int32_t)lane;
-        const bool valid = j < nc;
-        int ie = -1, ig = -1;
-        bool acc = false;
+    bool big = true, more = true;
+    // the cells of the stream at hand: lane t < kNtcCells holds cell t of the run
+    int c = 0, e0 = 0, ne = 0, g0 = 0, ng = 0, pre = 0;  // pre: candidates of the run's earlier cells
+    int total = 0, pos = 0;                              // candidates of the run, and taken (the same in every lane)
+    // this lane's candidate
+    int cc = 0, cj = 0, ie = 0, ig = 0;
+    uint32_t r2 = 0, r3 = 0;
+    unsigned held = 0;  // lanes whose candidate is held back
+    int n_pend = 0;
+    for (;;) {
+        // ---- the held candidates first, in order ----
+        int filled = __popc(held);
+        if (held) {
+            if ((held >> lane) & 1u) W.lane[__popc(held & lt_mask)] = lane;
+            __syncwarp();
+            const int src = lane < filled ? W.lane[lane] : 0;
+            cc = __shfl_sync(0xffffffffu, cc, src);
+            cj = __shfl_sync(0xffffffffu, cj, src);
+            ie = __shfl_sync(0xffffffffu, ie, src);
+            ig = __shfl_sync(0xffffffffu, ig, src);
+            r2 = __shfl_sync(0xffffffffu, r2, src);
+            r3 = __shfl_sync(0xffffffffu, r3, src);
+        }
+        // ---- then the next of the stream ----
+        while (filled < 32) {
+            if (pos == total) {
+                if (!more) break;
+                // the next cells: a listed one, or a run
+                uint32_t w = 0;
+                if (lane == 0) w = atomicAdd(big ? a.next_big : a.next, 1u);
+                w = __shfl_sync(0xffffffffu, w, 0);
+                if (w >= (big ? n_big : n_runs)) {
+                    if (big) big = false;
+                    else more = false;
+                    continue;
+                }
+                const int64_t first = big ? (int64_t)a.big[w] : (int64_t)w * kNtcCells;
+                int cnt = 0;
+                if (lane < (big ? 1 : kNtcCells) && first + lane < a.n_cells) {
+                    c = (int)first + lane;
+                    e0 = a.off_e[c];
+                    ne = a.off_e[c + 1] - e0;
+                    g0 = a.off_g[c];
+                    ng = a.off_g[c + 1] - g0;
+                    if (ne > 0 && ng > 0) cnt = ntc_count(a, c, ne, ng);
+                    if (!big && cnt >= kNtcBig) cnt = 0;  // listed
+                }
+                int inc = cnt;
+#pragma unroll
+                for (int d = 1; d < kNtcCells; d <<= 1) {
+                    const int o = __shfl_up_sync(0xffffffffu, inc, d);
+                    if (lane >= d) inc += o;
+                }
+                pre = inc - cnt;
+                total = __shfl_sync(0xffffffffu, inc, kNtcCells - 1);
+                pos = 0;
+                continue;
+            }
+            const int take = total - pos < 32 - filled ? total - pos : 32 - filled;
+            const int q = pos + lane - filled;  // candidate of the run
+            const bool mine = lane >= filled && lane < filled + take;
+            int t = 0;  // its cell: the last whose first candidate is not after it
+#pragma unroll
+            for (int d = kNtcCells / 2; d >= 1; d >>= 1) {
+                const int p = __shfl_sync(0xffffffffu, pre, t + d);
+                if (p <= q) t += d;
+            }
+            const int tc = __shfl_sync(0xffffffffu, c, t), tp = __shfl_sync(0xffffffffu, pre, t);
+            const int te0 = __shfl_sync(0xffffffffu, e0, t), tne = __shfl_sync(0xffffffffu, ne, t);
+            const int tg0 = __shfl_sync(0xffffffffu, g0, t), tng = __shfl_sync(0xffffffffu, ng, t);
+            if (mine) {
+                cc = tc;
+                cj = q - tp;
+                const Philox4 z = draw(a.seed, a.step, 6u | ((uint32_t)cj << 8), (uint32_t)cc);
+                ie = te0 + pick_index(z.r0, tne);
+                ig = tg0 + pick_index(z.r1, tng);
+                r2 = z.r2;
+                r3 = z.r3;
+            }
+            filled += take;
+            pos += take;
+        }
+        if (filled == 0) {  // the stream has ended
+            if (n_pend > 0) ntc_resolve(a, W, n_pend);
+            n_coll += n_pend;
+            break;
+        }
+        // ---- evaluate all of them on the momenta as they are ----
+        const bool have = lane < filled;
+        bool acc = false, hold = false;
         float ux = 0.0f, uy = 0.0f, uz = 0.0f, kx = 0.0f, ky = 0.0f, kz = 0.0f, x = 0.0f, F2 = 0.0f;
-        uint32_t r3 = 0;
-        if (valid) {
-            const Philox4 q = draw(a.seed, a.step, 6u | ((uint32_t)j << 8), (uint32_t)c);
-            ie = e0 + pick_index(q.r0, ne);
-            ig = g0 + pick_index(q.r1, ng);
+        if (have) {
             ux = a.u[0][ie];
             uy = a.u[1][ie];
             uz = a.u[2][ie];
             kx = a.k[0][ig];
             ky = a.k[1][ig];
             kz = a.k[2][ig];
+            const uint32_t be = (uint32_t)ie % kNtcBits, bg = (uint32_t)ig % kNtcBits;
+            hold = (((W.busy_e[be >> 5] >> (be & 31u)) | (W.busy_g[bg >> 5] >> (bg & 31u))) & 1u) != 0u;
             const Invariants inv = invariants_f32(ux, uy, uz, kx, ky, kz);
             float v = inv.v;
             x = inv.x;
             if (inv.gamma > a.gamma64) invariants_f64(ux, uy, uz, kx, ky, kz, &x, &v);
             F2 = kn_F2(x);
             const float ratio = inv.eps > 0.0f ? 0.5f * 0.375f * F2 * v : 0.0f;
-            acc = u24_closed0(q.r2) < ratio;
-            r3 = q.r3;
+            acc = u24_closed0(r2) < ratio;
         }
-        // the first candidate whose evaluation an earlier accepted one of the
-        // batch may have changed
-        bool stale = false;
+        // ---- which are final ----
+        const unsigned sharers = (__match_any_sync(0xffffffffu, have ? ie : -1 - lane) |
+                                  __match_any_sync(0xffffffffu, have ? ig : -1 - lane)) & lt_mask;
         const unsigned accm = __ballot_sync(0xffffffffu, acc);
-#pragma unroll 4
-        for (int i = 0; i < 31; ++i) {
-            const int iei = __shfl_sync(0xffffffffu, ie, i), igi = __shfl_sync(0xffffffffu, ig, i);
-            stale |= (int)lane > i && ((accm >> i) & 1u) && (iei == ie || igi == ig);
+        held = __ballot_sync(0xffffffffu, hold);
+        for (;;) {
+            const unsigned h = __ballot_sync(0xffffffffu, hold || (have && (sharers & (accm | held)) != 0u));
+            if (h == held) break;
+            held = h;
         }
-        const unsigned sm = __ballot_sync(0xffffffffu, stale && valid);
-        const int nv = nc - j0 < 32 ? nc - j0 : 32;
-        const int kf = sm ? __ffs(sm) - 1 : nv;  // candidates j0 .. j0 + kf - 1 are final
-        if ((int)lane < kf && acc) {
-            const Philox4 z = draw(a.seed, a.step, 7u | ((uint32_t)j << 8), (uint32_t)c);
-            const Angle ang = kn_sample_angle(x, r3 >> 8, F2);
-            collide_pair(ux, uy, uz, kx, ky, kz, x, ang, u24_closed0(z.r0), a.collide64_sq);
-            a.u[0][ie] = ux;
-            a.u[1][ie] = uy;
-            a.u[2][ie] = uz;
-            a.k[0][ig] = kx;
-            a.k[1][ig] = ky;
-            a.k[2][ig] = kz;
-            ++n_coll;
+        const bool push = acc && !((held >> lane) & 1u);
+        const unsigned pm = accm & ~held;
+        if (push) {
+            const int q = n_pend + __popc(pm & lt_mask);
+            W.u[0][q] = ux;
+            W.u[1][q] = uy;
+            W.u[2][q] = uz;
+            W.k[0][q] = kx;
+            W.k[1][q] = ky;
+            W.k[2][q] = kz;
+            W.x[q] = x;
+            W.F2[q] = F2;
+            W.ie[q] = ie;
+            W.ig[q] = ig;
+            W.c[q] = cc;
+            W.j[q] = cj;
+            W.r3[q] = r3;
+            ntc_mark(W, ie, ig);
         }
-        __syncwarp();  // the next batch reads the momenta written here
-        j0 += kf;
+        n_pend += __popc(pm);
+        __syncwarp();
+        // ---- collisions: 32 at a time; all of them once half the lanes are held back, or only held ones are left ----
+        if (n_pend >= 32) {
+            n_pend = ntc_resolve(a, W, n_pend);
+            n_coll += 32;
+        }
+        if (n_pend > 0 && (__popc(held) >= 16 || (held && !more && pos == total))) {
+            n_coll += n_pend;
+            n_pend = ntc_resolve(a, W, n_pend);
+        }
     }
-    return n_coll;
-}
-
-// NTC, second pass.  Warps first take the cells of many candidates from the
-// list, one cell per warp (ntc_cell_warp), so that the longest sequences
-// start at once; then every lane works through the candidates of the other
-// cells in order, taking the next cell from a shared counter when its cell
-// is done, so that a warp's lanes stay busy however unequal the cells'
-// candidate counts are.  A cell's candidates run in sequence, so the results
-// do not depend on which warp or lane takes the cell.
-__global__ void __launch_bounds__(256) k_ntc(NtcArgs a)
-{
-    const unsigned lane = threadIdx.x & 31u;
-    const unsigned lt_mask = (1u << lane) - 1u;
-    unsigned long long n_coll = 0;
-    const uint32_t n_big = *a.n_big;
-    for (;;) {
-        uint32_t w = 0;
-        if (lane == 0) w = atomicAdd(a.next_big, 1u);
-        w = __shfl_sync(0xffffffffu, w, 0);
-        if (w >= n_big) break;
-        n_coll += ntc_cell_warp(a, a.big[w]);
-    }
-    int64_t c = 0, nc = 0, j = 0;
-    int e0 = 0, ne = 0, g0 = 0, ng = 0;
-    bool done = false;
-    for (;;) {
-        // lanes with no candidate left take the next cells, one atomic per warp
-        const bool need = !done && j >= nc;
-        const unsigned want = __ballot_sync(0xffffffffu, need);
-        if (want) {
-            const int leader = __ffs(want) - 1;
-            uint32_t base = 0;
-            if ((int)lane == leader) base = atomicAdd(a.next, (uint32_t)__popc(want));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (need) {
-                c = (int64_t)base + __popc(want & lt_mask);
-                j = 0;
-                nc = 0;
-                if (c >= a.n_cells) {
-                    done = true;
-                } else {
-                    e0 = a.off_e[c];
-                    ne = a.off_e[c + 1] - e0;
-                    g0 = a.off_g[c];
-                    ng = a.off_g[c + 1] - g0;
-                    if (ne > 0 && ng > 0) {
-                        nc = ntc_count(a, (int32_t)c, ne, ng);
-                        if (nc >= kNtcBig) nc = 0;  // a listed cell: done above
-                    }
-                }
-            }
-        }
-        if (__all_sync(0xffffffffu, done)) break;
-        if (done || j >= nc) continue;
-        const Philox4 q = draw(a.seed, a.step, 6u | ((uint32_t)j << 8), (uint32_t)c);
-        const int ie = e0 + pick_index(q.r0, ne);
-        const int ig = g0 + pick_index(q.r1, ng);
-        float ux = a.u[0][ie], uy = a.u[1][ie], uz = a.u[2][ie];
-        float kx = a.k[0][ig], ky = a.k[1][ig], kz = a.k[2][ig];
-        const Invariants inv = invariants_f32(ux, uy, uz, kx, ky, kz);
-        float x = inv.x, v = inv.v;
-        if (inv.gamma > a.gamma64) invariants_f64(ux, uy, uz, kx, ky, kz, &x, &v);
-        const float F2 = kn_F2(x);
-        const float ratio = inv.eps > 0.0f ? 0.5f * 0.375f * F2 * v : 0.0f;
-        if (u24_closed0(q.r2) < ratio) {
-            const Philox4 z = draw(a.seed, a.step, 7u | ((uint32_t)j << 8), (uint32_t)c);
-            const Angle ang = kn_sample_angle(x, q.r3 >> 8, F2);
-            collide_pair(ux, uy, uz, kx, ky, kz, x, ang, u24_closed0(z.r0), a.collide64_sq);
-            a.u[0][ie] = ux;
-            a.u[1][ie] = uy;
-            a.u[2][ie] = uz;
-            a.k[0][ig] = kx;
-            a.k[1][ig] = ky;
-            a.k[2][ig] = kz;
-            ++n_coll;
-        }
-        ++j;
-    }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) n_coll += __shfl_xor_sync(0xffffffffu, n_coll, d);
     if (lane == 0 && n_coll) atomicAdd(&a.stats->scatters, n_coll);
 }
 
@@ -1008,17 +1103,18 @@ compton_status launch_scatter_ntc(compton_ctx* ctx, compton_species* e, compton_
     COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(a.next, 0, 3 * sizeof(uint32_t), stream));
     // persistent: the CTAs resident at once (work is taken cell by cell)
     int per_sm = 0;
-    COMPTON_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ntc, 256, 0));
+    COMPTON_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ntc, 32 * kNtcWarps, 0));
     if (per_sm < 1) per_sm = 1;
     int64_t blocks = (int64_t)ctx->n_sm * per_sm;
-    const int64_t need = (pairs->n_cells + 255) / 256;
+    // a warp per run of cells at most
+    const int64_t need = (pairs->n_cells + kNtcCells * kNtcWarps - 1) / (kNtcCells * kNtcWarps);
     if (blocks > need) blocks = need;
     {
         TimedScope ts_(ctx, COMPTON_K_NTC, stream);
         int64_t sb = (pairs->n_cells + 255) / 256;
         if (sb > (int64_t)ctx->n_sm * 8) sb = (int64_t)ctx->n_sm * 8;
         k_ntc_scan<<<(unsigned)sb, 256, 0, stream>>>(a);
-        k_ntc<<<(unsigned)blocks, 256, 0, stream>>>(a);
+        k_ntc<<<(unsigned)blocks, 32 * kNtcWarps, 0, stream>>>(a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_ntc");
     return COMPTON_OK;
