@@ -1,0 +1,63 @@
+"""The FP32 network kernel (warp tiles of 32 samples, 12 warps per CTA) at the
+edges of its tiles against the FP64 forward, and its SiLU on its own.
+
+Tolerances: |dr| <= 2e-6 as for every FP32 forward (64-term FP32 sums).  SiLU:
+relative 5e-7 for -87 < z (ex2.approx 2^-22, and the roundings of the sum, the
+Newton reciprocal and the product, 2^-24 each, and of the exponent's
+correction); below -87 (where SiLU is above -1.5e-36) absolute 1e-30."""
+import ctypes
+import os
+import shutil
+import subprocess
+
+import numpy as np
+import pytest
+
+from oracle import mlp as omlp
+from paper_2206_02937_gb300 import workloads as wl
+from tests.test_gpu_mlp import _run, _theta
+from tests.gpu_util import torch_cuda
+
+pytestmark = pytest.mark.gpu
+
+HERE = os.path.dirname(os.path.abspath(__file__))
+
+
+@pytest.mark.parametrize("features", [0, 1])
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 383, 4863, 4864, 4865, 58369])
+def test_tile_edges(n, features):
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    u, k = wl.c3(n, seed=40)
+    th = _theta(3, gain=1.5)
+    ref, _ = omlp.forward(th.astype(np.float32).astype(np.float64),
+                          omlp.features(u, k, mode="invariants" if features else "momenta"))
+    out, _ = _run(torch, th, u, k, [cg.MODE_MLP_FP32], calibrate=True, features=features)
+    assert np.abs(out[cg.MODE_MLP_FP32] - ref).max() <= 2e-6
+
+
+def test_silu_f32():
+    torch_cuda()
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    build = os.path.join(HERE, "_build")
+    os.makedirs(build, exist_ok=True)
+    so = os.path.join(build, "libsilu_f32.so")
+    subprocess.check_call([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-std=c++17", "-shared",
+                           "-Xcompiler", "-fPIC", "-o", so, os.path.join(HERE, "silu_f32_eval.cu")])
+    L = ctypes.CDLL(so)
+    L.silu_f32_eval.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
+    z = np.concatenate([np.linspace(-110.0, 110.0, 2_000_001), np.geomspace(1e-30, 1e30, 200_001),
+                        -np.geomspace(1e-30, 87.0, 200_001), [0.0, -1e4, -1e30, np.nan]]).astype(np.float32)
+    out = np.empty_like(z)
+    assert L.silu_f32_eval(z.ctypes.data, z.size, out.ctypes.data) == 0
+    z64 = z.astype(np.float64)
+    with np.errstate(over="ignore", invalid="ignore"):
+        exact = z64 / (1.0 + np.exp(-z64))
+    inner = z64 > -87.0
+    nz = inner & (exact != 0.0) & (np.abs(exact) > 1e-30)
+    rel = np.abs(out[nz] / exact[nz] - 1.0)
+    print("silu2_f32: max relative error", rel.max(), "mean", rel.mean())
+    assert rel.max() <= 5e-7
+    low = z64 <= -87.0
+    assert np.all(np.abs(out[low] - exact[low])[z64[low] > -1e20] <= 1e-30)
+    assert np.isnan(out[-1]) and out[-4] == 0.0
