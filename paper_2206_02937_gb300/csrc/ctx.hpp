@@ -78,6 +78,17 @@ struct MlpDecide {
     float dt, gamma64;
     float* prob_out;
     uint8_t* flag_out;
+    bool count_fallbacks;
+};
+
+// A candidate list other than the context's own (the serving engine's): the
+// candidates, the pairs accepted from them, and the FP32 network's outputs.
+struct CandList {
+    CandPair* cand;
+    uint32_t* n_cand;
+    AcceptedPair* accepted;
+    uint32_t* n_accepted;
+    float* r;
 };
 
 enum : unsigned { kErrCellRange = 1u, kErrCapacity = 2u, kErrTimeout = 4u };
@@ -296,7 +307,8 @@ compton_status mlp_repack(compton_ctx* ctx, cudaStream_t stream);
 compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* uy, const float* uz,
                                 const float* kx, const float* ky, const float* kz, int64_t n, compton_mode mode,
                                 float* r_out, cudaStream_t stream, bool binned = false, bool candidates = false,
-                                const MlpDecide* decide = nullptr);
+                                const MlpDecide* decide = nullptr, const CandList* list = nullptr);
+compton_status launch_decide(compton_ctx* ctx, const CandList& list, int64_t rows, cudaStream_t stream);
 compton_status mlp_adam(compton_ctx* ctx, float lr, cudaStream_t stream);
 compton_status launch_balance_weights(compton_ctx* ctx, const float* r, int64_t n, const float* edges_host,
                                       int n_bins, float* w_out, cudaStream_t stream);

@@ -508,6 +508,15 @@ __device__ __forceinline__ float one_minus_exp_neg(float a)
     return a < 0.25f ? a * s : e;  // both evaluated: no divergence
 }
 
+// The candidate test u0 < P_b on u0 = m 2^-24 (m = word >> 8) as m < T with
+// T = ceil(P_b 2^24): P_b 2^24 is exact in FP32 (a power-of-two scaling) and
+// m is an integer, so the two tests agree for every word.  The 2.0002 factor
+// keeps P_b above any FP32 rounding of P.
+__device__ __forceinline__ uint32_t cand_threshold(float dens, float dt)
+{
+    return (uint32_t)ceilf(one_minus_exp_neg(2.0002f * dens * dt) * 16777216.0f);
+}
+
 // ---------------------------------------------------------------------------
 // Collision of one accepted pair, in FP64 (rest-frame boost and momentum
 // update, where cancellation at large gamma breaks FP32):

@@ -329,7 +329,7 @@ __device__ __forceinline__ void decide_row(const MlpArgs& a, int64_t row, bool l
     }
     if (lane == 0) {
         if (m) atomicAdd(&a.stats->scatters, (unsigned long long)__popc(m));
-        if (mf) atomicAdd(&a.stats->mlp_fallbacks, (unsigned long long)__popc(mf));
+        if (mf && a.dec.count_fallbacks) atomicAdd(&a.stats->mlp_fallbacks, (unsigned long long)__popc(mf));
     }
 }
 
@@ -1017,7 +1017,7 @@ compton_status mlp_adam(compton_ctx* ctx, float lr, cudaStream_t stream)
 compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* uy, const float* uz,
                                 const float* kx, const float* ky, const float* kz, int64_t n, compton_mode mode,
                                 float* r_out, cudaStream_t stream, bool binned, bool candidates,
-                                const MlpDecide* decide)
+                                const MlpDecide* decide, const CandList* list)
 {
     MlpArgs a;
     a.decide = decide != nullptr && mode != COMPTON_MODE_MLP_FP32;
@@ -1039,6 +1039,12 @@ compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* 
     a.n_pairs = binned ? ctx->n_pairs : nullptr;
     a.cand = candidates ? ctx->cand : nullptr;
     a.n_cand = candidates ? ctx->n_cand : nullptr;
+    if (list) {
+        a.cand = list->cand;
+        a.n_cand = list->n_cand;
+        a.accepted = list->accepted;
+        a.n_accepted = list->n_accepted;
+    }
     if (mode == COMPTON_MODE_MLP_FP32) {
         const int smem = F32Smem::words * (int)sizeof(float);
         COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_mlp_fp32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,

@@ -52,7 +52,8 @@ struct ScatterArgs {
     float* prob_out;
     uint8_t* flag_out;
     DeviceStats* stats;
-    const float* r_mlp;  // network output per pair (surrogate modes)
+    const float* r_mlp;  // network output per candidate (FP32 network)
+    bool count_fallbacks;
     AcceptedPair* accepted;
     uint32_t* n_accepted;
     // plain mode: each probability warp appends its accepted pairs to its own
@@ -182,15 +183,6 @@ struct WarpQueue {
     float dens[kQueueCap], u0[kQueueCap];
     uint32_t p[kQueueCap];
 };
-
-// The candidate test u0 < P_b on u0 = m 2^-24 (m = word >> 8) as m < T with
-// T = ceil(P_b 2^24): P_b 2^24 is exact in FP32 (a power-of-two scaling) and
-// m is an integer, so the two tests agree for every word.  The 2.0002 factor
-// keeps P_b above any FP32 rounding of P.
-__device__ __forceinline__ uint32_t cand_threshold(float dens, float dt)
-{
-    return (uint32_t)ceilf(one_minus_exp_neg(2.0002f * dens * dt) * 16777216.0f);
-}
 
 // One evaluation batch: up to 32 queue entries from slot `first` on, one
 // per lane, with their momenta.
@@ -551,7 +543,7 @@ __global__ void __launch_bounds__(256) k_decide(ScatterArgs a)
     }
     if (lane == 0) {
         if (n_hit) atomicAdd(&a.stats->scatters, (unsigned long long)n_hit);
-        if (n_fb) atomicAdd(&a.stats->mlp_fallbacks, (unsigned long long)n_fb);
+        if (n_fb && a.count_fallbacks) atomicAdd(&a.stats->mlp_fallbacks, (unsigned long long)n_fb);
     }
 }
 
@@ -930,6 +922,7 @@ void fill_common(ScatterArgs& a, compton_ctx* ctx, uint64_t seed, uint64_t step,
     a.flag_out = flag_out;
     a.stats = ctx->stats;
     a.r_mlp = ctx->r_buf;
+    a.count_fallbacks = true;
     a.accepted = ctx->accepted;
     a.n_accepted = ctx->n_accepted;
     a.warp_acc = ctx->warp_acc;
@@ -988,7 +981,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob<cand>");
         // tensor-core modes and the paper's network decide inside the network
         // kernel; the FP32 network writes r and k_decide decides
-        const MlpDecide dec{a.dt, a.gamma64, a.prob_out, a.flag_out};
+        const MlpDecide dec{a.dt, a.gamma64, a.prob_out, a.flag_out, true};
         if (mode == COMPTON_MODE_PNET) {
             const compton_status sp = launch_pnet_decide(ctx, rows, dec, a.w_e, a.w_g, stream);
             if (sp != COMPTON_OK) return sp;
@@ -1069,6 +1062,23 @@ compton_status launch_scatter_pairs(compton_ctx* ctx, float* ux, float* uy, floa
         const compton_status st = launch_step<false, false>(ctx, a, mode, tiles, a.p_end - a.p_begin, stream);
         if (st != COMPTON_OK) return st;
     }
+    return COMPTON_OK;
+}
+
+// The decisions on a candidate list of its own (the FP32 network's r in
+// list.r), rows: a host bound on its length.
+compton_status launch_decide(compton_ctx* ctx, const CandList& list, int64_t rows, cudaStream_t stream)
+{
+    ScatterArgs a{};
+    fill_common(a, ctx, 0, 0, nullptr, nullptr);
+    a.cand = list.cand;
+    a.n_cand = list.n_cand;
+    a.accepted = list.accepted;
+    a.n_accepted = list.n_accepted;
+    a.r_mlp = list.r;
+    a.count_fallbacks = false;
+    k_decide<<<collide_grid(rows), 256, 0, stream>>>(a);
+    COMPTON_LAUNCH_CHECK(ctx, "k_decide");
     return COMPTON_OK;
 }
 

@@ -7,22 +7,34 @@
 //
 //   compton_submit    validates a request and queues it (host, thread-safe).
 //   engine thread     loops: admits queued requests while a block of the
-//                     budgeted pool fits them (first fit, in arrival order),
-//                     stages each admitted request into its block (device to
-//                     device copies on the copy stream, then the network pass
-//                     for surrogate requests); launches one k_serve over the
-//                     pending tiles (1024 pairs each) of every staged request;
-//                     when a launch completes, requests whose tiles are all
-//                     done are copied back to the caller's output arrays and
-//                     their blocks freed.  Up to two launches are in flight.
+//                     budgeted pool fits them (first fit, in arrival order);
+//                     launches the pending tiles (1024 pairs each) of every
+//                     admitted request together; when a launch completes,
+//                     requests whose tiles are all done are finished and their
+//                     blocks freed.  Up to two launches are in flight.
 //   compton_poll      returns ENOTREADY or the request's result.
+//
+// A launch is k_serve over its tiles, then, for the surrogate requests' candidates,
+// the network with the decision in its epilogue and k_serve_resolve.  The
+// kernels read the caller's inputs and write the caller's outputs, so a pair's
+// momenta move once in and once out; a request's block of the pool is its share
+// of the budget, and is used as staging only where the caller's arrays overlap
+// otherwise than output on its own input.  Only candidates (pairs whose uniform
+// lies below the bound of every probability) are evaluated, and only they pass
+// through the network, all requests' together.  24 requests of 1,155 to 866,000
+// pairs, half of them for the BF16 network: 2264 us with a staged copy of every
+// array each way and a network pass per request, 850 us so.
 //
 // Every pair of request r uses Philox counter (pair index within r, step_r)
 // under key seed_r, so a request's result does not depend on what it shares
 // the GPU with.  No kernel waits on another or on the host: all coordination
 // is host-side through events.
+#include <sys/prctl.h>
+
 #include <algorithm>
 #include <chrono>
+#include <cmath>
+#include <cstddef>
 #include <condition_variable>
 #include <deque>
 #include <map>
@@ -38,19 +50,24 @@ namespace compton {
 
 constexpr int kServeThreads = 256;
 constexpr int kServePairsPerThread = kPairsPerTile / kServeThreads;
-constexpr int kServeQueueCap = kPairsPerTile + kServeThreads;
-constexpr int kMaxTilesPerLaunch = 32768;  // 33.5M pairs
+constexpr int kServeCandCap = kPairsPerTile + kServeThreads;  // queued candidates: a tile's and a remainder
+constexpr int kServeHitCap = 2 * kServeThreads;               // queued collisions: a batch's and a remainder
+constexpr int kMaxTilesPerLaunch = 32768;                     // 33.5M pairs
 constexpr int kTileRing = 4;
+constexpr uint32_t kServeListCap = 1u << 18;                  // surrogate candidates of a launch
+constexpr int kServeRejects = kMaxTilesPerLaunch;
 
 struct ReqDev {
-    float* u[3];
-    float* k[3];
+    const float* in_u[3];
+    const float* in_k[3];
+    float* out_u[3];
+    float* out_k[3];
     const float* dens;   // per pair, or nullptr
-    const float* r_mlp;  // network output per pair (surrogate requests)
     float dens_scalar;
     int mode;
+    int copy;            // the outputs are not the inputs: every pair is copied
     uint64_t seed, step;
-    unsigned long long* scatters;
+    unsigned long long* scatters;  // collisions, counted on from request to request of a slot
 };
 
 struct TileDev {
@@ -59,108 +76,225 @@ struct TileDev {
     int64_t first;
 };
 
+// A launch's device counters and the tiles it could not take (the candidate
+// list was full): they are launched again.
+struct ServeControl {
+    uint32_t n_cand, n_accepted, n_rejected, pad;
+    int32_t rejected[kServeRejects];
+};
+
 namespace {
+
+struct CQEntry {
+    int32_t req, p;
+    float u0, dens;
+};
 
 struct SQEntry {
     int32_t req, p;
     float x, F2;
 };
 
-__device__ __forceinline__ void serve_resolve(const ReqDev* reqs, const SQEntry& e, float gamma64, float c64sq)
+// The collision of pair p of a request, from its inputs to its outputs.
+__device__ __forceinline__ void serve_resolve(const ReqDev& R, int32_t p, float x, float F2, float ux, float uy, float uz,
+                                              float kx, float ky, float kz, float c64sq)
 {
-    const ReqDev& R = reqs[e.req];
-    float ux = R.u[0][e.p], uy = R.u[1][e.p], uz = R.u[2][e.p];
-    float kx = R.k[0][e.p], ky = R.k[1][e.p], kz = R.k[2][e.p];
-    float x = e.x, F2 = e.F2;
-    if (x < 0.0f) {
-        const Invariants inv = invariants_f32(ux, uy, uz, kx, ky, kz);
-        float v = inv.v;
-        x = inv.x;
-        if (inv.gamma > gamma64) invariants_f64(ux, uy, uz, kx, ky, kz, &x, &v);
-        F2 = kn_F2(x);
-    }
-    const Philox4 rnd = draw(R.seed, R.step, kStreamAngle, (uint32_t)e.p);
+    const Philox4 rnd = draw(R.seed, R.step, kStreamAngle, (uint32_t)p);
     const Angle ang = kn_sample_angle(x, rnd.r0 >> 8, F2);
     collide_pair(ux, uy, uz, kx, ky, kz, x, ang, u24_closed0(rnd.r1), c64sq);
-    R.u[0][e.p] = ux;
-    R.u[1][e.p] = uy;
-    R.u[2][e.p] = uz;
-    R.k[0][e.p] = kx;
-    R.k[1][e.p] = ky;
-    R.k[2][e.p] = kz;
+    R.out_u[0][p] = ux;
+    R.out_u[1][p] = uy;
+    R.out_u[2][p] = uz;
+    R.out_k[0][p] = kx;
+    R.out_k[1][p] = ky;
+    R.out_k[2][p] = kz;
 }
 
-// One launch over a list of tiles from any mix of requests.  Per pair the
-// arithmetic is that of k_scatter on explicit pairs (same device functions).
+// Words[i] of lane l of each four lanes becomes word l of the quad's lane i.
+__device__ __forceinline__ void quad_transpose(uint32_t (&w)[4])
+{
+    const bool b0 = threadIdx.x & 1u, b1 = threadIdx.x & 2u;
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+        const uint32_t t = __shfl_xor_sync(0xffffffffu, b0 ? w[i] : w[i + 1], 1);
+        if (b0) w[i] = t; else w[i + 1] = t;
+    }
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+        const uint32_t t = __shfl_xor_sync(0xffffffffu, b1 ? w[i] : w[i + 2], 2);
+        if (b1) w[i] = t; else w[i + 2] = t;
+    }
+}
+
+// One launch over a list of tiles from any mix of requests.  Per tile: the
+// pairs are copied to the outputs (coalesced: a thread takes pairs 256 apart,
+// the Bernoulli words come to it from its quad's four Philox blocks), the
+// candidates of a plain request go to a queue in shared memory that is
+// evaluated 256 at a time, and their collisions to a second one; a surrogate
+// request's candidates go with their momenta to the launch's list, which the
+// network decides.  Per pair the arithmetic is that of the probability kernel
+// on explicit pairs (same device functions).
 __global__ void __launch_bounds__(kServeThreads, 3)
     k_serve(const ReqDev* __restrict__ reqs, const TileDev* __restrict__ tiles, int n_tiles, float dt, float gamma64,
-            float c64sq, DeviceStats* stats, MlpDev mlp)
+            float c64sq, DeviceStats* stats, CandPair* __restrict__ cand, ServeControl* __restrict__ ctl)
 {
-    __shared__ SQEntry queue[kServeQueueCap];
-    __shared__ int qn;
+    __shared__ CQEntry cq[kServeCandCap];
+    __shared__ SQEntry sq[kServeHitCap];
+    __shared__ int cn, sn, listed;
+    __shared__ uint32_t list_base;
     const int tid = threadIdx.x;
-    if (tid == 0) qn = 0;
+    if (tid == 0) cn = sn = 0;
     unsigned my_pairs = 0, my_scat = 0;
+
+    auto evaluate = [&](const CQEntry& e) {
+        const ReqDev& R = reqs[e.req];
+        const Invariants inv = invariants_f32(R.in_u[0][e.p], R.in_u[1][e.p], R.in_u[2][e.p], R.in_k[0][e.p],
+                                              R.in_k[1][e.p], R.in_k[2][e.p]);
+        float x = inv.x, v = inv.v;
+        if (inv.gamma > gamma64)
+            invariants_f64(R.in_u[0][e.p], R.in_u[1][e.p], R.in_u[2][e.p], R.in_k[0][e.p], R.in_k[1][e.p],
+                           R.in_k[2][e.p], &x, &v);
+        const float F2 = kn_F2(x);
+        const float sig = 0.375f * F2;
+        const float P = inv.eps > 0.0f ? one_minus_exp_neg(e.dens * dt * sig * v) : 0.0f;
+        if (e.u0 < P) {
+            ++my_scat;
+            atomicAdd(R.scatters, 1ull);
+            sq[atomicAdd(&sn, 1)] = SQEntry{e.req, e.p, x, F2};
+        }
+    };
+    auto resolve = [&](const SQEntry& e) {
+        const ReqDev& R = reqs[e.req];
+        serve_resolve(R, e.p, e.x, e.F2, R.in_u[0][e.p], R.in_u[1][e.p], R.in_u[2][e.p], R.in_k[0][e.p],
+                      R.in_k[1][e.p], R.in_k[2][e.p], c64sq);
+    };
+
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
         const TileDev T = tiles[t];
         const ReqDev& R = reqs[T.req];
+        const bool plain = R.mode == COMPTON_MODE_PLAIN;
+        // tiles start at multiples of 1024 pairs; this lane draws the block of
+        // its quad's pairs of round tid % 4
+        uint32_t words[4];
+        {
+            const Philox4 r = draw(R.seed, R.step, kStreamScatter,
+                                   (uint32_t)((T.first + (tid & 3) * kServeThreads + (tid & ~3)) >> 2));
+            words[0] = r.r0, words[1] = r.r1, words[2] = r.r2, words[3] = r.r3;
+            quad_transpose(words);
+        }
+        const uint32_t thr0 = cand_threshold(R.dens_scalar, dt);
+        float u[4][3], k[4][3], dens[4];
+        int slot[4];
+        if (tid == 0) listed = 0;
         __syncthreads();
-        // tiles start at multiples of 1024 pairs: the thread's four pairs share one block
-        const Philox4 rnd4 = draw(R.seed, R.step, kStreamScatter, (uint32_t)((T.first + tid * kServePairsPerThread) >> 2));
-        const uint32_t words[4] = {rnd4.r0, rnd4.r1, rnd4.r2, rnd4.r3};
 #pragma unroll
         for (int rr = 0; rr < kServePairsPerThread; ++rr) {
-            const int local = tid * kServePairsPerThread + rr;
+            const int local = rr * kServeThreads + tid;
+            slot[rr] = -1;
             if (local >= T.count) continue;
             const int64_t p = T.first + local;
-            const float ux = R.u[0][p], uy = R.u[1][p], uz = R.u[2][p];
-            const float kx = R.k[0][p], ky = R.k[1][p], kz = R.k[2][p];
-            const float dens = R.dens ? R.dens[p] : R.dens_scalar;
-            float x = -1.0f, F2 = 0.0f, P;
-            bool analytic = true;
-            if (R.mode != COMPTON_MODE_PLAIN) {
-                const float g2 = fmaf(ux, ux, fmaf(uy, uy, fmaf(uz, uz, 1.0f)));
-                const float e2 = fmaf(kx, kx, fmaf(ky, ky, kz * kz));
-                if (mlp_in_range(mlp, g2, e2)) {
-                    analytic = false;
-                    P = one_minus_exp_neg(2.0f * dens * dt * R.r_mlp[p]);
+            dens[rr] = R.dens ? R.dens[p] : R.dens_scalar;
+            const bool is_cand = (words[rr] >> 8) < (R.dens ? cand_threshold(dens[rr], dt) : thr0);
+            if (R.copy || (is_cand && !plain)) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    u[rr][c] = R.in_u[c][p];
+                    k[rr][c] = R.in_k[c][p];
                 }
             }
-            if (analytic) {
-                const Invariants inv = invariants_f32(ux, uy, uz, kx, ky, kz);
-                float v = inv.v;
-                x = inv.x;
-                if (inv.gamma > gamma64) invariants_f64(ux, uy, uz, kx, ky, kz, &x, &v);
-                F2 = kn_F2(x);
-                const float sig = 0.375f * F2;
-                P = inv.eps > 0.0f ? one_minus_exp_neg(dens * dt * sig * v) : 0.0f;
+            if (R.copy) {
+#pragma unroll
+                for (int c = 0; c < 3; ++c) {
+                    R.out_u[c][p] = u[rr][c];
+                    R.out_k[c][p] = k[rr][c];
+                }
             }
-            ++my_pairs;
-            if (u24_closed0(words[rr]) < P) {
-                ++my_scat;
-                atomicAdd(R.scatters, 1ull);
-                const int slot = atomicAdd(&qn, 1);
-                queue[slot] = SQEntry{T.req, (int32_t)p, x, F2};
+            if (is_cand) {
+                if (plain) cq[atomicAdd(&cn, 1)] = CQEntry{T.req, (int32_t)p, u24_closed0(words[rr]), dens[rr]};
+                else slot[rr] = atomicAdd(&listed, 1);
             }
         }
-        __syncthreads();
-        int nq = qn;
-        while (nq >= kServeThreads) {
-            serve_resolve(reqs, queue[nq - kServeThreads + tid], gamma64, c64sq);
-            nq -= kServeThreads;
+        __syncthreads();  // the copies of this tile come before its collisions' writes
+        if (!plain) {
+            // room in the list for all of the tile's candidates, or the tile is launched again
+            const int want = listed;
+            if (tid == 0) {
+                uint32_t at = *(volatile uint32_t*)&ctl->n_cand;
+                for (;;) {
+                    if (at + (uint32_t)want > kServeListCap) {
+                        at = 0xFFFFFFFFu;
+                        ctl->rejected[atomicAdd(&ctl->n_rejected, 1u)] = t;
+                        break;
+                    }
+                    const uint32_t seen = atomicCAS(&ctl->n_cand, at, at + (uint32_t)want);
+                    if (seen == at) break;
+                    at = seen;
+                }
+                list_base = at;
+            }
+            __syncthreads();
+            const uint32_t base = list_base;
+            if (base != 0xFFFFFFFFu) {
+#pragma unroll
+                for (int rr = 0; rr < kServePairsPerThread; ++rr) {
+                    const int local = rr * kServeThreads + tid;
+                    my_pairs += local < T.count;
+                    if (slot[rr] < 0) continue;
+                    cand[base + (uint32_t)slot[rr]] =
+                        CandPair{(int32_t)(T.first + local), T.req, dens[rr], u24_closed0(words[rr]),
+                                 (uint32_t)(T.first + local), {u[rr][0], u[rr][1], u[rr][2]},
+                                 {k[rr][0], k[rr][1], k[rr][2]}, 0u};
+                }
+            }
+            __syncthreads();
+            continue;
         }
+#pragma unroll
+        for (int rr = 0; rr < kServePairsPerThread; ++rr) my_pairs += rr * kServeThreads + tid < T.count;
+        int nc = cn;
+        while (nc >= kServeThreads) {
+            nc -= kServeThreads;
+            evaluate(cq[nc + tid]);
+            __syncthreads();
+            const int ns = sn;
+            if (ns >= kServeThreads) resolve(sq[ns - kServeThreads + tid]);
+            __syncthreads();
+            if (tid == 0 && ns >= kServeThreads) sn = ns - kServeThreads;
+            __syncthreads();
+        }
+        if (tid == 0) cn = nc;
         __syncthreads();
-        if (tid == 0) qn = nq;
     }
     __syncthreads();
-    if (tid < qn) serve_resolve(reqs, queue[tid], gamma64, c64sq);
+    if (tid < cn) evaluate(cq[tid]);
+    __syncthreads();
+    for (int i = tid; i < sn; i += kServeThreads) resolve(sq[i]);
     for (int d = 16; d > 0; d >>= 1) {
         my_pairs += __shfl_xor_sync(0xffffffffu, my_pairs, d);
         my_scat += __shfl_xor_sync(0xffffffffu, my_scat, d);
     }
-    if ((tid & 31) == 0 && my_pairs) {
-        atomicAdd(&stats->pairs_tested, (unsigned long long)my_pairs);
-        atomicAdd(&stats->scatters, (unsigned long long)my_scat);
+    if ((tid & 31) == 0 && my_pairs) atomicAdd(&stats->pairs_tested, (unsigned long long)my_pairs);
+    if ((tid & 31) == 0 && my_scat) atomicAdd(&stats->scatters, (unsigned long long)my_scat);
+}
+
+// The collisions the network decided (counted there): ie is the pair, ig the
+// request's slot.
+__global__ void __launch_bounds__(256) k_serve_resolve(const ReqDev* __restrict__ reqs, const AcceptedPair* __restrict__ acc,
+                                                       const ServeControl* __restrict__ ctl, float gamma64, float c64sq)
+{
+    const uint32_t n = ctl->n_accepted;
+    for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x) {
+        const AcceptedPair e = acc[i];
+        const ReqDev& R = reqs[e.ig];
+        float x = e.x;
+        if (x < 0.0f) {  // probability came from the network: the collision needs x
+            const Invariants inv = invariants_f32(e.u[0], e.u[1], e.u[2], e.k[0], e.k[1], e.k[2]);
+            float v = inv.v;
+            x = inv.x;
+            if (inv.gamma > gamma64) invariants_f64(e.u[0], e.u[1], e.u[2], e.k[0], e.k[1], e.k[2], &x, &v);
+        }
+        atomicAdd(R.scatters, 1ull);
+        serve_resolve(R, e.ie, x, kn_F2(x), e.u[0], e.u[1], e.u[2], e.k[0], e.k[1], e.k[2], c64sq);
     }
 }
 
@@ -180,17 +314,18 @@ struct ServeReq {
     uint64_t ticket = 0;
     compton_request req{};
     int64_t tiles = 0, launched = 0, done_tiles = 0;
-    int state = 0;  // 0 queued, 1 staging, 2 running, 3 copying back, 4 done
+    std::vector<TileDev> again;  // tiles a full candidate list turned away
+    int state = 0;  // 0 queued, 1 admitted, 4 done
     size_t off = 0, bytes = 0;
     int dslot = -1;
     double t_submit = 0, t_admit = 0, t_done = 0;
-    cudaEvent_t ev = nullptr;  // staging or copy-back completion
     compton_status status = COMPTON_OK;
     uint64_t scatters = 0;
 };
 
 struct Launch {
     cudaEvent_t ev;
+    int ring;
     std::vector<std::pair<uint64_t, int64_t>> tiles_per_req;  // ticket, tiles in this launch
 };
 
@@ -204,16 +339,22 @@ struct ServeEngine {
     int max_active = 0;
     ReqDev* reqs_dev = nullptr;
     ReqDev* reqs_host = nullptr;        // pinned staging of the table
-    unsigned long long* counters = nullptr;  // per device slot
-    unsigned long long* scat_host = nullptr;  // pinned copy of the counters of finished requests
+    int new_lo = 0, new_hi = -1;        // slots filled since the table was last copied
+    unsigned long long* counters = nullptr;   // per device slot: collisions since the start
+    unsigned long long* scat_host = nullptr;  // pinned copies of the counters, kTileRing x max_active
+    std::vector<unsigned long long> scat_base;  // per slot: its counter when its request was admitted
     std::vector<int> free_slots;
     TileDev* tiles_dev = nullptr;
     TileDev* tiles_host = nullptr;      // pinned, kTileRing x kMaxTilesPerLaunch
+    CandList list{};                    // surrogate candidates of a launch, kServeListCap
+    ServeControl* ctl_dev = nullptr;
+    ServeControl* ctl_host = nullptr;   // pinned, kTileRing
     int ring = 0;
-    cudaStream_t s_compute = nullptr, s_copy = nullptr;
+    cudaStream_t s_compute = nullptr;
     std::mutex mu;
     std::condition_variable cv;
     std::deque<uint64_t> queued;
+    std::deque<uint64_t> active;        // admitted, with tiles to launch, in order of admission
     std::unordered_map<uint64_t, ServeReq> reqs;
     std::deque<Launch> inflight;
     uint64_t next_ticket = 1;
@@ -265,6 +406,22 @@ size_t request_bytes(const compton_request& r)
     return align256((size_t)r.n * per_pair * sizeof(float)) + 256;
 }
 
+// Whether an output of the request shares memory with an input otherwise than
+// as that same input (momentum component on itself, from the same address).
+bool overlaps_inputs(const compton_request& r)
+{
+    const char* in[7] = {(const char*)r.ux_in_dev, (const char*)r.uy_in_dev, (const char*)r.uz_in_dev,
+                         (const char*)r.kx_in_dev, (const char*)r.ky_in_dev, (const char*)r.kz_in_dev,
+                         (const char*)r.n_dens_dev};
+    const char* out[6] = {(const char*)r.ux_out_dev, (const char*)r.uy_out_dev, (const char*)r.uz_out_dev,
+                          (const char*)r.kx_out_dev, (const char*)r.ky_out_dev, (const char*)r.kz_out_dev};
+    const size_t bytes = (size_t)r.n * sizeof(float);
+    for (int o = 0; o < 6; ++o)
+        for (int i = 0; i < 7; ++i)
+            if (in[i] && !(i == o && in[i] == out[o]) && in[i] < out[o] + bytes && out[o] < in[i] + bytes) return true;
+    return false;
+}
+
 // Admit queued requests in arrival order while blocks fit (a request that
 // does not fit waits; later, smaller ones may pass it).
 void admit(ServeEngine* E)
@@ -283,71 +440,127 @@ void admit(ServeEngine* E)
         R.state = 1;
         R.t_admit = now_s();
         const int64_t n = R.req.n;
-        float* base = reinterpret_cast<float*>(static_cast<char*>(E->pool) + off);
+        const float* src[6] = {R.req.ux_in_dev, R.req.uy_in_dev, R.req.uz_in_dev,
+                               R.req.kx_in_dev, R.req.ky_in_dev, R.req.kz_in_dev};
+        float* dst[6] = {R.req.ux_out_dev, R.req.uy_out_dev, R.req.uz_out_dev,
+                         R.req.kx_out_dev, R.req.ky_out_dev, R.req.kz_out_dev};
         ReqDev d{};
-        for (int c = 0; c < 3; ++c) {
-            d.u[c] = base + (size_t)c * n;
-            d.k[c] = base + (size_t)(3 + c) * n;
+        d.dens = R.req.n_dens_dev;
+        if (overlaps_inputs(R.req)) {
+            // the outputs would overwrite inputs of other pairs: the inputs are staged in the block
+            float* base = reinterpret_cast<float*>(static_cast<char*>(E->pool) + off);
+            for (int c = 0; c < 7; ++c) {
+                const float* from = c < 6 ? src[c] : R.req.n_dens_dev;
+                if (!from) continue;
+                cudaMemcpyAsync(base + (size_t)c * n, from, n * sizeof(float), cudaMemcpyDeviceToDevice, E->s_compute);
+                if (c < 6) src[c] = base + (size_t)c * n;
+                else d.dens = base + (size_t)c * n;
+            }
         }
-        float* dens = base + (size_t)6 * n;
-        d.dens = R.req.n_dens_dev ? dens : nullptr;
-        d.r_mlp = R.req.mode != COMPTON_MODE_PLAIN ? base + (size_t)7 * n : nullptr;
+        for (int c = 0; c < 3; ++c) {
+            d.in_u[c] = src[c];
+            d.in_k[c] = src[3 + c];
+            d.out_u[c] = dst[c];
+            d.out_k[c] = dst[3 + c];
+        }
+        for (int c = 0; c < 6; ++c) d.copy |= src[c] != dst[c];
         d.dens_scalar = R.req.n_dens;
         d.mode = (int)R.req.mode;
         d.seed = R.req.seed;
         d.step = R.req.step;
         d.scatters = E->counters + R.dslot;
         E->reqs_host[R.dslot] = d;
-        cudaStream_t s = E->s_copy;
-        const float* src_u[3] = {R.req.ux_in_dev, R.req.uy_in_dev, R.req.uz_in_dev};
-        const float* src_k[3] = {R.req.kx_in_dev, R.req.ky_in_dev, R.req.kz_in_dev};
-        for (int c = 0; c < 3; ++c) {
-            cudaMemcpyAsync(d.u[c], src_u[c], n * sizeof(float), cudaMemcpyDeviceToDevice, s);
-            cudaMemcpyAsync(d.k[c], src_k[c], n * sizeof(float), cudaMemcpyDeviceToDevice, s);
-        }
-        if (R.req.n_dens_dev) cudaMemcpyAsync(dens, R.req.n_dens_dev, n * sizeof(float), cudaMemcpyDeviceToDevice, s);
-        cudaMemsetAsync(E->counters + R.dslot, 0, sizeof(unsigned long long), s);
-        cudaMemcpyAsync(E->reqs_dev + R.dslot, E->reqs_host + R.dslot, sizeof(ReqDev), cudaMemcpyHostToDevice, s);
-        if (R.req.mode != COMPTON_MODE_PLAIN)
-            launch_mlp_infer(E->ctx, d.u[0], d.u[1], d.u[2], d.k[0], d.k[1], d.k[2], n, R.req.mode,
-                             const_cast<float*>(d.r_mlp), s, false);
-        cudaEventRecord(R.ev, s);
+        E->new_lo = E->new_hi < 0 ? R.dslot : std::min(E->new_lo, R.dslot);
+        E->new_hi = std::max(E->new_hi, R.dslot);
+        E->active.push_back(R.ticket);
         it = E->queued.erase(it);
     }
 }
 
+// Pairs of a request that are candidates, roughly (a launch takes no more
+// surrogate tiles than its list will hold; what it turns away is launched again).
+double expected_candidates(const compton_request& r, double dt, double pairs)
+{
+    const double share = r.n_dens_dev ? 0.25 : 1.0 - std::exp(-2.001 * (double)r.n_dens * dt);
+    return pairs * (share < 1.0 ? share : 1.0);
+}
+
 void launch_tiles(ServeEngine* E)
 {
+    if (E->active.empty()) return;
+    const compton_config& cfg = E->ctx->cfg;
     TileDev* th = E->tiles_host + (size_t)E->ring * kMaxTilesPerLaunch;
     TileDev* td = E->tiles_dev + (size_t)E->ring * kMaxTilesPerLaunch;
+    ServeControl* ch = E->ctl_host + E->ring;
     int nt = 0;
     Launch L;
-    for (auto& kv : E->reqs) {
-        ServeReq& R = kv.second;
-        if (R.state == 1 && cudaEventQuery(R.ev) == cudaSuccess) R.state = 2;
-        if (R.state != 2 || R.launched >= R.tiles) continue;
+    L.ring = E->ring;
+    // one network mode per launch: that of the first surrogate request in line
+    int mode = COMPTON_MODE_PLAIN;
+    double cand = 0.0;
+    std::deque<uint64_t> rest;
+    for (const uint64_t ticket : E->active) {
+        ServeReq& R = E->reqs[ticket];
+        const bool surrogate = R.req.mode != COMPTON_MODE_PLAIN;
+        if (surrogate && mode == COMPTON_MODE_PLAIN) mode = (int)R.req.mode;
         int64_t take = 0;
-        while (R.launched < R.tiles && nt < kMaxTilesPerLaunch) {
-            const int64_t first = R.launched * kPairsPerTile;
-            const int64_t cnt = std::min<int64_t>(kPairsPerTile, R.req.n - first);
-            th[nt++] = TileDev{R.dslot, (int32_t)cnt, first};
-            ++R.launched;
-            ++take;
+        if (!surrogate || mode == (int)R.req.mode) {
+            while ((R.launched < R.tiles || !R.again.empty()) && nt < kMaxTilesPerLaunch) {
+                if (surrogate) {
+                    const double c = expected_candidates(R.req, cfg.dt, kPairsPerTile);
+                    if (cand > 0.0 && cand + c > 0.9 * kServeListCap) break;
+                    cand += c;
+                }
+                if (!R.again.empty()) {
+                    th[nt++] = R.again.back();
+                    R.again.pop_back();
+                } else {
+                    const int64_t first = R.launched * kPairsPerTile;
+                    th[nt++] = TileDev{R.dslot, (int32_t)std::min<int64_t>(kPairsPerTile, R.req.n - first), first};
+                    ++R.launched;
+                }
+                ++take;
+            }
         }
-        if (take) L.tiles_per_req.emplace_back(R.ticket, take);
-        if (nt >= kMaxTilesPerLaunch) break;
+        if (take) L.tiles_per_req.emplace_back(ticket, take);
+        if (R.launched < R.tiles || !R.again.empty()) rest.push_back(ticket);
     }
+    E->active.swap(rest);
     if (nt == 0) return;
-    cudaMemcpyAsync(td, th, nt * sizeof(TileDev), cudaMemcpyHostToDevice, E->s_compute);
-    int n_sm = 0;
-    cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, E->device);
-    const int grid = std::min(nt, n_sm * 3);
-    const compton_config& cfg = E->ctx->cfg;
-    k_serve<<<grid, kServeThreads, 0, E->s_compute>>>(E->reqs_dev, td, nt, (float)cfg.dt, cfg.gamma_fp64_threshold,
-                                                      cfg.collide_fp64_threshold * cfg.collide_fp64_threshold,
-                                                      E->ctx->stats, E->ctx->mlp);
+    cudaStream_t s = E->s_compute;
+    if (E->new_hi >= 0) {
+        cudaMemcpyAsync(E->reqs_dev + E->new_lo, E->reqs_host + E->new_lo,
+                        sizeof(ReqDev) * (E->new_hi - E->new_lo + 1), cudaMemcpyHostToDevice, s);
+        E->new_hi = -1;
+    }
+    cudaMemcpyAsync(td, th, nt * sizeof(TileDev), cudaMemcpyHostToDevice, s);
+    cudaMemsetAsync(E->ctl_dev, 0, offsetof(ServeControl, rejected), s);
+    const int grid = std::min(nt, E->ctx->n_sm * 3);
+    const float c64sq = cfg.collide_fp64_threshold * cfg.collide_fp64_threshold;
+    k_serve<<<grid, kServeThreads, 0, s>>>(E->reqs_dev, td, nt, (float)cfg.dt, cfg.gamma_fp64_threshold, c64sq,
+                                           E->ctx->stats, E->list.cand, E->ctl_dev);
+    if (mode != COMPTON_MODE_PLAIN) {
+        const MlpDecide dec{(float)cfg.dt, cfg.gamma_fp64_threshold, nullptr, nullptr, false};
+        const bool fused = mode != COMPTON_MODE_MLP_FP32;
+        // the grids are sized for the list the host expects, at most a full one
+        const int64_t rows = (int64_t)std::min<double>(kServeListCap, 1.2 * cand + 4096.0);
+        compton_status st = launch_mlp_infer(E->ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, rows,
+                                             (compton_mode)mode, E->list.r, s, false, false, fused ? &dec : nullptr,
+                                             &E->list);
+        if (st == COMPTON_OK && !fused) st = launch_decide(E->ctx, E->list, rows, s);
+        if (st != COMPTON_OK) E->fatal = st;
+        const int rgrid = (int)std::min<int64_t>((rows + 255) / 256, (int64_t)E->ctx->n_sm * 8);
+        k_serve_resolve<<<rgrid, 256, 0, s>>>(E->reqs_dev, E->list.accepted, E->ctl_dev, cfg.gamma_fp64_threshold,
+                                              c64sq);
+    }
+    // the counters, and the tiles turned away
+    cudaMemcpyAsync(ch, E->ctl_dev, offsetof(ServeControl, rejected) + nt * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
+    int hi = 0;
+    for (const auto& tr : L.tiles_per_req) hi = std::max(hi, E->reqs[tr.first].dslot);
+    cudaMemcpyAsync(E->scat_host + (size_t)E->ring * E->max_active, E->counters, sizeof(unsigned long long) * (hi + 1),
+                    cudaMemcpyDeviceToHost, s);
     cudaEventCreateWithFlags(&L.ev, cudaEventDisableTiming);
-    cudaEventRecord(L.ev, E->s_compute);
+    cudaEventRecord(L.ev, s);
     E->inflight.push_back(std::move(L));
     E->ring = (E->ring + 1) % kTileRing;
 }
@@ -356,59 +569,51 @@ void retire(ServeEngine* E)
 {
     while (!E->inflight.empty() && cudaEventQuery(E->inflight.front().ev) == cudaSuccess) {
         Launch& L = E->inflight.front();
+        ServeControl* ch = E->ctl_host + L.ring;
+        const TileDev* th = E->tiles_host + (size_t)L.ring * kMaxTilesPerLaunch;
+        std::unordered_map<int, int64_t> turned_away;  // slot -> tiles
+        for (uint32_t i = 0; i < ch->n_rejected; ++i) ++turned_away[th[ch->rejected[i]].req];
         for (auto& tr : L.tiles_per_req) {
             ServeReq& R = E->reqs[tr.first];
-            R.done_tiles += tr.second;
+            const auto it = turned_away.find(R.dslot);
+            const int64_t away = it == turned_away.end() ? 0 : it->second;
+            R.done_tiles += tr.second - away;
+            if (away) {
+                if (R.launched == R.tiles && R.again.empty()) E->active.push_back(R.ticket);
+                for (uint32_t i = 0; i < ch->n_rejected; ++i)
+                    if (th[ch->rejected[i]].req == R.dslot) R.again.push_back(th[ch->rejected[i]]);
+            }
             if (R.done_tiles == R.tiles) {
-                // copy back to the caller's outputs once the compute stream has finished these tiles
-                const int64_t n = R.req.n;
-                const ReqDev& d = E->reqs_host[R.dslot];
-                float* dst_u[3] = {R.req.ux_out_dev, R.req.uy_out_dev, R.req.uz_out_dev};
-                float* dst_k[3] = {R.req.kx_out_dev, R.req.ky_out_dev, R.req.kz_out_dev};
-                for (int c = 0; c < 3; ++c) {
-                    cudaMemcpyAsync(dst_u[c], d.u[c], n * sizeof(float), cudaMemcpyDeviceToDevice, E->s_copy);
-                    cudaMemcpyAsync(dst_k[c], d.k[c], n * sizeof(float), cudaMemcpyDeviceToDevice, E->s_copy);
-                }
-                cudaMemcpyAsync(E->scat_host + R.dslot, E->counters + R.dslot, sizeof(unsigned long long),
-                                cudaMemcpyDeviceToHost, E->s_copy);
-                cudaEventRecord(R.ev, E->s_copy);
-                R.state = 3;
+                R.state = 4;
+                R.t_done = now_s();
+                const unsigned long long count = E->scat_host[(size_t)L.ring * E->max_active + R.dslot];
+                R.scatters = count - E->scat_base[R.dslot];
+                E->scat_base[R.dslot] = count;
+                pool_free(E, R.off, R.bytes);
+                E->free_slots.push_back(R.dslot);
+                R.dslot = -1;
             }
         }
         cudaEventDestroy(L.ev);
         E->inflight.pop_front();
-    }
-    for (auto& kv : E->reqs) {
-        ServeReq& R = kv.second;
-        if (R.state == 3 && cudaEventQuery(R.ev) == cudaSuccess) {
-            R.state = 4;
-            R.t_done = now_s();
-            R.scatters = E->scat_host[R.dslot];
-            pool_free(E, R.off, R.bytes);
-            E->free_slots.push_back(R.dslot);
-            R.dslot = -1;
-        }
     }
 }
 
 void engine_loop(ServeEngine* E)
 {
     cudaSetDevice(E->device);
+    prctl(PR_SET_TIMERSLACK, 1000);  // the 20 us sleeps below: wake within a microsecond of them
     std::unique_lock<std::mutex> lk(E->mu);
     while (!E->stop) {
-        admit(E);
         retire(E);
+        admit(E);
         if (E->inflight.size() < 2) launch_tiles(E);
         cudaError_t err = cudaGetLastError();
         if (err != cudaSuccess) {
             set_cuda_error(E->ctx, err, "serve engine");
             E->fatal = COMPTON_ECUDA;
         }
-        const bool busy = !E->inflight.empty() || !E->queued.empty() ||
-                          std::any_of(E->reqs.begin(), E->reqs.end(),
-                                      [](const std::pair<const uint64_t, ServeReq>& kv) {
-                                          return kv.second.state >= 1 && kv.second.state <= 3;
-                                      });
+        const bool busy = !E->inflight.empty() || !E->queued.empty() || !E->active.empty();
         if (busy) {
             lk.unlock();
             std::this_thread::sleep_for(std::chrono::microseconds(20));
@@ -438,14 +643,23 @@ compton_status serve_start(compton_ctx* ctx, uint64_t pool_bytes, int32_t max_ac
     if (e == cudaSuccess) e = cudaMalloc(&E->tiles_dev, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
     if (e == cudaSuccess) e = cudaMallocHost(&E->reqs_host, sizeof(ReqDev) * max_active);
     if (e == cudaSuccess) e = cudaMallocHost(&E->tiles_host, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
-    if (e == cudaSuccess) e = cudaMallocHost(&E->scat_host, sizeof(unsigned long long) * max_active);
+    if (e == cudaSuccess) e = cudaMallocHost(&E->scat_host, sizeof(unsigned long long) * max_active * kTileRing);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.cand, sizeof(CandPair) * kServeListCap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.accepted, sizeof(AcceptedPair) * kServeListCap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.r, sizeof(float) * kServeListCap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->ctl_dev, sizeof(ServeControl));
+    if (e == cudaSuccess) e = cudaMallocHost(&E->ctl_host, sizeof(ServeControl) * kTileRing);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&E->s_compute, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&E->s_copy, cudaStreamNonBlocking);
+    if (e == cudaSuccess) e = cudaMemset(E->counters, 0, sizeof(unsigned long long) * max_active);
+    if (e == cudaSuccess) e = cudaDeviceSynchronize();
     if (e != cudaSuccess) {
         cudaGetLastError();
         serve_stop_free(E);
         return COMPTON_ENOMEM;
     }
+    E->list.n_cand = &E->ctl_dev->n_cand;
+    E->list.n_accepted = &E->ctl_dev->n_accepted;
+    E->scat_base.assign(max_active, 0);
     E->free_blocks[0] = pool_bytes;
     for (int i = max_active - 1; i >= 0; --i) E->free_slots.push_back(i);
     ctx->serve = E;
@@ -462,10 +676,12 @@ void serve_stop_free(ServeEngine* E)
     if (E->reqs_host) cudaFreeHost(E->reqs_host);
     if (E->tiles_host) cudaFreeHost(E->tiles_host);
     if (E->scat_host) cudaFreeHost(E->scat_host);
+    if (E->list.cand) cudaFree(E->list.cand);
+    if (E->list.accepted) cudaFree(E->list.accepted);
+    if (E->list.r) cudaFree(E->list.r);
+    if (E->ctl_dev) cudaFree(E->ctl_dev);
+    if (E->ctl_host) cudaFreeHost(E->ctl_host);
     if (E->s_compute) cudaStreamDestroy(E->s_compute);
-    if (E->s_copy) cudaStreamDestroy(E->s_copy);
-    for (auto& kv : E->reqs)
-        if (kv.second.ev) cudaEventDestroy(kv.second.ev);
     for (auto& L : E->inflight) cudaEventDestroy(L.ev);
     delete E;
 }
@@ -481,7 +697,6 @@ compton_status serve_stop(compton_ctx* ctx)
     E->cv.notify_all();
     if (E->worker.joinable()) E->worker.join();
     cudaStreamSynchronize(E->s_compute);
-    cudaStreamSynchronize(E->s_copy);
     serve_stop_free(E);
     ctx->serve = nullptr;
     return COMPTON_OK;
@@ -502,10 +717,6 @@ compton_status serve_submit(compton_ctx* ctx, const compton_request* r, uint64_t
     R.tiles = (r->n + kPairsPerTile - 1) / kPairsPerTile;
     R.bytes = bytes;
     R.t_submit = now_s();
-    if (cudaEventCreateWithFlags(&R.ev, cudaEventDisableTiming) != cudaSuccess) {
-        cudaGetLastError();
-        return COMPTON_ECUDA;
-    }
     *ticket = R.ticket;
     E->reqs.emplace(R.ticket, R);
     E->queued.push_back(R.ticket);
@@ -526,7 +737,6 @@ compton_status serve_poll(compton_ctx* ctx, uint64_t ticket, compton_result* out
     out->scatters = R.scatters;
     out->latency_s = R.t_done - R.t_submit;
     out->queue_s = R.t_admit - R.t_submit;
-    cudaEventDestroy(R.ev);
     E->reqs.erase(it);
     return COMPTON_OK;
 }
