@@ -23,7 +23,7 @@
 // lies below the bound of every probability) are evaluated, and only they pass
 // through the network, all requests' together.  24 requests of 1,155 to 866,000
 // pairs, half of them for the BF16 network: 2264 us with a staged copy of every
-// array each way and a network pass per request, 850 us so.
+// array each way and a network pass per request, 430 us so.
 //
 // Every pair of request r uses Philox counter (pair index within r, step_r)
 // under key seed_r, so a request's result does not depend on what it shares
@@ -79,7 +79,8 @@ struct TileDev {
 // A launch's device counters and the tiles it could not take (the candidate
 // list was full): they are launched again.
 struct ServeControl {
-    uint32_t n_cand, n_accepted, n_rejected, pad;
+    uint32_t n_cand, n_accepted, n_rejected;
+    uint32_t n_reserved;  // candidates of all tiles, those turned away too
     int32_t rejected[kServeRejects];
 };
 
@@ -94,6 +95,15 @@ struct SQEntry {
     int32_t req, p;
     float x, F2;
 };
+
+// One more collision of request req for every thread that is here: one atomic
+// per request and warp.
+__device__ __forceinline__ void count_hit(const ReqDev* reqs, int32_t req)
+{
+    const unsigned peers = __match_any_sync(__activemask(), req);
+    if ((int)(threadIdx.x & 31u) == __ffs(peers) - 1)
+        atomicAdd(reqs[req].scatters, (unsigned long long)__popc(peers));
+}
 
 // The collision of pair p of a request, from its inputs to its outputs.
 __device__ __forceinline__ void serve_resolve(const ReqDev& R, int32_t p, float x, float F2, float ux, float uy, float uz,
@@ -159,7 +169,7 @@ __global__ void __launch_bounds__(kServeThreads, 3)
         const float P = inv.eps > 0.0f ? one_minus_exp_neg(e.dens * dt * sig * v) : 0.0f;
         if (e.u0 < P) {
             ++my_scat;
-            atomicAdd(R.scatters, 1ull);
+            count_hit(reqs, e.req);
             sq[atomicAdd(&sn, 1)] = SQEntry{e.req, e.p, x, F2};
         }
     };
@@ -219,16 +229,13 @@ __global__ void __launch_bounds__(kServeThreads, 3)
             // room in the list for all of the tile's candidates, or the tile is launched again
             const int want = listed;
             if (tid == 0) {
-                uint32_t at = *(volatile uint32_t*)&ctl->n_cand;
-                for (;;) {
-                    if (at + (uint32_t)want > kServeListCap) {
-                        at = 0xFFFFFFFFu;
-                        ctl->rejected[atomicAdd(&ctl->n_rejected, 1u)] = t;
-                        break;
-                    }
-                    const uint32_t seen = atomicCAS(&ctl->n_cand, at, at + (uint32_t)want);
-                    if (seen == at) break;
-                    at = seen;
+                // the reservations that fit are the first ones: what they hold has no gaps
+                uint32_t at = want > 0 ? atomicAdd(&ctl->n_reserved, (uint32_t)want) : 0u;
+                if (at + (uint32_t)want > kServeListCap) {
+                    at = 0xFFFFFFFFu;
+                    ctl->rejected[atomicAdd(&ctl->n_rejected, 1u)] = t;
+                } else if (want > 0) {
+                    atomicAdd(&ctl->n_cand, (uint32_t)want);
                 }
                 list_base = at;
             }
@@ -293,7 +300,7 @@ __global__ void __launch_bounds__(256) k_serve_resolve(const ReqDev* __restrict_
             x = inv.x;
             if (inv.gamma > gamma64) invariants_f64(e.u[0], e.u[1], e.u[2], e.k[0], e.k[1], e.k[2], &x, &v);
         }
-        atomicAdd(R.scatters, 1ull);
+        count_hit(reqs, e.ig);
         serve_resolve(R, e.ie, x, kn_F2(x), e.u[0], e.u[1], e.u[2], e.k[0], e.k[1], e.k[2], c64sq);
     }
 }
