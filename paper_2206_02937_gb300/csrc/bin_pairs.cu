@@ -3,7 +3,8 @@
 // cells, in which the particles are binned; from this binning a list of
 // colliding leptons and photons is produced for each cell").
 //
-// Six launches per call, both species in each:
+// Six launches per call, both species in each (a small call: k_bin_small, which
+// does all before the sort in one, and the sort):
 //   k_count        histogram of cell indices by run boundaries, order check
 //   k_scan_reduce  per-tile sums of N_e,c, N_g,c and M_c = min(N_e,c, N_g,c)
 //   k_scan_blocks  exclusive scan of the tile sums (one CTA)
@@ -158,10 +159,11 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
 // 512^2 cells, 64 + 64 per cell, a tenth of them moved: the placement takes
 // 0.087 ms by index and 0.368 ms by record, the sort after it 0.34 ms each.
 enum SortSource : int { kInPlace = 0, kByIndex = 1, kRecords = 2 };
+constexpr uint32_t kIndexPlaced = 0xFFFFFFFFu;  // k_bin_small has placed indices, whatever the order
 __device__ __forceinline__ SortSource sort_source(uint32_t unsorted, int64_t n)
 {
     if (unsorted == 0) return kInPlace;
-    return (int64_t)unsorted * 4 < n ? kByIndex : kRecords;
+    return unsorted == kIndexPlaced || (int64_t)unsorted * 4 < n ? kByIndex : kRecords;
 }
 
 // ---------------------------------------------------------------------------
@@ -297,6 +299,42 @@ __device__ __forceinline__ void write_sort_tiles(int32_t* stile, int64_t nb, int
     for (int64_t b = b_lo; b <= b_hi; ++b) stile[b] = (int32_t)(c + 1);
 }
 
+// The maps' entries of cell c: counts ne, ng, exclusive prefixes p, np_total pairs in all.
+__device__ __forceinline__ void scan_cell(const ScanFinalArgs& a, int64_t c, int32_t ne, int32_t ng, const Tri& p,
+                                          int64_t np_total)
+{
+    const int64_t m = ne < ng ? ne : ng;
+    a.off_e[c] = (int32_t)p.e;
+    a.off_g[c] = (int32_t)p.g;
+    const int64_t nmax = ne > ng ? ne : ng;
+    CellInfo ci;
+    ci.pair_off = (int32_t)p.m;
+    ci.e_start = (int32_t)p.e;
+    ci.g_start = (int32_t)p.g;
+    ci.dens = (float)((double)nmax * a.w_over_v);
+    a.cinfo[c] = ci;
+    if (m > 0) {
+        // scatter tiles whose first pair lies in [p.m, p.m + m)
+        for (int64_t t = (p.m + kPairsPerTile - 1) / kPairsPerTile; t * kPairsPerTile < p.m + m; ++t)
+            a.tile_cell[t] = (int32_t)c;
+        if (p.m + m == np_total) a.tile_cell[(np_total + kPairsPerTile - 1) / kPairsPerTile] = (int32_t)c;
+    }
+    write_sort_tiles(a.stile_e, a.nb_e, p.e, ne, c);
+    write_sort_tiles(a.stile_g, a.nb_g, p.g, ng, c);
+    if (c == a.C - 1) {
+        a.off_e[a.C] = (int32_t)(p.e + ne);
+        a.off_g[a.C] = (int32_t)(p.g + ng);
+    }
+}
+
+__device__ __forceinline__ void scan_ends(const ScanFinalArgs& a)
+{
+    a.stile_e[0] = 0;
+    a.stile_g[0] = 0;
+    a.stile_e[a.nb_e] = (int32_t)a.C;
+    a.stile_g[a.nb_g] = (int32_t)a.C;
+}
+
 __global__ void __launch_bounds__(256) k_scan_final(ScanFinalArgs a)
 {
     const int64_t c0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPer;
@@ -315,44 +353,157 @@ __global__ void __launch_bounds__(256) k_scan_final(ScanFinalArgs a)
     p.g += a.block_sums[a.n_tiles + blockIdx.x];
     p.m += a.block_sums[2 * a.n_tiles + blockIdx.x];
     const int64_t np_total = *a.n_pairs;
-    const int64_t n_pair_tiles = (np_total + kPairsPerTile - 1) / kPairsPerTile;
 #pragma unroll
     for (int j = 0; j < kScanPer; ++j) {
         const int64_t c = c0 + j;
         if (c >= a.C) break;
-        const int64_t m = ne[j] < ng[j] ? ne[j] : ng[j];
-        a.off_e[c] = (int32_t)p.e;
-        a.off_g[c] = (int32_t)p.g;
-        const int64_t nmax = ne[j] > ng[j] ? ne[j] : ng[j];
-        CellInfo ci;
-        ci.pair_off = (int32_t)p.m;
-        ci.e_start = (int32_t)p.e;
-        ci.g_start = (int32_t)p.g;
-        ci.dens = (float)((double)nmax * a.w_over_v);
-        a.cinfo[c] = ci;
-        if (m > 0) {
-            // scatter tiles whose first pair lies in [p.m, p.m + m)
-            for (int64_t t = (p.m + kPairsPerTile - 1) / kPairsPerTile; t * kPairsPerTile < p.m + m; ++t)
-                a.tile_cell[t] = (int32_t)c;
-            if (p.m + m == np_total) a.tile_cell[n_pair_tiles] = (int32_t)c;
-        }
-        write_sort_tiles(a.stile_e, a.nb_e, p.e, ne[j], c);
-        write_sort_tiles(a.stile_g, a.nb_g, p.g, ng[j], c);
+        scan_cell(a, c, ne[j], ng[j], p, np_total);
         a.count_e[c] = 0;  // becomes the insertion cursor of k_place
         a.count_g[c] = 0;
-        if (c == a.C - 1) {
-            a.off_e[a.C] = (int32_t)(p.e + ne[j]);
-            a.off_g[a.C] = (int32_t)(p.g + ng[j]);
-        }
         p.e += ne[j];
         p.g += ng[j];
-        p.m += m;
+        p.m += ne[j] < ng[j] ? ne[j] : ng[j];
     }
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        a.stile_e[0] = 0;
-        a.stile_g[0] = 0;
-        a.stile_e[a.nb_e] = (int32_t)a.C;
-        a.stile_g[a.nb_g] = (int32_t)a.C;
+    if (blockIdx.x == 0 && threadIdx.x == 0) scan_ends(a);
+}
+
+// ---------------------------------------------------------------------------
+// The binning before the sort of a small call, in one launch and one CTA:
+// histogram (by run boundaries, as k_count) and order check, the scan over
+// cells with all its maps, and, for input not in cell order, the placed
+// indices.  The five launches and the memset it replaces take 2 to 5 us each
+// however little they do; one CTA walks 8192 + 8192 particles in about as long.
+// Whole plain step, its launches in a graph, in order / in no order: 64 cells of
+// 64 + 64 20.8 / 26.3 us against 28.8 / 33.7; 128 cells 22.8 / 33.3 against 30.2
+// / 36.9; 256 cells (not taken) 25.9 / 44.7 against 31.0 / 38.4.
+// ---------------------------------------------------------------------------
+constexpr int kSmallThreads = 1024;
+constexpr int kSmallCells = 4096;
+constexpr int64_t kSmallParticles = 16384;
+
+struct BinSmallArgs {
+    const int32_t* cell[2];
+    ScanFinalArgs scan;  // n_e, n_g, C, offsets, CellInfo, tile maps
+    int64_t* n_pairs;
+    int32_t* idx[2];
+    uint32_t* unsorted;
+    DeviceStats* stats;
+};
+
+__global__ void __launch_bounds__(kSmallThreads) k_bin_small(const __grid_constant__ BinSmallArgs a)
+{
+    __shared__ int32_t count[2][kSmallCells];  // counts, then the next place of each cell
+    __shared__ int3 warp_tot[kSmallThreads / 32];
+    __shared__ int disorder[2];
+    const int tid = threadIdx.x, C = (int)a.scan.C;
+    for (int c = tid; c < C; c += kSmallThreads) count[0][c] = count[1][c] = 0;
+    if (tid < 2) disorder[tid] = 0;
+    __syncthreads();
+    // ---- histogram: half the CTA per species, four consecutive positions per
+    // thread, the next four's loads in flight ----
+    const int hs = tid / (kSmallThreads / 2), ht = tid % (kSmallThreads / 2);
+    bool any_bad = false, dis = false;
+    {
+        const int32_t* __restrict__ cell = a.cell[hs];
+        const int n = (int)(hs == 0 ? a.scan.n_e : a.scan.n_g);
+        const bool vec = (reinterpret_cast<uintptr_t>(cell) & 15u) == 0;
+        constexpr int kStep = 4 * (kSmallThreads / 2);
+        const unsigned lane = lane_id();
+        auto edge = [&](int j0) -> int32_t {
+            if (lane == 0) return j0 > 0 && j0 - 1 < n ? cell[j0 - 1] : -1;
+            if (lane == 31) return j0 + 4 < n ? cell[j0 + 4] : -1;
+            return -1;
+        };
+        int i0 = 4 * ht;
+        int4 q = load_cells4(cell, i0, n, vec);
+        int32_t e = edge(i0);
+        for (int b = 0; b < n; b += kStep, i0 += kStep) {  // the same trips in every thread of the half
+            int4 qn = make_int4(-1, -1, -1, -1);
+            int32_t en = -1;
+            if (b + kStep < n) {
+                qn = load_cells4(cell, i0 + kStep, n, vec);
+                en = edge(i0 + kStep);
+            }
+            const int32_t v[4] = {q.x, q.y, q.z, q.w};
+            int32_t prev = __shfl_up_sync(0xffffffffu, v[3], 1), next = __shfl_down_sync(0xffffffffu, v[0], 1);
+            if (lane == 0) prev = e;
+            if (lane == 31) next = e;
+            q = qn;
+            e = en;
+#pragma unroll
+            for (int j = 0; j < 4; ++j) {
+                const int i = i0 + j;
+                if (i >= n) break;
+                const int32_t c = v[j], pc = j == 0 ? prev : v[j - 1], nc = j == 3 ? next : v[j + 1];
+                const bool ok = (uint32_t)c < (uint32_t)C;
+                any_bad |= !ok;
+                dis |= !ok || (i > 0 && pc > c);
+                const bool first = i == 0 || pc != c, last = i + 1 == n || nc != c;
+                if (ok && (first || last)) atomicAdd(&count[hs][c], (last ? i + 1 : 0) - (first ? i : 0));
+            }
+        }
+    }
+    if (dis) disorder[hs] = 1;
+    if (any_bad) atomicOr(&a.stats->error_flags, (unsigned long long)kErrCellRange);
+    __syncthreads();
+    // ---- scan over cells, kPer consecutive ones per thread ----
+    constexpr int kPer = kSmallCells / kSmallThreads;
+    const int c0 = tid * kPer;
+    int ne[kPer], ng[kPer];
+    int3 v = make_int3(0, 0, 0);  // electrons, photons, pairs
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        ne[j] = c0 + j < C ? count[0][c0 + j] : 0;
+        ng[j] = c0 + j < C ? count[1][c0 + j] : 0;
+        v = make_int3(v.x + ne[j], v.y + ng[j], v.z + (ne[j] < ng[j] ? ne[j] : ng[j]));
+    }
+    int3 inc = v;
+#pragma unroll
+    for (int d = 1; d < 32; d <<= 1) {
+        const int x = __shfl_up_sync(0xffffffffu, inc.x, d), y = __shfl_up_sync(0xffffffffu, inc.y, d),
+                  z = __shfl_up_sync(0xffffffffu, inc.z, d);
+        if (lane_id() >= (unsigned)d) inc = make_int3(inc.x + x, inc.y + y, inc.z + z);
+    }
+    if (lane_id() == 31) warp_tot[tid >> 5] = inc;
+    __syncthreads();
+    int3 p = make_int3(inc.x - v.x, inc.y - v.y, inc.z - v.z);
+    int np_total = 0;
+    for (int w = 0; w < kSmallThreads / 32; ++w) {
+        const int3 t = warp_tot[w];
+        if (w < (tid >> 5)) p = make_int3(p.x + t.x, p.y + t.y, p.z + t.z);
+        np_total += t.z;
+    }
+    const ScanFinalArgs& f = a.scan;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) {
+        const int c = c0 + j;
+        if (c >= C) break;
+        const Tri t{p.x, p.y, p.z};
+        scan_cell(f, c, ne[j], ng[j], t, np_total);
+        count[0][c] = p.x;
+        count[1][c] = p.y;
+        p = make_int3(p.x + ne[j], p.y + ng[j], p.z + (ne[j] < ng[j] ? ne[j] : ng[j]));
+    }
+    if (tid == 0) {
+        scan_ends(f);
+        *a.n_pairs = np_total;
+    }
+    if (tid < 2) a.unsorted[tid] = disorder[tid] ? kIndexPlaced : 0u;
+    __syncthreads();
+    // ---- places ----
+    if (disorder[hs]) {
+        const int n = (int)(hs == 0 ? a.scan.n_e : a.scan.n_g);
+        const int32_t* __restrict__ cell = a.cell[hs];
+        int32_t* __restrict__ idx = a.idx[hs];
+        constexpr int kStride = kSmallThreads / 2;
+        for (int i = ht; i < n; i += 8 * kStride) {
+            int32_t c[8];
+#pragma unroll
+            for (int k = 0; k < 8; ++k) c[k] = i + k * kStride < n ? cell[i + k * kStride] : -1;
+#pragma unroll
+            for (int k = 0; k < 8; ++k)
+                if ((uint32_t)c[k] < (uint32_t)C) idx[atomicAdd(&count[hs][c[k]], 1)] = i + k * kStride;
+        }
     }
 }
 
@@ -875,37 +1026,14 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
     const int64_t C = ctx->cfg.n_cells;
     const int64_t ne = e_in->n, ng = g_in->n;
     const int64_t n_tiles = (C + kScanTile - 1) / kScanTile;
-    // count[0], count[1] and unsorted lie in one block of the workspace
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->count[0], 0,
-                                          reinterpret_cast<char*>(ctx->unsorted + 2) -
-                                              reinterpret_cast<char*>(ctx->count[0]),
-                                          stream));
-
     const int64_t nmax = ne > ng ? ne : ng;
-    const dim3 cgrid(grid_for((nmax + 3) / 4, kCountThreads, ctx->n_sm * kCountCtasPerSm), 2);  // four per thread
-    {
-        TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
-        // 32-bit positions when the grid's last visited position fits
-        const int64_t span = (nmax + 127) / 128 * 128 + (int64_t)cgrid.x * kCountThreads * 4;
-        if (span < ((int64_t)1 << 31))
-            k_count<int32_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
-                                                                  ctx->count[0], ctx->count[1], ctx->unsorted,
-                                                                  ctx->stats);
-        else
-            k_count<int64_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
-                                                                  ctx->count[0], ctx->count[1], ctx->unsorted,
-                                                                  ctx->stats);
-    }
-    COMPTON_LAUNCH_CHECK(ctx, "k_count");
-    TimedScope scan_scope(ctx, COMPTON_K_SCAN, stream);
-    k_scan_reduce<<<(unsigned)n_tiles, 256, 0, stream>>>(ctx->count[0], ctx->count[1], C, ctx->block_sums,
-                                                         n_tiles);
-    COMPTON_LAUNCH_CHECK(ctx, "k_scan_reduce");
-    k_scan_blocks<<<1, 1024, 0, stream>>>(ctx->block_sums, n_tiles, ctx->n_pairs);
-    COMPTON_LAUNCH_CHECK(ctx, "k_scan_blocks");
-
     const int64_t nb_e = (ne + kSortTile - 1) / kSortTile;
     const int64_t nb_g = (ng + kSortTile - 1) / kSortTile;
+    // with per-particle weights a cell's density is its larger count; each
+    // pair scales it by its own heavier weight
+    const bool weighted = e_in->w_dev || g_in->w_dev;
+    const compton_species* ins[2] = {e_in, g_in};
+    compton_species* outs[2] = {e_out, g_out};
     ScanFinalArgs sf;
     sf.count_e = ctx->count[0];
     sf.count_g = ctx->count[1];
@@ -923,38 +1051,76 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
     sf.nb_e = nb_e;
     sf.nb_g = nb_g;
     sf.n_pairs = ctx->n_pairs;
-    // with per-particle weights a cell's density is its larger count; each
-    // pair scales it by its own heavier weight
-    const bool weighted = e_in->w_dev || g_in->w_dev;
     sf.w_over_v = weighted ? 1.0 : ctx->cfg.w_over_v;
-    k_scan_final<<<(unsigned)n_tiles, 256, 0, stream>>>(sf);
-    scan_scope.end();
-    COMPTON_LAUNCH_CHECK(ctx, "k_scan_final");
+    const KeyDraw key_draw(ctx->cfg.seed, step, kStreamPairE, kStreamPairG);
 
-    const dim3 pgrid(grid_for(nmax, kPlaceThreads, ctx->n_sm * kPlaceCtasPerSm), 2);
-    PlaceArgs pa;
-    const compton_species* ins[2] = {e_in, g_in};
-    compton_species* outs[2] = {e_out, g_out};
-    for (int s = 0; s < 2; ++s) {
-        pa.cell[s] = ins[s]->cell_dev;
-        pa.id[s] = ins[s]->id_dev;
-        pa.u[s][0] = ins[s]->ux_dev;
-        pa.u[s][1] = ins[s]->uy_dev;
-        pa.u[s][2] = ins[s]->uz_dev;
-        pa.w[s] = ins[s]->w_dev;
-        pa.n[s] = ins[s]->n;
-        pa.off[s] = ctx->off[s];
-        pa.cursor[s] = ctx->count[s];
-        pa.rec[s] = ctx->rec[s];
+    if (C <= kSmallCells && ne + ng <= kSmallParticles) {
+        BinSmallArgs bs;
+        for (int s = 0; s < 2; ++s) {
+            bs.cell[s] = ins[s]->cell_dev;
+            bs.idx[s] = reinterpret_cast<int32_t*>(ctx->rec[s]);
+        }
+        bs.scan = sf;
+        bs.n_pairs = ctx->n_pairs;
+        bs.unsorted = ctx->unsorted;
+        bs.stats = ctx->stats;
+        TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
+        k_bin_small<<<1, kSmallThreads, 0, stream>>>(bs);
+        COMPTON_LAUNCH_CHECK(ctx, "k_bin_small");
+    } else {
+        // count[0], count[1] and unsorted lie in one block of the workspace
+        COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->count[0], 0,
+                                              reinterpret_cast<char*>(ctx->unsorted + 2) -
+                                                  reinterpret_cast<char*>(ctx->count[0]),
+                                              stream));
+        const dim3 cgrid(grid_for((nmax + 3) / 4, kCountThreads, ctx->n_sm * kCountCtasPerSm), 2);  // four per thread
+        {
+            TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
+            // 32-bit positions when the grid's last visited position fits
+            const int64_t span = (nmax + 127) / 128 * 128 + (int64_t)cgrid.x * kCountThreads * 4;
+            if (span < ((int64_t)1 << 31))
+                k_count<int32_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
+                                                                      ctx->count[0], ctx->count[1], ctx->unsorted,
+                                                                      ctx->stats);
+            else
+                k_count<int64_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
+                                                                      ctx->count[0], ctx->count[1], ctx->unsorted,
+                                                                      ctx->stats);
+        }
+        COMPTON_LAUNCH_CHECK(ctx, "k_count");
+        TimedScope scan_scope(ctx, COMPTON_K_SCAN, stream);
+        k_scan_reduce<<<(unsigned)n_tiles, 256, 0, stream>>>(ctx->count[0], ctx->count[1], C, ctx->block_sums,
+                                                             n_tiles);
+        COMPTON_LAUNCH_CHECK(ctx, "k_scan_reduce");
+        k_scan_blocks<<<1, 1024, 0, stream>>>(ctx->block_sums, n_tiles, ctx->n_pairs);
+        COMPTON_LAUNCH_CHECK(ctx, "k_scan_blocks");
+        k_scan_final<<<(unsigned)n_tiles, 256, 0, stream>>>(sf);
+        scan_scope.end();
+        COMPTON_LAUNCH_CHECK(ctx, "k_scan_final");
+
+        const dim3 pgrid(grid_for(nmax, kPlaceThreads, ctx->n_sm * kPlaceCtasPerSm), 2);
+        PlaceArgs pa;
+        for (int s = 0; s < 2; ++s) {
+            pa.cell[s] = ins[s]->cell_dev;
+            pa.id[s] = ins[s]->id_dev;
+            pa.u[s][0] = ins[s]->ux_dev;
+            pa.u[s][1] = ins[s]->uy_dev;
+            pa.u[s][2] = ins[s]->uz_dev;
+            pa.w[s] = ins[s]->w_dev;
+            pa.n[s] = ins[s]->n;
+            pa.off[s] = ctx->off[s];
+            pa.cursor[s] = ctx->count[s];
+            pa.rec[s] = ctx->rec[s];
+        }
+        pa.unsorted = ctx->unsorted;
+        pa.C = C;
+        pa.draw = key_draw;
+        {
+            TimedScope ts_(ctx, COMPTON_K_PLACE, stream);
+            k_place<<<pgrid, kPlaceThreads, 0, stream>>>(pa);
+        }
+        COMPTON_LAUNCH_CHECK(ctx, "k_place");
     }
-    pa.unsorted = ctx->unsorted;
-    pa.C = C;
-    pa.draw = KeyDraw(ctx->cfg.seed, step, kStreamPairE, kStreamPairG);
-    {
-        TimedScope ts_(ctx, COMPTON_K_PLACE, stream);
-        k_place<<<pgrid, kPlaceThreads, 0, stream>>>(pa);
-    }
-    COMPTON_LAUNCH_CHECK(ctx, "k_place");
 
     if (nb_e + nb_g > 0) {
         SortGatherArgs sg;
@@ -975,7 +1141,7 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
             sg.stile[s] = ctx->stile[s];
             sg.n[s] = ins[s]->n;
         }
-        sg.draw = pa.draw;
+        sg.draw = key_draw;
         sg.unsorted = ctx->unsorted;
         sg.nb_e = nb_e;
         const int smem = (int)kSortSmem;

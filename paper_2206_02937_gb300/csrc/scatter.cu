@@ -194,8 +194,11 @@ struct Batch {
 // kCandOut (the surrogate modes' first kernel): the same filter, but each
 // batch of candidates goes with its momenta to the context's candidate list
 // (one atomic per batch) instead of being evaluated.
-template <bool kBinned, bool kWeighted, bool kCandOut = false>
-__global__ void __launch_bounds__(kProbThreads, 4) k_pair_prob(ScatterArgs a)
+// kResolve (a small call): every warp resolves its own accepted pairs at the
+// end, which saves the collision kernel's launch; where warps have many pairs
+// the collisions' registers and the idle lanes cost more than the launch.
+template <bool kBinned, bool kWeighted, bool kCandOut = false, bool kResolve = false>
+__global__ void __launch_bounds__(kProbThreads, kResolve ? 2 : 4) k_pair_prob(ScatterArgs a)
 {
     __shared__ WarpWindow s_win[kProbWarps];
     __shared__ WarpQueue s_queue[kProbWarps];
@@ -448,6 +451,11 @@ __global__ void __launch_bounds__(kProbThreads, 4) k_pair_prob(ScatterArgs a)
             a.accepted[acc_base + n_acc + __popc(m & lt_mask)] =
                 AcceptedPair{c.ie, c.ig, x, c.p, {c.u[0], c.u[1], c.u[2]}, {c.k[0], c.k[1], c.k[2]}, {0u, 0u}};
         n_acc += __popc(m);
+    }
+
+    if (kResolve) {
+        __syncwarp();  // the warp's entries are visible to every lane
+        for (uint32_t i = lane; i < n_acc; i += 32) resolve(a, a.accepted[acc_base + i]);
     }
 
     // counters: the warp's accepted count for the collision kernel, warp
@@ -947,6 +955,11 @@ compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, cu
     return COMPTON_OK;
 }
 
+// Pair tiles up to which a plain step resolves its collisions in the
+// probability kernel: one chunk of 128 pairs per warp, about four collisions,
+// which take less than the 6 us of the collision kernel's launch.
+constexpr unsigned kResolveTiles = 32;
+
 // The step after the pair list is known: probability and trial of every
 // pair (plain: one kernel; surrogate: candidates, network, decisions), then
 // the collisions.  Tiles: pair tiles of this launch; rows: a host bound on
@@ -955,9 +968,14 @@ template <bool kBinned, bool kWeighted>
 compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, unsigned tiles, int64_t rows,
                            cudaStream_t stream)
 {
-    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->n_accepted, 0, sizeof(uint32_t), stream));
     if (mode == COMPTON_MODE_PLAIN) {
         const unsigned grid = prob_grid(ctx, tiles);
+        if (tiles <= kResolveTiles) {
+            TimedScope ts_(ctx, COMPTON_K_PROB, stream);
+            k_pair_prob<kBinned, kWeighted, false, true><<<grid, kProbThreads, 0, stream>>>(a);
+            COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
+            return COMPTON_OK;
+        }
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
             k_pair_prob<kBinned, kWeighted><<<grid, kProbThreads, 0, stream>>>(a);
@@ -972,6 +990,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         COMPTON_LAUNCH_CHECK(ctx, "k_collide_regions");
         return COMPTON_OK;
     } else {
+        COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->n_accepted, 0, sizeof(uint32_t), stream));
         COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->n_cand, 0, sizeof(uint32_t), stream));
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
