@@ -7,7 +7,7 @@
 // does all before the sort in one, and the sort):
 //   k_count        histogram of cell indices by run boundaries, order check
 //   k_scan_reduce  per-tile sums of N_e,c, N_g,c and M_c = min(N_e,c, N_g,c)
-//   k_scan_blocks  exclusive scan of the tile sums (one CTA)
+//   k_scan_blocks  exclusive scan of the tile sums (one CTA; many cells only)
 //   k_scan_final   per-cell offsets, CellInfo, tile maps; resets the cursors
 //   k_place        input not in cell order only: each particle's index (input
 //                  nearly in order) or its record (key, id, momentum) placed
@@ -67,6 +67,7 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
                                                         int32_t* __restrict__ count_e, int32_t* __restrict__ count_g,
                                                         uint32_t* __restrict__ unsorted, DeviceStats* stats)
 {
+    chain_start();
     const int s = blockIdx.y;
     const int32_t* __restrict__ cell = s == 0 ? cell_e : cell_g;
     const Idx n = (Idx)(s == 0 ? n_e : n_g);
@@ -212,6 +213,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const int32_t* __restrict__
                                                      const int32_t* __restrict__ count_g, int64_t C,
                                                      int64_t* __restrict__ block_sums, int64_t n_tiles)
 {
+    chain_start();
     const int64_t c0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPer;
     Tri v{0, 0, 0};
 #pragma unroll
@@ -234,6 +236,7 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const int32_t* __restrict__
 __global__ void __launch_bounds__(1024) k_scan_blocks(int64_t* __restrict__ block_sums, int64_t n_tiles,
                                                       int64_t* __restrict__ n_pairs)
 {
+    chain_start();
     __shared__ int64_t warp_tot[32];
     for (int s = 0; s < 3; ++s) {
         int64_t* a = block_sums + s * n_tiles;
@@ -284,7 +287,7 @@ struct ScanFinalArgs {
     int32_t* stile_e;
     int32_t* stile_g;
     int64_t nb_e, nb_g;  // sort tiles per species
-    const int64_t* n_pairs;
+    int64_t* n_pairs;
     double w_over_v;
 };
 
@@ -335,8 +338,47 @@ __device__ __forceinline__ void scan_ends(const ScanFinalArgs& a)
     a.stile_g[a.nb_g] = (int32_t)a.C;
 }
 
-__global__ void __launch_bounds__(256) k_scan_final(ScanFinalArgs a)
+// The sums of the tiles before this block's, and the pairs of all tiles in
+// *total_m: each block adds them up itself, which takes it about as long as
+// waiting for one block's scan of them and saves that launch.
+__device__ __forceinline__ Tri tiles_before(const ScanFinalArgs& a, int64_t* total_m)
 {
+    __shared__ Tri warp_sum[8];
+    __shared__ int64_t warp_m[8];
+    Tri s{0, 0, 0};
+    int64_t tm = 0;
+    for (int64_t t = threadIdx.x; t < a.n_tiles; t += 256) {
+        const int64_t m = a.block_sums[2 * a.n_tiles + t];
+        tm += m;
+        if (t < (int64_t)blockIdx.x) s = tri_add(s, Tri{a.block_sums[t], a.block_sums[a.n_tiles + t], m});
+    }
+#pragma unroll
+    for (int d = 16; d > 0; d >>= 1) {
+        s.e += __shfl_xor_sync(0xffffffffu, s.e, d);
+        s.g += __shfl_xor_sync(0xffffffffu, s.g, d);
+        s.m += __shfl_xor_sync(0xffffffffu, s.m, d);
+        tm += __shfl_xor_sync(0xffffffffu, tm, d);
+    }
+    if (lane_id() == 0) {
+        warp_sum[threadIdx.x >> 5] = s;
+        warp_m[threadIdx.x >> 5] = tm;
+    }
+    __syncthreads();
+    s = warp_sum[0];
+    tm = warp_m[0];
+    for (int w = 1; w < 8; ++w) {
+        s = tri_add(s, warp_sum[w]);
+        tm += warp_m[w];
+    }
+    *total_m = tm;
+    return s;
+}
+
+// kOwnPrefix: block_sums hold the tiles' sums (k_scan_blocks has not run).
+template <bool kOwnPrefix>
+__global__ void __launch_bounds__(256) k_scan_final(const __grid_constant__ ScanFinalArgs a)
+{
+    chain_start();
     const int64_t c0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPer;
     int32_t ne[kScanPer], ng[kScanPer];
     Tri v{0, 0, 0};
@@ -349,10 +391,15 @@ __global__ void __launch_bounds__(256) k_scan_final(ScanFinalArgs a)
     }
     Tri total;
     Tri p = block_excl_scan_256(v, &total);
-    p.e += a.block_sums[blockIdx.x];
-    p.g += a.block_sums[a.n_tiles + blockIdx.x];
-    p.m += a.block_sums[2 * a.n_tiles + blockIdx.x];
-    const int64_t np_total = *a.n_pairs;
+    int64_t np_total;
+    if (kOwnPrefix) {
+        p = tri_add(p, tiles_before(a, &np_total));
+        if (blockIdx.x == 0 && threadIdx.x == 0) *a.n_pairs = np_total;
+    } else {
+        p = tri_add(p, Tri{a.block_sums[blockIdx.x], a.block_sums[a.n_tiles + blockIdx.x],
+                           a.block_sums[2 * a.n_tiles + blockIdx.x]});
+        np_total = *a.n_pairs;
+    }
 #pragma unroll
     for (int j = 0; j < kScanPer; ++j) {
         const int64_t c = c0 + j;
@@ -392,6 +439,7 @@ struct BinSmallArgs {
 
 __global__ void __launch_bounds__(kSmallThreads) k_bin_small(const __grid_constant__ BinSmallArgs a)
 {
+    chain_start();
     __shared__ int32_t count[2][kSmallCells];  // counts, then the next place of each cell
     __shared__ int3 warp_tot[kSmallThreads / 32];
     __shared__ int disorder[2];
@@ -555,8 +603,10 @@ __device__ __forceinline__ void claim_places(const int32_t* __restrict__ off, in
     if (c >= 0 && lane == (unsigned)leader) first_place = off[c] + atomicAdd(&cursor[c], __popc(peers));
 }
 
+template <bool kChained>
 __global__ void __launch_bounds__(kPlaceThreads, 2048 / kPlaceThreads) k_place(const __grid_constant__ PlaceArgs a)
 {
+    if (kChained) chain_start();
     const int s = blockIdx.y;
     const int64_t n = a.n[s];
     const SortSource source = sort_source(a.unsorted[s], n);
@@ -949,9 +999,12 @@ __device__ void sort_giant_cell(const SortGatherArgs& g, int s, const SortSrc& t
 }
 
 constexpr size_t kSortSmem = (size_t)kSortCap * (4 + 4 * kBucketsPerSlot + 4 + 12 + 2 + 2);
+static_assert(kSortSmem <= 48 * 1024, "above what a launch may take without asking for it");
 
+template <bool kChained>
 __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(const __grid_constant__ SortGatherArgs g)
 {
+    if (kChained) chain_start();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     SortSmem m;
     m.id = reinterpret_cast<uint32_t*>(smem_raw);
@@ -1003,6 +1056,13 @@ __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(const __grid_c
         c = e;
     }
 }
+
+// Tiles of the scan up to which k_scan_final adds up the tiles before its own
+// (half a million cells; every block reads all the sums, 12 KB of them in the
+// L2 there, and their number grows with the square).  301^2 cells, 89 tiles: the
+// step 347 us with the block scan and launches one by one, 334 with the sums
+// taken here and launches chained.
+constexpr int64_t kOwnPrefixTiles = 512;
 
 // CTAs per SM and species of the grid-stride histogram (the launch's second
 // grid dimension takes the two species), which runs in one wave of 1024-thread CTAs: 0.0394 ms on the 512^2 step against
@@ -1065,7 +1125,7 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
         bs.unsorted = ctx->unsorted;
         bs.stats = ctx->stats;
         TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
-        k_bin_small<<<1, kSmallThreads, 0, stream>>>(bs);
+        launch_chained(k_bin_small, 1, kSmallThreads, 0, stream, bs);
         COMPTON_LAUNCH_CHECK(ctx, "k_bin_small");
     } else {
         // count[0], count[1] and unsorted lie in one block of the workspace
@@ -1079,22 +1139,24 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
             // 32-bit positions when the grid's last visited position fits
             const int64_t span = (nmax + 127) / 128 * 128 + (int64_t)cgrid.x * kCountThreads * 4;
             if (span < ((int64_t)1 << 31))
-                k_count<int32_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
-                                                                      ctx->count[0], ctx->count[1], ctx->unsorted,
-                                                                      ctx->stats);
+                launch_chained(k_count<int32_t>, cgrid, kCountThreads, 0, stream, e_in->cell_dev, ne, g_in->cell_dev,
+                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, ctx->stats);
             else
-                k_count<int64_t><<<cgrid, kCountThreads, 0, stream>>>(e_in->cell_dev, ne, g_in->cell_dev, ng, C,
-                                                                      ctx->count[0], ctx->count[1], ctx->unsorted,
-                                                                      ctx->stats);
+                launch_chained(k_count<int64_t>, cgrid, kCountThreads, 0, stream, e_in->cell_dev, ne, g_in->cell_dev,
+                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, ctx->stats);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_count");
         TimedScope scan_scope(ctx, COMPTON_K_SCAN, stream);
-        k_scan_reduce<<<(unsigned)n_tiles, 256, 0, stream>>>(ctx->count[0], ctx->count[1], C, ctx->block_sums,
-                                                             n_tiles);
+        launch_chained(k_scan_reduce, (unsigned)n_tiles, 256, 0, stream, ctx->count[0], ctx->count[1], C,
+                       ctx->block_sums, n_tiles);
         COMPTON_LAUNCH_CHECK(ctx, "k_scan_reduce");
-        k_scan_blocks<<<1, 1024, 0, stream>>>(ctx->block_sums, n_tiles, ctx->n_pairs);
-        COMPTON_LAUNCH_CHECK(ctx, "k_scan_blocks");
-        k_scan_final<<<(unsigned)n_tiles, 256, 0, stream>>>(sf);
+        if (n_tiles <= kOwnPrefixTiles) {
+            launch_chained(k_scan_final<true>, (unsigned)n_tiles, 256, 0, stream, sf);
+        } else {
+            launch_chained(k_scan_blocks, 1, 1024, 0, stream, ctx->block_sums, n_tiles, ctx->n_pairs);
+            COMPTON_LAUNCH_CHECK(ctx, "k_scan_blocks");
+            launch_chained(k_scan_final<false>, (unsigned)n_tiles, 256, 0, stream, sf);
+        }
         scan_scope.end();
         COMPTON_LAUNCH_CHECK(ctx, "k_scan_final");
 
@@ -1117,7 +1179,10 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
         pa.draw = key_draw;
         {
             TimedScope ts_(ctx, COMPTON_K_PLACE, stream);
-            k_place<<<pgrid, kPlaceThreads, 0, stream>>>(pa);
+            if ((int64_t)pgrid.x * pgrid.y <= kChainBlocks)
+                launch_chained(k_place<true>, pgrid, kPlaceThreads, 0, stream, pa);
+            else
+                k_place<false><<<pgrid, kPlaceThreads, 0, stream>>>(pa);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_place");
     }
@@ -1145,10 +1210,11 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
         sg.unsorted = ctx->unsorted;
         sg.nb_e = nb_e;
         const int smem = (int)kSortSmem;
-        COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_sort_gather, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                                   smem));
         TimedScope ts_(ctx, COMPTON_K_SORT, stream);
-        k_sort_gather<<<(unsigned)(nb_e + nb_g), kSortThreads, smem, stream>>>(sg);
+        if (nb_e + nb_g <= kChainBlocks)
+            launch_chained(k_sort_gather<true>, (unsigned)(nb_e + nb_g), kSortThreads, smem, stream, sg);
+        else
+            k_sort_gather<false><<<(unsigned)(nb_e + nb_g), kSortThreads, smem, stream>>>(sg);
         COMPTON_LAUNCH_CHECK(ctx, "k_sort_gather");
     }
     return COMPTON_OK;

@@ -18,6 +18,14 @@
 
 namespace compton {
 
+// First statement of a kernel launched with launch_chained: waits until the
+// stream's previous kernel has completed and its writes are visible (nothing is
+// read before), then lets the next one's blocks be placed.
+__device__ __forceinline__ void chain_start()
+{
+    asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------
 // Philox4x32-10 from its published definition: ten rounds; each round takes
 // the two 32x32->64 products of words 0 and 2 with the round multipliers,

@@ -157,6 +157,7 @@ constexpr int kFinishThreads = 1024;
 template <bool kAdam>
 __global__ void __launch_bounds__(kFinishThreads) k_mlp_finish(MlpDev m, AdamArgs ad)
 {
+    chain_start();
     __shared__ float w[64][65];  // the layer's weights [out][in], layer 0 zero-padded to 64 inputs
     __shared__ float hb[64];     // half biases
     __shared__ float red[32];
@@ -433,6 +434,7 @@ __device__ __forceinline__ bool group_sync_or(int g, bool flag)
 template <bool kFp8>
 __global__ void __launch_bounds__(kMlpThreads, kMlpMinCtas) k_mlp_tc(MlpArgs a)
 {
+    chain_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint8_t* Wt = sm + kOffW;
@@ -667,6 +669,7 @@ static_assert(kTaOffBB % 256 == 0 && kTaOffOnes % 256 == 0, "32-byte swizzled bl
 
 __global__ void __launch_bounds__(kTaThreads, 1) k_mlp_ta(MlpArgs a)
 {
+    chain_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x;
@@ -842,6 +845,7 @@ struct F32Smem {
 template <bool kCalib>
 __global__ void __launch_bounds__(kF32Threads, 1) k_mlp_fp32(MlpArgs a)
 {
+    chain_start();
     extern __shared__ __align__(16) float smf[];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const MlpDev& m = a.m;
@@ -996,7 +1000,7 @@ int grid_persistent(const void* kernel, int threads, int smem, int64_t work_item
 
 compton_status mlp_repack(compton_ctx* ctx, cudaStream_t stream)
 {
-    k_mlp_finish<false><<<5, kFinishThreads, 0, stream>>>(ctx->mlp, AdamArgs{});
+    launch_chained(k_mlp_finish<false>, 5, kFinishThreads, 0, stream, ctx->mlp, AdamArgs{});
     COMPTON_LAUNCH_CHECK(ctx, "k_mlp_finish");
     return COMPTON_OK;
 }
@@ -1007,7 +1011,7 @@ compton_status mlp_adam(compton_ctx* ctx, float lr, cudaStream_t stream)
     if (inject_fault()) return set_injected_error(ctx, "k_mlp_finish");  // before the update, not after it
     const double step = (double)(ctx->adam_step + 1);
     AdamArgs ad{lr, 0.9f, 0.999f, 1e-7f, 1.0f - (float)std::pow(0.9, step), 1.0f - (float)std::pow(0.999, step)};
-    k_mlp_finish<true><<<5, kFinishThreads, 0, stream>>>(ctx->mlp, ad);
+    launch_chained(k_mlp_finish<true>, 5, kFinishThreads, 0, stream, ctx->mlp, ad);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "k_mlp_finish");
     ctx->adam_step += 1;
@@ -1052,7 +1056,7 @@ compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* 
         const int grid = f32_grid(ctx, n);
         {
             TimedScope ts_(ctx, COMPTON_K_MLP, stream);
-            k_mlp_fp32<false><<<grid, kF32Threads, smem, stream>>>(a);
+            launch_chained(k_mlp_fp32<false>, grid, kF32Threads, smem, stream, a);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_mlp_fp32");
         return COMPTON_OK;
@@ -1064,7 +1068,7 @@ compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* 
         const int grid_ta = grid_persistent(kt, kTaThreads, (int)kTaSmemLaunch, n, kTileM * kTaGroups);
         {
             TimedScope ts_(ctx, COMPTON_K_MLP, stream);
-            k_mlp_ta<<<grid_ta, kTaThreads, kTaSmemLaunch, stream>>>(a);
+            launch_chained(k_mlp_ta, grid_ta, kTaThreads, kTaSmemLaunch, stream, a);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_mlp_ta");
         return COMPTON_OK;
@@ -1074,8 +1078,8 @@ compton_status launch_mlp_infer(compton_ctx* ctx, const float* ux, const float* 
     const int grid = grid_persistent(kern, kMlpThreads, (int)kSmemTc, n, kTileM * kMlpGroups);
     {
         TimedScope ts_(ctx, COMPTON_K_MLP, stream);
-        if (fp8) k_mlp_tc<true><<<grid, kMlpThreads, kSmemTc, stream>>>(a);
-        else k_mlp_tc<false><<<grid, kMlpThreads, kSmemTc, stream>>>(a);
+        if (fp8) launch_chained(k_mlp_tc<true>, grid, kMlpThreads, kSmemTc, stream, a);
+        else launch_chained(k_mlp_tc<false>, grid, kMlpThreads, kSmemTc, stream, a);
     }
     COMPTON_LAUNCH_CHECK(ctx, fp8 ? "k_mlp_tc<fp8>" : "k_mlp_tc<bf16>");
     return COMPTON_OK;
@@ -1130,7 +1134,7 @@ compton_status launch_mlp_calibrate(compton_ctx* ctx, const float* ux, const flo
     COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.amax, 0, 4 * sizeof(float), stream));
     COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_mlp_fp32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     const int grid = f32_grid(ctx, n);
-    k_mlp_fp32<true><<<grid, kF32Threads, smem, stream>>>(a);
+    launch_chained(k_mlp_fp32<true>, grid, kF32Threads, smem, stream, a);
     COMPTON_LAUNCH_CHECK(ctx, "k_mlp_fp32<calib>");
     k_mlp_set_act_scales<<<1, 32, 0, stream>>>(ctx->mlp);
     COMPTON_LAUNCH_CHECK(ctx, "k_mlp_set_act_scales");

@@ -15,6 +15,7 @@
 //                    w, the inference images rebuilt, acc cleared for the
 //                    next step.
 #include "ctx.hpp"
+#include "device_math.cuh"
 #include "features.cuh"
 
 namespace compton {
@@ -88,6 +89,7 @@ __device__ __forceinline__ float dot4(float4 x, float4 y, float t)
 
 __global__ void __launch_bounds__(kTrThreads, 1) k_train_f32(TrainArgs a)
 {
+    chain_start();
     extern __shared__ __align__(16) float sm[];
     using S = TrainSmem;
     const int tid = threadIdx.x;
@@ -394,7 +396,7 @@ compton_status launch_mlp_train_step(compton_ctx* ctx, const float* ux, const fl
         COMPTON_CUDA_TRY(ctx, cudaFuncSetAttribute(k_train_f32, cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
         const int64_t tiles = (n + kTrTile - 1) / kTrTile;
         const unsigned grid = (unsigned)(tiles < ctx->n_sm ? tiles : ctx->n_sm);
-        k_train_f32<<<grid, kTrThreads, smem, stream>>>(a);
+        launch_chained(k_train_f32, grid, kTrThreads, smem, stream, a);
         COMPTON_LAUNCH_CHECK(ctx, "k_train_f32");
     }
     st = mlp_adam(ctx, lr, stream);

@@ -147,6 +147,7 @@ struct TrainTcArgs {
 
 __global__ void __launch_bounds__(kTcThreads, 1) k_train_tc(TrainTcArgs a)
 {
+    chain_start();
     extern __shared__ uint8_t smem_raw[];
     uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const int tid = threadIdx.x;
@@ -420,7 +421,7 @@ compton_status launch_mlp_grad_tc(compton_ctx* ctx, const float* ux, const float
                                                (int)kSmemTrainTc));
     const int64_t tiles = (n + kTT - 1) / kTT;
     const int64_t grid = tiles < ctx->n_sm ? tiles : ctx->n_sm;  // one CTA per SM (all 512 TMEM columns)
-    k_train_tc<<<(unsigned)grid, kTcThreads, kSmemTrainTc, stream>>>(a);
+    launch_chained(k_train_tc, (unsigned)grid, kTcThreads, kSmemTrainTc, stream, a);
     COMPTON_LAUNCH_CHECK(ctx, "k_train_tc");
     return COMPTON_OK;
 }

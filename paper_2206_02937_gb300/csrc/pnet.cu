@@ -110,6 +110,7 @@ __device__ __forceinline__ void stage_params(const PnetDev& p, float* th)
 template <bool kCand>
 __global__ void __launch_bounds__(kPnetThreads, 3) k_pnet_infer(PnetArgs a)
 {
+    chain_start();
     __shared__ float th[kPnetParams];
     stage_params(a.p, th);
     const unsigned lane = threadIdx.x & 31u;
@@ -237,6 +238,7 @@ __device__ __forceinline__ void train_rows(int p, int& ra, int& rb)
 template <int kS>
 __global__ void __launch_bounds__(kTrainThreads, 1) k_pnet_train(PnetArgs a, float lr, float b1t, float b2t)
 {
+    chain_start();
     constexpr int kStride = kS + 4;
     extern __shared__ __align__(16) float rows[];  // [kTrainRows][kStride]
     __shared__ float th[kPnetParams];
@@ -385,7 +387,7 @@ compton_status launch_pnet_infer(compton_ctx* ctx, const float* ux, const float*
     a.r_out = r_out;
     {
         TimedScope ts_(ctx, COMPTON_K_MLP, stream);
-        k_pnet_infer<false><<<pnet_grid(n), kPnetThreads, 0, stream>>>(a);
+        launch_chained(k_pnet_infer<false>, pnet_grid(n), kPnetThreads, 0, stream, a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_pnet_infer");
     return COMPTON_OK;
@@ -414,7 +416,7 @@ compton_status launch_pnet_decide(compton_ctx* ctx, int64_t rows, const MlpDecid
     a.range.range_e2max = ctx->pnet.range[2];
     {
         TimedScope ts_(ctx, COMPTON_K_MLP, stream);
-        k_pnet_infer<true><<<pnet_grid(rows), kPnetThreads, 0, stream>>>(a);
+        launch_chained(k_pnet_infer<true>, pnet_grid(rows), kPnetThreads, 0, stream, a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_pnet_infer<cand>");
     return COMPTON_OK;
@@ -453,8 +455,8 @@ compton_status launch_pnet_train_step(compton_ctx* ctx, const float* ux, const f
                                                    cudaFuncAttributeMaxDynamicSharedMemorySize, smem));
     // the launch is the whole step: an injected failure comes before it, so that no failed call has updated anything
     if (inject_fault()) return set_injected_error(ctx, "k_pnet_train");
-    if (big) k_pnet_train<kTrainTileBig><<<grid, kTrainThreads, smem, stream>>>(a, lr, b1t, b2t);
-    else k_pnet_train<kTrainTile><<<grid, kTrainThreads, smem, stream>>>(a, lr, b1t, b2t);
+    if (big) launch_chained(k_pnet_train<kTrainTileBig>, grid, kTrainThreads, smem, stream, a, lr, b1t, b2t);
+    else launch_chained(k_pnet_train<kTrainTile>, grid, kTrainThreads, smem, stream, a, lr, b1t, b2t);
     const cudaError_t e = cudaGetLastError();
     if (e != cudaSuccess) return set_cuda_error(ctx, e, "k_pnet_train");
     P.step = step;

@@ -200,6 +200,7 @@ struct Batch {
 template <bool kBinned, bool kWeighted, bool kCandOut = false, bool kResolve = false>
 __global__ void __launch_bounds__(kProbThreads, kResolve ? 2 : 4) k_pair_prob(ScatterArgs a)
 {
+    chain_start();
     __shared__ WarpWindow s_win[kProbWarps];
     __shared__ WarpQueue s_queue[kProbWarps];
     const unsigned lane = threadIdx.x & 31u;
@@ -476,8 +477,10 @@ __global__ void __launch_bounds__(kProbThreads, kResolve ? 2 : 4) k_pair_prob(Sc
 // 0.083, 0.072, 0.066 and 0.065 ms on the 512^2 step; the regions' lengths
 // vary, and with one warp each the longest set the kernel's time).
 constexpr int kCollideWarps = 8;
+template <bool kChained>
 __global__ void __launch_bounds__(128) k_collide_regions(ScatterArgs a, int prob_warps)
 {
+    if (kChained) chain_start();
     const int64_t total = a.n_pairs ? *a.n_pairs : a.p_end;
     const int64_t pbase = a.n_pairs ? 0 : a.p_begin;
     const int64_t n_chunks = total > pbase ? (total - pbase + kChunkPairs - 1) / kChunkPairs : 0;
@@ -499,6 +502,7 @@ __global__ void __launch_bounds__(128) k_collide_regions(ScatterArgs a, int prob
 // path (counted); the decision; accepted pairs to the list.
 __global__ void __launch_bounds__(256) k_decide(ScatterArgs a)
 {
+    chain_start();
     const uint32_t n = *a.n_cand;
     const unsigned lane = threadIdx.x & 31u;
     unsigned n_hit = 0, n_fb = 0;
@@ -555,8 +559,10 @@ __global__ void __launch_bounds__(256) k_decide(ScatterArgs a)
     }
 }
 
+template <bool kChained>
 __global__ void __launch_bounds__(256) k_collide(ScatterArgs a)
 {
+    if (kChained) chain_start();
     const uint32_t n = *a.n_accepted;
     const uint32_t stride = gridDim.x * blockDim.x;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += stride) resolve(a, a.accepted[i]);
@@ -949,7 +955,9 @@ compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, cu
 {
     {
         TimedScope ts_(ctx, COMPTON_K_COLLIDE, stream);
-        k_collide<<<collide_grid(rows), 256, 0, stream>>>(a);
+        const unsigned grid = (unsigned)collide_grid(rows);
+        if (grid <= kChainBlocks) launch_chained(k_collide<true>, grid, 256, 0, stream, a);
+        else k_collide<false><<<grid, 256, 0, stream>>>(a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_collide");
     return COMPTON_OK;
@@ -972,20 +980,22 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         const unsigned grid = prob_grid(ctx, tiles);
         if (tiles <= kResolveTiles) {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
-            k_pair_prob<kBinned, kWeighted, false, true><<<grid, kProbThreads, 0, stream>>>(a);
+            launch_chained(k_pair_prob<kBinned, kWeighted, false, true>, grid, kProbThreads, 0, stream, a);
             COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
             return COMPTON_OK;
         }
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
-            k_pair_prob<kBinned, kWeighted><<<grid, kProbThreads, 0, stream>>>(a);
+            launch_chained(k_pair_prob<kBinned, kWeighted>, grid, kProbThreads, 0, stream, a);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
         const int prob_warps = (int)grid * kProbWarps;
         {
             TimedScope ts_(ctx, COMPTON_K_COLLIDE, stream);
             // kCollideWarps warps per region, four to a CTA
-            k_collide_regions<<<(kCollideWarps * prob_warps + 3) / 4, 128, 0, stream>>>(a, prob_warps);
+            const unsigned cgrid = (unsigned)(kCollideWarps * prob_warps + 3) / 4;
+            if (cgrid <= kChainBlocks) launch_chained(k_collide_regions<true>, cgrid, 128, 0, stream, a, prob_warps);
+            else k_collide_regions<false><<<cgrid, 128, 0, stream>>>(a, prob_warps);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_collide_regions");
         return COMPTON_OK;
@@ -995,7 +1005,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
             // the candidate filter of the plain kernel, candidates to the list
-            k_pair_prob<kBinned, kWeighted, true><<<prob_grid(ctx, tiles), kProbThreads, 0, stream>>>(a);
+            launch_chained(k_pair_prob<kBinned, kWeighted, true>, prob_grid(ctx, tiles), kProbThreads, 0, stream, a);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob<cand>");
         // tensor-core modes and the paper's network decide inside the network
@@ -1012,7 +1022,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         if (st != COMPTON_OK) return st;
         if (!fused) {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
-            k_decide<<<collide_grid(rows), 256, 0, stream>>>(a);
+            launch_chained(k_decide, collide_grid(rows), 256, 0, stream, a);
         }
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
@@ -1096,7 +1106,7 @@ compton_status launch_decide(compton_ctx* ctx, const CandList& list, int64_t row
     a.n_accepted = list.n_accepted;
     a.r_mlp = list.r;
     a.count_fallbacks = false;
-    k_decide<<<collide_grid(rows), 256, 0, stream>>>(a);
+    launch_chained(k_decide, collide_grid(rows), 256, 0, stream, a);
     COMPTON_LAUNCH_CHECK(ctx, "k_decide");
     return COMPTON_OK;
 }
