@@ -134,9 +134,9 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
         delete ctx;
         return COMPTON_EINVAL;
     }
-    const size_t o_ac = cv.take<float>(cfg->max_train_batch > 0 ? NP + 3 : 1);
+    const size_t o_ac = cv.take<char>(cfg->max_train_batch > 0 ? compton::kMlpAccBytes : 1);
     size_t o_rb = cv.take<float>(P > 0 ? P : 1);
-    size_t o_pn = cv.take<float>(4 * compton::kPnetParams + 2 + compton::kPnetParams + 2 + 1);
+    size_t o_pn = cv.take<float>(5 * compton::kPnetParams + 3 + 4);
     const size_t total = align_up(cv.used, 256);
     if (cfg->mem_budget_bytes && total > cfg->mem_budget_bytes) {
         delete ctx;
@@ -188,7 +188,9 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
     m.hist = reinterpret_cast<int*>(base + o_hi);
     if (cfg->max_train_batch > 0) {
         m.acc = reinterpret_cast<float*>(base + o_ac);
-        m.ticket = reinterpret_cast<uint32_t*>(m.acc + NP + 2);
+        m.ticket = reinterpret_cast<uint32_t*>(m.acc + NP);
+        static_assert((compton::kMlpParams + 1) % 2 == 0, "doubles on 8 bytes");
+        m.acc_loss = reinterpret_cast<double*>(m.acc + NP + 1);
     }
     ctx->r_buf = reinterpret_cast<float*>(base + o_rb);
     {
@@ -200,7 +202,9 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
         pn.adam_v = pb + 3 * compton::kPnetParams;
         pn.loss = pb + 4 * compton::kPnetParams;
         pn.acc = pn.loss + 2;
-        pn.ticket = reinterpret_cast<uint32_t*>(pn.acc + compton::kPnetParams + 2);
+        pn.ticket = reinterpret_cast<uint32_t*>(pn.acc + compton::kPnetParams);
+        static_assert((5 * compton::kPnetParams + 3) % 2 == 0, "doubles on 8 bytes");
+        pn.acc_loss = reinterpret_cast<double*>(pn.acc + compton::kPnetParams + 1);
         pn.fs[0] = 1.0f;
         pn.fs[1] = 7.0f;
         pn.fs[2] = 1e-4f;

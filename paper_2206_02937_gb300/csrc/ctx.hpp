@@ -100,6 +100,7 @@ struct DeviceStats {
 // Surrogate network: 6 -> 64 -> 64 -> 64 -> 64 -> 1, parameter vector of
 // 12993 floats (W0 64x6, b0, W1 64x64, b1, W2, b2, W3, b3, W4 1x64, b4).
 constexpr int kMlpParams = 12993;
+constexpr size_t kMlpAccBytes = 4 * (kMlpParams + 1) + 2 * 8;  // MlpDev::acc, ticket and acc_loss, one after another
 __host__ __device__ constexpr int mlp_off_w(int l)
 {
     return l == 0 ? 0 : l == 1 ? 448 : l == 2 ? 4608 : l == 3 ? 8768 : 12928;
@@ -115,8 +116,10 @@ struct MlpDev {
     float* grad;         // [kMlpParams] gradient sums of the last step
     float* adam_m;       // [kMlpParams]
     float* adam_v;       // [kMlpParams]
-    float* acc;          // [kMlpParams + 2] sums of the step in flight (gradient, weighted |error|,
-                         // weights), zero between steps; nullptr without training
+    float* acc;          // [kMlpParams] gradient sums of the step in flight, zero between steps;
+                         // nullptr without training
+    double* acc_loss;    // [2] its weighted |error| and weights, likewise (FP64: hundreds of adds
+                         // into one number, in the order in which the blocks come)
     uint32_t* ticket;    // blocks of k_mlp_finish that have read the weight sum, zero between steps
     void* wbf16;         // 4 x 8 KB BF16 tiles, 128-byte swizzled K-major
     void* whalf;         // inference image: 4 x 8 KB BF16 tiles of W / 2 (layer 0 with b / 2 as
@@ -156,7 +159,8 @@ struct PnetDev {
     float* adam_m;  // [kPnetParams]
     float* adam_v;  // [kPnetParams]
     float* loss;    // [2] weighted |error| sum, weight sum of the last step
-    float* acc;     // [kPnetParams + 2] sums of the step in flight (gradient, then loss), zero between steps
+    float* acc;     // [kPnetParams] gradient sums of the step in flight, zero between steps
+    double* acc_loss;  // [2] its weighted |error| and weights, likewise
     uint32_t* ticket;  // blocks of the step in flight that have added their sums, zero between steps
     float fs[4];    // feature scales s_u, n_u, s_k, n_k
     float range[3]; // training range: gamma^2 max, eps^2 min, eps^2 max
@@ -206,7 +210,7 @@ struct compton_ctx {
     compton::MlpDev mlp{};
     bool mlp_loaded = false;
     int64_t adam_step = 0;
-    bool train_dirty = false;       // mlp.acc may hold the sums of a step that failed half-way
+    bool train_dirty = false;       // mlp.acc, acc_loss may hold the sums of a step that failed half-way
     float* r_buf = nullptr;         // [max_particles] network output per pair (surrogate modes)
     compton::ServeEngine* serve = nullptr;  // continuous-batching engine (compton_serve_start)
     compton::KernelTiming* timing = nullptr;  // per-kernel event pairs (compton_kernel_timing)

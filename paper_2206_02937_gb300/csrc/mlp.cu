@@ -163,14 +163,14 @@ __global__ void __launch_bounds__(kFinishThreads) k_mlp_finish(MlpDev m, AdamArg
     __shared__ float red[32];
     const int l = blockIdx.x, tid = threadIdx.x;
     float ws = 0.0f;
-    if (kAdam) ws = m.acc[kMlpParams + 1];
+    if (kAdam) ws = (float)m.acc_loss[1];
     if (l == 4) {
         if (tid < 64) m.w4[tid] = finish_param<kAdam>(m, ad, mlp_off_w(4) + tid, ws);
         if (tid == 64) m.b4[0] = finish_param<kAdam>(m, ad, mlp_off_b(4), ws);
         if (kAdam && tid == 65) {
-            m.loss[0] = m.acc[kMlpParams];
+            m.loss[0] = (float)m.acc_loss[0];
             m.loss[1] = ws;
-            m.acc[kMlpParams] = 0.0f;
+            m.acc_loss[0] = 0.0;
         }
     } else {
         float amax = 0.0f;
@@ -207,7 +207,7 @@ __global__ void __launch_bounds__(kFinishThreads) k_mlp_finish(MlpDev m, AdamArg
         // every thread of this CTA has read the weight sum
         __threadfence();
         if (atomicAdd(m.ticket, 1u) == gridDim.x - 1) {
-            m.acc[kMlpParams + 1] = 0.0f;
+            m.acc_loss[1] = 0.0;
             *m.ticket = 0u;
         }
     }

@@ -290,8 +290,8 @@ __global__ void __launch_bounds__(kTrThreads, 1) k_train_f32(TrainArgs a)
         }
         if ((tid & 31) == 0) {
             atomicAdd(&acc[mlp_off_b(4)], db4);
-            atomicAdd(&acc[kMlpParams], loss_num);
-            atomicAdd(&acc[kMlpParams + 1], wsum);
+            atomicAdd(&m.acc_loss[0], (double)loss_num);
+            atomicAdd(&m.acc_loss[1], (double)wsum);
         }
     }
 }
@@ -374,7 +374,7 @@ compton_status launch_mlp_train_step(compton_ctx* ctx, const float* ux, const fl
     // the accumulators are zero between steps (k_mlp_finish clears them); after
     // a step that failed between its two launches they are cleared here
     if (ctx->train_dirty)
-        COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.acc, 0, sizeof(float) * (kMlpParams + 2), stream));
+        COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->mlp.acc, 0, kMlpAccBytes, stream));
     ctx->train_dirty = true;
     compton_status st;
     if (ctx->train_tc) {

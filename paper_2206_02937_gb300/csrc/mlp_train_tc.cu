@@ -385,8 +385,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_train_tc(TrainTcArgs a)
             }
             if (lane == 0) {
                 atomicAdd(&m.acc[mlp_off_b(4)], db4);
-                atomicAdd(&m.acc[kMlpParams], loss_num);
-                atomicAdd(&m.acc[kMlpParams + 1], wsum);
+                atomicAdd(&m.acc_loss[0], (double)loss_num);
+                atomicAdd(&m.acc_loss[1], (double)wsum);
             }
         }
     }

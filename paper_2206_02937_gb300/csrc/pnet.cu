@@ -323,7 +323,8 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_pnet_train(PnetArgs a, flo
         }
         __syncthreads();
     }
-    if (tid < kTrainSums) atomicAdd(&a.p.acc[tid], sum);
+    if (tid < kPnetParams) atomicAdd(&a.p.acc[tid], sum);
+    else if (tid < kTrainSums) atomicAdd(&a.p.acc_loss[tid - kPnetParams], (double)sum);
     __threadfence();
     __syncthreads();
     if (tid == 0) last = atomicAdd(a.p.ticket, 1u) == gridDim.x - 1;
@@ -331,7 +332,7 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_pnet_train(PnetArgs a, flo
     if (!last) return;
     // the sums of every block are in acc: Adam (beta 0.9, 0.999) on the mean over the weights
     __threadfence();
-    const float wsum = __ldcg(&a.p.acc[kPnetParams + 1]);
+    const float wsum = (float)__ldcg(&a.p.acc_loss[1]);
     if (tid < kPnetParams) {
         const float gr = __ldcg(&a.p.acc[tid]) / wsum;
         a.p.grad[tid] = gr;
@@ -342,10 +343,11 @@ __global__ void __launch_bounds__(kTrainThreads, 1) k_pnet_train(PnetArgs a, flo
         const float mh = m / (1.0f - b1t), vh = v / (1.0f - b2t);
         a.p.theta[tid] -= lr * mh / (sqrtf(vh) + 1e-7f);
     } else if (tid < kTrainSums) {
-        a.p.loss[tid - kPnetParams] = __ldcg(&a.p.acc[tid]);
+        a.p.loss[tid - kPnetParams] = (float)__ldcg(&a.p.acc_loss[tid - kPnetParams]);
     }
     __syncthreads();
-    if (tid < kTrainSums) a.p.acc[tid] = 0.0f;
+    if (tid < kPnetParams) a.p.acc[tid] = 0.0f;
+    else if (tid < kTrainSums) a.p.acc_loss[tid - kPnetParams] = 0.0;
     if (tid == 0) *a.p.ticket = 0u;
 }
 
