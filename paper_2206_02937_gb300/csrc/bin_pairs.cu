@@ -36,16 +36,22 @@ constexpr int kCountThreads = 1024;  // threads per histogram CTA (256, 512: 1 u
 __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 
 // ---------------------------------------------------------------------------
-// Histogram and order check.  Every maximal run of equal in-range cell
-// indices at positions [i_s, i_e] adds i_e + 1 - i_s to its cell: the first
-// element adds -i_s, the last i_e + 1 (one atomic when they coincide).  This
-// counts any input exactly (a cell's runs sum to its size; int32 wrap-around
-// cancels), costs one atomic per element of shuffled input and two per run
-// of input in cell order.  Each thread takes four consecutive positions with
-// one vector load; the neighbours across threads come by shuffle.
+// Histogram and order check.  A warp walks one stretch of the positions, 128 at
+// a time, four per lane by one vector load; a run of equal cell indices begins
+// at the first of the 128 and wherever the index changes.  The lane that holds a
+// run's beginning adds its length to the cell: the end is the lane's next
+// beginning or, by one shuffle, the first one of a later lane.  So a position
+// costs its load and one comparison, and a lane repeats the rest for each
+// beginning it holds (one turn for most of input in cell order).
 // unsorted[s] counts the positions at which the cell index descends, plus one
 // per warp that saw an index outside [0, C): only if it is not zero does the
 // placement run, and by its size the placement takes its form (sort_source).
+//
+// What bounds it: instruction issue (113 instructions per 128 positions of input
+// in cell order; 140 when every position was looked at as first and last of its
+// run).  512^2 cells of 64 + 64: 36.0 us so before, 32.5 now (20 us of reads); a
+// tenth of them moved 78 and 71; 128^3 cells of 16 + 16 64.3 and 58.5; 301 x 257
+// cells of 40 + 40 in no order 49.3 and 49.2 (one atomic per position).
 // ---------------------------------------------------------------------------
 template <typename Idx>
 __device__ __forceinline__ int4 load_cells4(const int32_t* __restrict__ cell, Idx i, Idx n, bool vec)
@@ -62,7 +68,7 @@ __device__ __forceinline__ int4 load_cells4(const int32_t* __restrict__ cell, Id
 // Positions in Idx: 32-bit when every position the grid visits fits (the
 // launch checks), else 64-bit.
 template <typename Idx>
-__global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restrict__ cell_e, int64_t n_e,
+__global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_count(const int32_t* __restrict__ cell_e, int64_t n_e,
                                                         const int32_t* __restrict__ cell_g, int64_t n_g, int64_t C,
                                                         int32_t* __restrict__ count_e, int32_t* __restrict__ count_g,
                                                         uint32_t* __restrict__ unsorted, DeviceStats* stats)
@@ -72,75 +78,55 @@ __global__ void __launch_bounds__(kCountThreads) k_count(const int32_t* __restri
     const int32_t* __restrict__ cell = s == 0 ? cell_e : cell_g;
     const Idx n = (Idx)(s == 0 ? n_e : n_g);
     int32_t* __restrict__ count = s == 0 ? count_e : count_g;
-    const unsigned lane = lane_id();
-    const Idx stride = (Idx)gridDim.x * (Idx)blockDim.x * 4;
-    const Idx n_round = (n + 127) / 128 * 128;  // whole warps in every iteration
+    const unsigned lane = lane_id(), gt_mask = 0xfffffffeu << lane;
     const bool vec = (reinterpret_cast<uintptr_t>(cell) & 15u) == 0;
     // cell indices are int32, so C above 2^31 admits every non-negative one
     const uint32_t C32 = C > 0x80000000ll ? 0x80000000u : (uint32_t)C;
     uint32_t descents = 0;
     bool bad = false;
-    // the next group's loads are issued before this group is processed, so
-    // two groups per thread are in flight
-    auto edge = [&](Idx j0) -> int32_t {
-        if (lane == 0) return (j0 > 0 && j0 - 1 < n) ? cell[j0 - 1] : -1;
-        if (lane == 31) return j0 + 4 < n ? cell[j0 + 4] : -1;
-        return -1;
+    // a warp's positions lie one after another, so the cell index before its
+    // next 128 is the last of these; their load is in flight meanwhile
+    const int64_t n_groups = ((int64_t)n + 127) / 128, warps = (int64_t)gridDim.x * (kCountThreads / 32);
+    const int64_t w = (int64_t)blockIdx.x * (kCountThreads / 32) + (threadIdx.x >> 5);
+    Idx base = (Idx)(n_groups * w / warps) * 128;
+    const Idx stop = (Idx)(n_groups * (w + 1) / warps) * 128;  // (of whole groups)
+    // no index descends from the lowest value
+    int32_t before = base > 0 && base < stop ? cell[base - 1] : INT32_MIN;
+    auto load = [&](Idx at) {
+        if (vec && at + 128 <= n) return *reinterpret_cast<const int4*>(cell + at + 4 * (Idx)lane);
+        return load_cells4(cell, (Idx)(at + 4 * (Idx)lane), n, vec);
     };
-    Idx i0 = ((Idx)blockIdx.x * (Idx)blockDim.x + (Idx)threadIdx.x) * 4;
     int4 q = make_int4(-1, -1, -1, -1);
-    int32_t e = -1;
-    if (i0 < n_round) {
-        q = load_cells4(cell, i0, n, vec);
-        e = edge(i0);
-    }
-    for (; i0 < n_round; i0 += stride) {
-        int4 qn = make_int4(-1, -1, -1, -1);
-        int32_t en = -1;
-        if (i0 + stride < n_round) {
-            qn = load_cells4(cell, i0 + stride, n, vec);
-            en = edge(i0 + stride);
+    if (base < stop) q = load(base);
+    for (; base < stop; base += 128) {
+        const int4 v = q;
+        if (base + 128 < stop) q = load(base + 128);
+        const int32_t left = __shfl_up_sync(0xffffffffu, v.w, 1), prev = lane == 0 ? before : left;
+        // the lane's positions at which a run begins
+        uint32_t f = (lane == 0 || v.x != prev ? 1u : 0u) | (v.y != v.x ? 2u : 0u) | (v.z != v.y ? 4u : 0u) |
+                     (v.w != v.z ? 8u : 0u);
+        uint32_t end = 128u;
+        if (base + 128 > n) {  // the last positions of the array
+            end = (uint32_t)(n - base);
+            f &= 4u * lane >= end ? 0u : end - 4u * lane >= 4u ? 15u : (1u << (end - 4u * lane)) - 1u;
         }
-        const int32_t v[4] = {q.x, q.y, q.z, q.w};
-        int32_t prev = __shfl_up_sync(0xffffffffu, v[3], 1);
-        int32_t next = __shfl_down_sync(0xffffffffu, v[0], 1);
-        if (lane == 0) prev = e;
-        if (lane == 31) next = e;
-        q = qn;
-        e = en;
-        if (i0 > 0 && i0 + 4 < n) {
-            // interior group: no end of the array in reach, 32-bit positions
-            // (the counts wrap in int32 as in the general path)
-            const int32_t base = (int32_t)i0;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const int32_t c = v[j];
-                const int32_t pc = j == 0 ? prev : v[j - 1];
-                const int32_t nc = j == 3 ? next : v[j + 1];
-                const bool ok = (uint32_t)c < C32;
-                bad |= !ok;
-                descents += pc > c;
-                const bool first = pc != c, last = nc != c;
-                if (ok && (first || last))
-                    atomicAdd(&count[c], (last ? base + j + 1 : 0) - (first ? base + j : 0));
-            }
-            continue;
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            const Idx i = i0 + j;
-            if (i >= n) break;
-            const int32_t c = v[j];
-            const int32_t pc = j == 0 ? prev : v[j - 1];
-            const int32_t nc = j == 3 ? next : v[j + 1];
-            const bool ok = c >= 0 && (int64_t)c < C;
+        // where the lane's last run ends: the first beginning in a later lane
+        const unsigned later = __ballot_sync(0xffffffffu, f != 0u) & gt_mask;
+        const uint32_t first = __shfl_sync(0xffffffffu, 4u * lane + (uint32_t)__ffs((int)f) - 1u, __ffs((int)later) - 1);
+        const uint32_t stop_at = later ? first : end;
+        while (f) {
+            const uint32_t j = (uint32_t)__ffs((int)f) - 1u;
+            f &= f - 1u;
+            const int32_t c = j & 2u ? (j & 1u ? v.w : v.z) : (j & 1u ? v.y : v.x);
+            const int32_t from = j & 2u ? (j & 1u ? v.z : v.y) : (j & 1u ? v.x : prev);
+            const uint32_t len = (f ? 4u * lane + (uint32_t)__ffs((int)f) - 1u : stop_at) - 4u * lane - j;
+            const bool ok = (uint32_t)c < C32;
             bad |= !ok;
-            descents += i > 0 && pc > c;
-            const bool first = ok && (i == 0 || pc != c);
-            const bool last = ok && (i + 1 == n || nc != c);
-            if (first || last)
-                atomicAdd(&count[c], (last ? (int32_t)(i + 1) : 0) - (first ? (int32_t)i : 0));
+            descents += from > c;
+            if (ok) atomicAdd(&count[c], (int32_t)len);
         }
+        __syncwarp();
+        before = __shfl_sync(0xffffffffu, v.w, 31);  // (the last positions are alone partial)
     }
     const bool any_bad = __any_sync(0xffffffffu, bad);
     descents = __reduce_add_sync(0xffffffffu, descents);
@@ -170,8 +156,9 @@ __device__ __forceinline__ SortSource sort_source(uint32_t unsorted, int64_t n)
 // ---------------------------------------------------------------------------
 // Scan over cells, in three passes.  Values per cell: N_e, N_g, M = min.
 // ---------------------------------------------------------------------------
+// Sums fit 32 bits: a species has fewer than 2^31 particles.
 struct Tri {
-    int64_t e, g, m;
+    int32_t e, g, m;
 };
 
 __device__ __forceinline__ Tri tri_add(Tri a, Tri b) { return {a.e + b.e, a.g + b.g, a.m + b.m}; }
@@ -180,33 +167,39 @@ __device__ __forceinline__ Tri warp_incl_scan(Tri v)
 {
 #pragma unroll
     for (int d = 1; d < 32; d <<= 1) {
-        const int64_t e = __shfl_up_sync(0xffffffffu, v.e, d);
-        const int64_t g = __shfl_up_sync(0xffffffffu, v.g, d);
-        const int64_t m = __shfl_up_sync(0xffffffffu, v.m, d);
+        const int32_t e = __shfl_up_sync(0xffffffffu, v.e, d);
+        const int32_t g = __shfl_up_sync(0xffffffffu, v.g, d);
+        const int32_t m = __shfl_up_sync(0xffffffffu, v.m, d);
         if (lane_id() >= (unsigned)d) v = {v.e + e, v.g + g, v.m + m};
     }
     return v;
 }
 
-// Exclusive scan of one Tri per thread over a block of 256 threads; returns
-// the exclusive prefix and writes the block total to *total.
-__device__ __forceinline__ Tri block_excl_scan_256(Tri v, Tri* total)
+// Exclusive scan of one Tri per thread over a block of 256 threads.
+__device__ __forceinline__ Tri block_excl_scan_256(Tri v)
 {
     __shared__ Tri warp_tot[8];
     const Tri inc = warp_incl_scan(v);
     const int w = threadIdx.x >> 5;
     if (lane_id() == 31) warp_tot[w] = inc;
     __syncthreads();
-    if (w == 0) {
-        Tri t = lane_id() < 8 ? warp_tot[lane_id()] : Tri{0, 0, 0};
-        t = warp_incl_scan(t);
-        if (lane_id() < 8) warp_tot[lane_id()] = t;
-    }
-    __syncthreads();
-    const Tri before = w > 0 ? warp_tot[w - 1] : Tri{0, 0, 0};
-    *total = warp_tot[7];
-    __syncthreads();
+    Tri before{0, 0, 0};
+#pragma unroll
+    for (int t = 0; t < 7; ++t)
+        if (t < w) before = tri_add(before, warp_tot[t]);
     return {before.e + inc.e - v.e, before.g + inc.g - v.g, before.m + inc.m - v.m};
+}
+
+// Four consecutive counts from c0 (a multiple of 4) on, zeros past the end.
+static_assert(kScanPer == 4, "a vector of counts per thread");
+__device__ __forceinline__ int4 load_counts(const int32_t* __restrict__ count, int64_t c0, int64_t C)
+{
+    if (c0 + 3 < C) return *reinterpret_cast<const int4*>(count + c0);
+    int4 v = make_int4(0, 0, 0, 0);
+    if (c0 < C) v.x = count[c0];
+    if (c0 + 1 < C) v.y = count[c0 + 1];
+    if (c0 + 2 < C) v.z = count[c0 + 2];
+    return v;
 }
 
 __global__ void __launch_bounds__(256) k_scan_reduce(const int32_t* __restrict__ count_e,
@@ -215,21 +208,18 @@ __global__ void __launch_bounds__(256) k_scan_reduce(const int32_t* __restrict__
 {
     chain_start();
     const int64_t c0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPer;
-    Tri v{0, 0, 0};
-#pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-        const int64_t c = c0 + j;
-        if (c < C) {
-            const int64_t a = count_e[c], b = count_g[c];
-            v = tri_add(v, Tri{a, b, a < b ? a : b});
-        }
-    }
-    Tri total;
-    block_excl_scan_256(v, &total);
+    const int4 a = load_counts(count_e, c0, C), b = load_counts(count_g, c0, C);
+    Tri v{a.x + a.y + a.z + a.w, b.x + b.y + b.z + b.w, min(a.x, b.x) + min(a.y, b.y) + min(a.z, b.z) + min(a.w, b.w)};
+    __shared__ Tri warp_sum[8];
+    v = {__reduce_add_sync(0xffffffffu, v.e), __reduce_add_sync(0xffffffffu, v.g),
+         __reduce_add_sync(0xffffffffu, v.m)};
+    if (lane_id() == 0) warp_sum[threadIdx.x >> 5] = v;
+    __syncthreads();
     if (threadIdx.x == 0) {
-        block_sums[blockIdx.x] = total.e;
-        block_sums[n_tiles + blockIdx.x] = total.g;
-        block_sums[2 * n_tiles + blockIdx.x] = total.m;
+        for (int w = 1; w < 8; ++w) v = tri_add(v, warp_sum[w]);
+        block_sums[blockIdx.x] = v.e;
+        block_sums[n_tiles + blockIdx.x] = v.g;
+        block_sums[2 * n_tiles + blockIdx.x] = v.m;
     }
 }
 
@@ -293,40 +283,38 @@ struct ScanFinalArgs {
 
 // Sort tiles of a species whose first cell is c+1: every b >= 1 with
 // o < b*T <= o+n (the tile boundary lies inside or at the end of cell c).
-__device__ __forceinline__ void write_sort_tiles(int32_t* stile, int64_t nb, int64_t o, int64_t n, int64_t c)
+__device__ __forceinline__ void write_sort_tiles(int32_t* stile, int64_t nb, uint32_t o, uint32_t n, int64_t c)
 {
-    if (n <= 0) return;
-    const int64_t b_lo = o / kSortTile + 1;
-    int64_t b_hi = (o + n) / kSortTile;
-    if (b_hi > nb - 1) b_hi = nb - 1;
-    for (int64_t b = b_lo; b <= b_hi; ++b) stile[b] = (int32_t)(c + 1);
+    if (n == 0) return;
+    const uint32_t b_lo = o / kSortTile + 1;
+    uint32_t b_hi = (o + n) / kSortTile;
+    if (b_hi > nb - 1) b_hi = (uint32_t)(nb - 1);
+    for (uint32_t b = b_lo; b <= b_hi; ++b) stile[b] = (int32_t)(c + 1);
 }
 
-// The maps' entries of cell c: counts ne, ng, exclusive prefixes p, np_total pairs in all.
+// The maps' entries of cell c, except its offsets: counts ne, ng, exclusive prefixes p, np_total pairs in all.
 __device__ __forceinline__ void scan_cell(const ScanFinalArgs& a, int64_t c, int32_t ne, int32_t ng, const Tri& p,
                                           int64_t np_total)
 {
-    const int64_t m = ne < ng ? ne : ng;
-    a.off_e[c] = (int32_t)p.e;
-    a.off_g[c] = (int32_t)p.g;
-    const int64_t nmax = ne > ng ? ne : ng;
+    const uint32_t m = (uint32_t)(ne < ng ? ne : ng), end = (uint32_t)p.m + m;
+    const int32_t nmax = ne > ng ? ne : ng;
     CellInfo ci;
-    ci.pair_off = (int32_t)p.m;
-    ci.e_start = (int32_t)p.e;
-    ci.g_start = (int32_t)p.g;
+    ci.pair_off = p.m;
+    ci.e_start = p.e;
+    ci.g_start = p.g;
     ci.dens = (float)((double)nmax * a.w_over_v);
     a.cinfo[c] = ci;
     if (m > 0) {
         // scatter tiles whose first pair lies in [p.m, p.m + m)
-        for (int64_t t = (p.m + kPairsPerTile - 1) / kPairsPerTile; t * kPairsPerTile < p.m + m; ++t)
+        for (uint32_t t = ((uint32_t)p.m + kPairsPerTile - 1) / kPairsPerTile; t * kPairsPerTile < end; ++t)
             a.tile_cell[t] = (int32_t)c;
-        if (p.m + m == np_total) a.tile_cell[(np_total + kPairsPerTile - 1) / kPairsPerTile] = (int32_t)c;
+        if (end == np_total) a.tile_cell[(np_total + kPairsPerTile - 1) / kPairsPerTile] = (int32_t)c;
     }
-    write_sort_tiles(a.stile_e, a.nb_e, p.e, ne, c);
-    write_sort_tiles(a.stile_g, a.nb_g, p.g, ng, c);
+    write_sort_tiles(a.stile_e, a.nb_e, (uint32_t)p.e, (uint32_t)ne, c);
+    write_sort_tiles(a.stile_g, a.nb_g, (uint32_t)p.g, (uint32_t)ng, c);
     if (c == a.C - 1) {
-        a.off_e[a.C] = (int32_t)(p.e + ne);
-        a.off_g[a.C] = (int32_t)(p.g + ng);
+        a.off_e[a.C] = p.e + ne;
+        a.off_g[a.C] = p.g + ng;
     }
 }
 
@@ -341,75 +329,78 @@ __device__ __forceinline__ void scan_ends(const ScanFinalArgs& a)
 // The sums of the tiles before this block's, and the pairs of all tiles in
 // *total_m: each block adds them up itself, which takes it about as long as
 // waiting for one block's scan of them and saves that launch.
-__device__ __forceinline__ Tri tiles_before(const ScanFinalArgs& a, int64_t* total_m)
+__device__ __forceinline__ Tri tiles_before(const ScanFinalArgs& a, int32_t* total_m)
 {
-    __shared__ Tri warp_sum[8];
-    __shared__ int64_t warp_m[8];
-    Tri s{0, 0, 0};
-    int64_t tm = 0;
+    __shared__ int4 warp_sum[8];
+    int4 s = make_int4(0, 0, 0, 0);
     for (int64_t t = threadIdx.x; t < a.n_tiles; t += 256) {
-        const int64_t m = a.block_sums[2 * a.n_tiles + t];
-        tm += m;
-        if (t < (int64_t)blockIdx.x) s = tri_add(s, Tri{a.block_sums[t], a.block_sums[a.n_tiles + t], m});
+        const int32_t m = (int32_t)a.block_sums[2 * a.n_tiles + t];
+        s.w += m;
+        if (t < (int64_t)blockIdx.x) {
+            s.x += (int32_t)a.block_sums[t];
+            s.y += (int32_t)a.block_sums[a.n_tiles + t];
+            s.z += m;
+        }
     }
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        s.e += __shfl_xor_sync(0xffffffffu, s.e, d);
-        s.g += __shfl_xor_sync(0xffffffffu, s.g, d);
-        s.m += __shfl_xor_sync(0xffffffffu, s.m, d);
-        tm += __shfl_xor_sync(0xffffffffu, tm, d);
-    }
-    if (lane_id() == 0) {
-        warp_sum[threadIdx.x >> 5] = s;
-        warp_m[threadIdx.x >> 5] = tm;
-    }
+    s = make_int4(__reduce_add_sync(0xffffffffu, s.x), __reduce_add_sync(0xffffffffu, s.y),
+                  __reduce_add_sync(0xffffffffu, s.z), __reduce_add_sync(0xffffffffu, s.w));
+    if (lane_id() == 0) warp_sum[threadIdx.x >> 5] = s;
     __syncthreads();
-    s = warp_sum[0];
-    tm = warp_m[0];
-    for (int w = 1; w < 8; ++w) {
-        s = tri_add(s, warp_sum[w]);
-        tm += warp_m[w];
+    Tri sum{0, 0, 0};
+    int32_t tm = 0;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+        const int4 t = warp_sum[w];
+        sum = tri_add(sum, Tri{t.x, t.y, t.z});
+        tm += t.w;
     }
     *total_m = tm;
-    return s;
+    return sum;
 }
 
+// What bounds it: the stores of the maps (24 bytes per cell and the cleared
+// counts' 8) and, with few tiles, its chain of loads and barriers.  2 million
+// cells: 31 us with 64-bit sums and a load and a store per count, 21 us so.
 // kOwnPrefix: block_sums hold the tiles' sums (k_scan_blocks has not run).
 template <bool kOwnPrefix>
 __global__ void __launch_bounds__(256) k_scan_final(const __grid_constant__ ScanFinalArgs a)
 {
     chain_start();
     const int64_t c0 = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanPer;
-    int32_t ne[kScanPer], ng[kScanPer];
+    const int4 ce = load_counts(a.count_e, c0, a.C), cg = load_counts(a.count_g, c0, a.C);
+    const int32_t ne[kScanPer] = {ce.x, ce.y, ce.z, ce.w}, ng[kScanPer] = {cg.x, cg.y, cg.z, cg.w};
     Tri v{0, 0, 0};
 #pragma unroll
-    for (int j = 0; j < kScanPer; ++j) {
-        const int64_t c = c0 + j;
-        ne[j] = c < a.C ? a.count_e[c] : 0;
-        ng[j] = c < a.C ? a.count_g[c] : 0;
-        v = tri_add(v, Tri{ne[j], ng[j], ne[j] < ng[j] ? ne[j] : ng[j]});
-    }
-    Tri total;
-    Tri p = block_excl_scan_256(v, &total);
-    int64_t np_total;
+    for (int j = 0; j < kScanPer; ++j) v = tri_add(v, Tri{ne[j], ng[j], min(ne[j], ng[j])});
+    Tri p = block_excl_scan_256(v);
+    int32_t np_total;
     if (kOwnPrefix) {
         p = tri_add(p, tiles_before(a, &np_total));
         if (blockIdx.x == 0 && threadIdx.x == 0) *a.n_pairs = np_total;
     } else {
-        p = tri_add(p, Tri{a.block_sums[blockIdx.x], a.block_sums[a.n_tiles + blockIdx.x],
-                           a.block_sums[2 * a.n_tiles + blockIdx.x]});
-        np_total = *a.n_pairs;
+        p = tri_add(p, Tri{(int32_t)a.block_sums[blockIdx.x], (int32_t)a.block_sums[a.n_tiles + blockIdx.x],
+                           (int32_t)a.block_sums[2 * a.n_tiles + blockIdx.x]});
+        np_total = (int32_t)*a.n_pairs;
+    }
+    // offsets out; the counts become the insertion cursors of k_place
+    if (c0 + 3 < a.C) {
+        *reinterpret_cast<int4*>(a.off_e + c0) = make_int4(p.e, p.e + ce.x, p.e + ce.x + ce.y, p.e + ce.x + ce.y + ce.z);
+        *reinterpret_cast<int4*>(a.off_g + c0) = make_int4(p.g, p.g + cg.x, p.g + cg.x + cg.y, p.g + cg.x + cg.y + cg.z);
+        *reinterpret_cast<int4*>(a.count_e + c0) = make_int4(0, 0, 0, 0);
+        *reinterpret_cast<int4*>(a.count_g + c0) = make_int4(0, 0, 0, 0);
     }
 #pragma unroll
     for (int j = 0; j < kScanPer; ++j) {
         const int64_t c = c0 + j;
         if (c >= a.C) break;
+        if (c0 + 3 >= a.C) {
+            a.off_e[c] = p.e;
+            a.off_g[c] = p.g;
+            a.count_e[c] = 0;
+            a.count_g[c] = 0;
+        }
         scan_cell(a, c, ne[j], ng[j], p, np_total);
-        a.count_e[c] = 0;  // becomes the insertion cursor of k_place
-        a.count_g[c] = 0;
-        p.e += ne[j];
-        p.g += ng[j];
-        p.m += ne[j] < ng[j] ? ne[j] : ng[j];
+        p = tri_add(p, Tri{ne[j], ng[j], min(ne[j], ng[j])});
     }
     if (blockIdx.x == 0 && threadIdx.x == 0) scan_ends(a);
 }
@@ -527,6 +518,8 @@ __global__ void __launch_bounds__(kSmallThreads) k_bin_small(const __grid_consta
         const int c = c0 + j;
         if (c >= C) break;
         const Tri t{p.x, p.y, p.z};
+        f.off_e[c] = t.e;
+        f.off_g[c] = t.g;
         scan_cell(f, c, ne[j], ng[j], t, np_total);
         count[0][c] = p.x;
         count[1][c] = p.y;
@@ -1064,7 +1057,7 @@ __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(const __grid_c
 // taken here and launches chained.
 constexpr int64_t kOwnPrefixTiles = 512;
 
-// CTAs per SM and species of the grid-stride histogram (the launch's second
+// CTAs per SM and species of the histogram (the launch's second
 // grid dimension takes the two species), which runs in one wave of 1024-thread CTAs: 0.0394 ms on the 512^2 step against
 // 0.0404 with four and 0.0435 with eight.
 constexpr int kCountCtasPerSm = 2;
