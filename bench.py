@@ -36,11 +36,19 @@ L2_NOTE = "inputs larger than L2 (particle state ~1.3 GB resident, 129 MB L2)"
 # is now, scaled to a launch by its units; the profile file gives the command.
 # A kernel changed since its capture must be taken out of this table.
 MEASURED_TRAFFIC = {
-    "k_sort_gather": ((134.677504e6 + 111.480576e6) / 8372876, "particle",
+    "k_sort_gather": ((134.654976e6 + 111.112704e6) / 8372876, "particle",
                       "profiles/k_sort_gather_in_place_256x256.md"),
-    "k_count": (34.025472e6 / 8372876, "particle", "profiles/k_count_256x256.md"),
-    "k_pair_prob": ((97.137152e6 + 4.566784e6) / 4186438, "pair", "profiles/k_pair_prob_256x256.md"),
+    "k_count": (34.025216e6 / 8372876, "particle", "profiles/k_count_256x256.md"),
+    "k_pair_prob": ((97.116672e6 + 4.020480e6) / 4186438, "pair", "profiles/k_pair_prob_256x256.md"),
 }
+
+
+def step_launches(cells, particles, pairs):
+    """Kernels that a plain step launches: histogram, two scan kernels (a third above 512 tiles of 1024 cells),
+    placement and sort (a small call: one kernel and the sort), then probability and collisions (up to 32 tiles of
+    1024 pairs: one kernel)."""
+    small = cells <= 4096 and particles <= 16384
+    return (2 if small else 5 + (cells > 512 * 1024)) + (1 if pairs <= 32 * 1024 else 2)
 
 
 def parse():
@@ -292,8 +300,9 @@ def run_ours(args, rank: int, world: int, local_rank: int):
 
     # per-kernel device times: the same steps once more with the library's
     # event timing on (kept out of the headline region above).  The library
-    # keeps the last 64 launches of each kernel slot and the scan slot
-    # launches three kernels per step, so 20 steps keep every launch.
+    # keeps the last 64 timed scopes of each kernel slot and a step opens one
+    # per slot (the scan's covers its two or three kernels), so 20 steps keep
+    # every one.
     kt_steps = min(args.steps, 20)
     cg.compton_kernel_timing(ctx, True)
     for i in range(kt_steps):
@@ -384,7 +393,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
            "candidates_per_s": st_ntc["pairs_tested"] / args.steps / (ntc_ms * 1e-3),
            "collisions_per_step": st_ntc["scatters"] / args.steps,
            "collision_ratio_ntc_to_pairing_same_state": same["ntc"] / max(1, same["pairing"]),
-           "note": "bin + NTC candidates per cell (each cell's candidates in order: cells of 32 or more a warp each, the others a lane each from a shared queue); the ratio "
+           "note": "bin + NTC candidates per cell (each cell's candidates in order: a stream of candidates per warp, collisions 32 at a time); the ratio "
                    "compares both schemes on the same binned particles over 3 draws (NTC uses the linear "
                    "probability, pairing 1 - exp(-a): expected about 1 + n dt <s v>/2)"}
 
@@ -445,7 +454,7 @@ def run_ours(args, rank: int, world: int, local_rank: int):
             "roofline_bin_shuffled": {"bound": "hbm", "achieved": achieved_bin_shuf, "peak": hbm_peak,
                                       "unit": "GB/s", "frac": achieved_bin_shuf / hbm_peak,
                                       "algorithmic_bytes_per_launch": bytes_bin_shuf, "input": "shuffled"},
-            "gpu_launches": 8 * args.steps,
+            "gpu_launches": step_launches(w.n_cells, w.n_e + w.n_g, min(w.n_e, w.n_g)) * args.steps,
             "clocks": clk.summary(),
             "cpu_baseline": cpu, "cpu_baseline_all_cores": cpu_all,
             "e2e": e2e,
@@ -1198,7 +1207,8 @@ def run_c5(args, rank: int, world: int, local_rank: int):
                        "mode": "plain (headline); sweep of the surrogate in FP32/BF16/FP8",
                        "l2": "inputs larger than L2", "generate_s": t_gen},
             "pairs_per_step": stats["pairs_tested"] / args.steps,
-            "clocks": clk.summary(), "cpu_baseline": cpu, "gpu_launches": 8 * args.steps,
+            "clocks": clk.summary(), "cpu_baseline": cpu,
+            "gpu_launches": step_launches(args.c5_side ** 3, 32 * args.c5_side ** 3, 16 * args.c5_side ** 3) * args.steps,
             "precision_sweep": sweep, "train": train,
             "spectrum_note": "L1 distance of normalised 64-bin log10(eps) histograms (eps in [1e-5, 1e5]) of the "
                              "photons that scattered; vs plain over all pairs, vs the FP64 oracle over the subsample",

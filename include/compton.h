@@ -500,7 +500,7 @@ compton_status compton_cell_offsets_noalloc(const int32_t* cell_dev, int64_t n, 
 /* Kernel slots of compton_kernel_times. */
 typedef enum compton_kernel_slot {
     COMPTON_K_COUNT = 0,   /* histogram and order check                    */
-    COMPTON_K_SCAN = 1,    /* the three scan kernels together              */
+    COMPTON_K_SCAN = 1,    /* the scan kernels together                    */
     COMPTON_K_PLACE = 2,   /* keyed placement (shuffled input)             */
     COMPTON_K_SORT = 3,    /* per-cell sort and sorted copy                */
     COMPTON_K_PROB = 4,    /* probability and Bernoulli trial of all pairs */

@@ -3,8 +3,8 @@
 // cells, in which the particles are binned; from this binning a list of
 // colliding leptons and photons is produced for each cell").
 //
-// Six launches per call, both species in each (a small call: k_bin_small, which
-// does all before the sort in one, and the sort):
+// Five launches per call (six above 512 scan tiles), both species in each (a
+// small call: k_bin_small, which does all before the sort in one, and the sort):
 //   k_count        histogram of cell indices by run boundaries, order check
 //   k_scan_reduce  per-tile sums of N_e,c, N_g,c and M_c = min(N_e,c, N_g,c)
 //   k_scan_blocks  exclusive scan of the tile sums (one CTA; many cells only)

@@ -14,13 +14,14 @@
 //                inputs zero-padded to K = 64), FP8 E4M3 tiles (K padded to 128)
 //                with per-tensor scales, transposed FP32 copies for the CUDA
 //                core path, biases and the output layer.
-//   k_mlp_bf16   tcgen05 forward: 128 samples per tile, one row per thread;
+//   k_mlp_ta     BF16 forward on tcgen05: 128 samples per tile, one row per thread;
 //                per hidden layer four 128x64x16 BF16 MMAs into a 64-column
-//                FP32 TMEM accumulator, then bias + SiLU in registers and the
-//                BF16 activations written back to shared memory as the next
-//                layer's A operand; the 64 -> 1 output layer on the CUDA cores.
-//   k_mlp_fp8    the same with E4M3 operands (kind::f8f6f4, K = 32 per MMA)
-//                and per-tensor scales, FP32 accumulation.
+//                FP32 TMEM accumulator, then SiLU in registers and the BF16
+//                activations written to TMEM as the next layer's A operand;
+//                the 64 -> 1 output layer on the CUDA cores.
+//   k_mlp_tc     the same with the A operand in shared memory: E4M3 operands
+//                (kind::f8f6f4, K = 32 per MMA) and per-tensor scales, FP32
+//                accumulation; or BF16.
 //   k_mlp_fp32   FP32 forward on the CUDA cores (reference precision).
 #include <cuda_bf16.h>
 #include <cuda_fp8.h>

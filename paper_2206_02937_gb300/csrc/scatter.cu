@@ -5,7 +5,8 @@
 // updated; Sec. 3.2: the probability comes from the Klein-Nishina cross
 // section in the lepton rest frame, carried back to the simulation frame).
 //
-// Two kernels per step:
+// Two kernels per step (up to 32 pair tiles one: k_pair_prob then resolves its
+// own accepted pairs):
 //   k_pair_prob  persistent CTAs (four per SM) of eight independent warps:
 //                each warp owns a contiguous run of 128-pair chunks (32 lanes
 //                x 4 consecutive pairs, one Philox block per lane for the
