@@ -74,6 +74,7 @@ constexpr int kSiluFmaPairs = 1;
 // BF16 on k_mlp_ta (the A operand in tensor memory) instead of k_mlp_tc<false>.
 constexpr bool kBf16TmemA = true;
 
+__device__ __forceinline__ float silu_exact(float z) { return z / (1.0f + expf(-z)); }
 __device__ __forceinline__ float sigmoid_exact(float z) { return 1.0f / (1.0f + expf(-z)); }
 
 __device__ __forceinline__ uint32_t pack_bf16x2(float lo, float hi)
@@ -910,7 +911,15 @@ __global__ void __launch_bounds__(kF32Threads, 1) k_mlp_fp32(MlpArgs a)
             for (int p = 0; p < 8; ++p) {
                 float v[8];
 #pragma unroll
-                for (int q = 0; q < 4; ++q) act::upk2(act::silu2_f32(acc[p][q]), v[2 * q], v[2 * q + 1]);
+                for (int q = 0; q < 4; ++q) {
+                    if (kCalib) {  // the scales' last bits decide FP8 roundings: SiLU by the library's functions
+                        act::upk2(acc[p][q], v[2 * q], v[2 * q + 1]);
+                        v[2 * q] = silu_exact(v[2 * q]);
+                        v[2 * q + 1] = silu_exact(v[2 * q + 1]);
+                    } else {
+                        act::upk2(act::silu2_f32(acc[p][q]), v[2 * q], v[2 * q + 1]);
+                    }
+                }
                 if (kCalib && l < 3) {
 #pragma unroll
                     for (int q = 0; q < 8; ++q)
