@@ -454,14 +454,19 @@ compton_status compton_serve_stop(struct compton_ctx* ctx);
 /* Queue a request; returns at once with a ticket.  The engine admits it when
  * a block of the pool fits it and runs its tiles together with the other
  * admitted requests.  The caller keeps the input and output arrays alive and
- * unchanged until compton_poll returns OK.  ERANGE if the request can never
- * fit the pool, EBUSY if the queue is full (retry), ENOMODEL for a surrogate
- * mode without a network.  Thread-safe. */
+ * unchanged until compton_poll returns anything but ENOTREADY.  ERANGE if the
+ * request can never fit the pool, EBUSY if the queue is full (retry),
+ * ENOMODEL for a surrogate mode without a network.  Thread-safe. */
 compton_status compton_submit(struct compton_ctx* ctx, const compton_request* req, uint64_t* ticket);
 
-/* ENOTREADY until the request's outputs are written, then OK with *out
- * filled (the ticket is retired).  EINVAL for an unknown ticket.
- * Thread-safe. */
+/* ENOTREADY until the request has ended, then its status, with *out filled
+ * (the ticket is retired): OK with its outputs written, or ECUDA if the
+ * engine could not run it.  A launch of the engine that fails ends its own
+ * requests and all that are unfinished with the error, none of them before
+ * its work in flight has ended; the outputs of such a request (an in-place
+ * one's inputs with them) are undefined, and compton_submit returns the error
+ * until the engine is stopped and started again.  EINVAL for an unknown
+ * ticket.  Thread-safe. */
 compton_status compton_poll(struct compton_ctx* ctx, uint64_t ticket, compton_result* out);
 
 /* Pool bytes in use now, the peak since start, and the pool size. */

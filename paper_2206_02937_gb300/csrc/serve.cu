@@ -11,7 +11,10 @@
 //                     launches the pending tiles (1024 pairs each) of every
 //                     admitted request together; when a launch completes,
 //                     requests whose tiles are all done are finished and their
-//                     blocks freed.  Up to two launches are in flight.
+//                     blocks freed.  Up to two launches are in flight.  After
+//                     a launch that failed nothing more is launched: its
+//                     requests and the unfinished others end with the error,
+//                     each once nothing of it is in flight.
 //   compton_poll      returns ENOTREADY or the request's result.
 //
 // A launch is k_serve over its tiles, then, for the surrogate requests' candidates,
@@ -321,6 +324,7 @@ struct ServeReq {
     uint64_t ticket = 0;
     compton_request req{};
     int64_t tiles = 0, launched = 0, done_tiles = 0;
+    int64_t flying = 0;  // tiles in launches that are not retired
     std::vector<TileDev> again;  // tiles a full candidate list turned away
     int state = 0;  // 0 queued, 1 admitted, 4 done
     size_t off = 0, bytes = 0;
@@ -331,8 +335,10 @@ struct ServeReq {
 };
 
 struct Launch {
-    cudaEvent_t ev;
-    int ring;
+    cudaEvent_t ev = nullptr;
+    int ring = 0;
+    compton_status status = COMPTON_OK;      // of every request in it
+    compton_status net_status = COMPTON_OK;  // of its surrogate requests
     std::vector<std::pair<uint64_t, int64_t>> tiles_per_req;  // ticket, tiles in this launch
 };
 
@@ -429,13 +435,22 @@ bool overlaps_inputs(const compton_request& r)
     return false;
 }
 
+// A CUDA call of the engine: its failure ends the serving.
+bool note(ServeEngine* E, cudaError_t e)
+{
+    if (e == cudaSuccess) return true;
+    cudaGetLastError();
+    E->fatal = set_cuda_error(E->ctx, e, "serve engine");
+    return false;
+}
+
 // Admit queued requests in arrival order while blocks fit (a request that
 // does not fit waits; later, smaller ones may pass it).
 void admit(ServeEngine* E)
 {
     for (auto it = E->queued.begin(); it != E->queued.end();) {
         ServeReq& R = E->reqs[*it];
-        if (E->free_slots.empty()) break;
+        if (E->free_slots.empty() || E->fatal != COMPTON_OK) break;
         size_t off;
         if (!pool_alloc(E, R.bytes, &off)) {
             ++it;
@@ -459,7 +474,8 @@ void admit(ServeEngine* E)
             for (int c = 0; c < 7; ++c) {
                 const float* from = c < 6 ? src[c] : R.req.n_dens_dev;
                 if (!from) continue;
-                cudaMemcpyAsync(base + (size_t)c * n, from, n * sizeof(float), cudaMemcpyDeviceToDevice, E->s_compute);
+                note(E, cudaMemcpyAsync(base + (size_t)c * n, from, n * sizeof(float), cudaMemcpyDeviceToDevice,
+                                        E->s_compute));
                 if (c < 6) src[c] = base + (size_t)c * n;
                 else d.dens = base + (size_t)c * n;
             }
@@ -492,13 +508,71 @@ double expected_candidates(const compton_request& r, double dt, double pairs)
     return pairs * (share < 1.0 ? share : 1.0);
 }
 
+// The launch's table, tiles and k_serve.
+compton_status launch_serve(ServeEngine* E, const TileDev* th, TileDev* td, int nt)
+{
+    compton_ctx* ctx = E->ctx;
+    const compton_config& cfg = ctx->cfg;
+    cudaStream_t s = E->s_compute;
+    if (E->new_hi >= 0) {
+        COMPTON_CUDA_TRY(ctx, cudaMemcpyAsync(E->reqs_dev + E->new_lo, E->reqs_host + E->new_lo,
+                                              sizeof(ReqDev) * (E->new_hi - E->new_lo + 1), cudaMemcpyHostToDevice, s));
+        E->new_hi = -1;
+    }
+    COMPTON_CUDA_TRY(ctx, cudaMemcpyAsync(td, th, nt * sizeof(TileDev), cudaMemcpyHostToDevice, s));
+    COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(E->ctl_dev, 0, offsetof(ServeControl, rejected), s));
+    const int grid = std::min(nt, ctx->n_sm * 3);
+    k_serve<<<grid, kServeThreads, 0, s>>>(E->reqs_dev, td, nt, (float)cfg.dt, cfg.gamma_fp64_threshold,
+                                           cfg.collide_fp64_threshold * cfg.collide_fp64_threshold, ctx->stats,
+                                           E->list.cand, E->ctl_dev);
+    COMPTON_LAUNCH_CHECK(ctx, "k_serve");
+    return COMPTON_OK;
+}
+
+// The network, the decisions and the collisions of the launch's candidates,
+// about `rows` of them (a full list at most).
+compton_status launch_candidates(ServeEngine* E, int mode, int64_t rows)
+{
+    compton_ctx* ctx = E->ctx;
+    const compton_config& cfg = ctx->cfg;
+    cudaStream_t s = E->s_compute;
+    const MlpDecide dec{(float)cfg.dt, cfg.gamma_fp64_threshold, nullptr, nullptr, false};
+    const bool fused = mode != COMPTON_MODE_MLP_FP32;
+    compton_status st = launch_mlp_infer(ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, rows,
+                                         (compton_mode)mode, E->list.r, s, false, false, fused ? &dec : nullptr,
+                                         &E->list);
+    if (st == COMPTON_OK && !fused) st = launch_decide(ctx, E->list, rows, s);
+    if (st != COMPTON_OK) return st;
+    const int rgrid = (int)std::min<int64_t>((rows + 255) / 256, (int64_t)ctx->n_sm * 8);
+    k_serve_resolve<<<rgrid, 256, 0, s>>>(E->reqs_dev, E->list.accepted, E->ctl_dev, cfg.gamma_fp64_threshold,
+                                          cfg.collide_fp64_threshold * cfg.collide_fp64_threshold);
+    COMPTON_LAUNCH_CHECK(ctx, "k_serve_resolve");
+    return COMPTON_OK;
+}
+
+// The counters and the tiles turned away, to the host, and the launch's event.
+compton_status launch_results(ServeEngine* E, Launch& L, int nt)
+{
+    compton_ctx* ctx = E->ctx;
+    cudaStream_t s = E->s_compute;
+    COMPTON_CUDA_TRY(ctx, cudaMemcpyAsync(E->ctl_host + L.ring, E->ctl_dev,
+                                          offsetof(ServeControl, rejected) + nt * sizeof(int32_t),
+                                          cudaMemcpyDeviceToHost, s));
+    int hi = 0;
+    for (const auto& tr : L.tiles_per_req) hi = std::max(hi, E->reqs[tr.first].dslot);
+    COMPTON_CUDA_TRY(ctx, cudaMemcpyAsync(E->scat_host + (size_t)L.ring * E->max_active, E->counters,
+                                          sizeof(unsigned long long) * (hi + 1), cudaMemcpyDeviceToHost, s));
+    COMPTON_CUDA_TRY(ctx, cudaEventCreateWithFlags(&L.ev, cudaEventDisableTiming));
+    COMPTON_CUDA_TRY(ctx, cudaEventRecord(L.ev, s));
+    return COMPTON_OK;
+}
+
 void launch_tiles(ServeEngine* E)
 {
-    if (E->active.empty()) return;
+    if (E->active.empty() || E->fatal != COMPTON_OK) return;
     const compton_config& cfg = E->ctx->cfg;
     TileDev* th = E->tiles_host + (size_t)E->ring * kMaxTilesPerLaunch;
     TileDev* td = E->tiles_dev + (size_t)E->ring * kMaxTilesPerLaunch;
-    ServeControl* ch = E->ctl_host + E->ring;
     int nt = 0;
     Launch L;
     L.ring = E->ring;
@@ -530,80 +604,93 @@ void launch_tiles(ServeEngine* E)
             }
         }
         if (take) L.tiles_per_req.emplace_back(ticket, take);
+        R.flying += take;
         if (R.launched < R.tiles || !R.again.empty()) rest.push_back(ticket);
     }
     E->active.swap(rest);
     if (nt == 0) return;
-    cudaStream_t s = E->s_compute;
-    if (E->new_hi >= 0) {
-        cudaMemcpyAsync(E->reqs_dev + E->new_lo, E->reqs_host + E->new_lo,
-                        sizeof(ReqDev) * (E->new_hi - E->new_lo + 1), cudaMemcpyHostToDevice, s);
-        E->new_hi = -1;
-    }
-    cudaMemcpyAsync(td, th, nt * sizeof(TileDev), cudaMemcpyHostToDevice, s);
-    cudaMemsetAsync(E->ctl_dev, 0, offsetof(ServeControl, rejected), s);
-    const int grid = std::min(nt, E->ctx->n_sm * 3);
-    const float c64sq = cfg.collide_fp64_threshold * cfg.collide_fp64_threshold;
-    k_serve<<<grid, kServeThreads, 0, s>>>(E->reqs_dev, td, nt, (float)cfg.dt, cfg.gamma_fp64_threshold, c64sq,
-                                           E->ctx->stats, E->list.cand, E->ctl_dev);
-    if (mode != COMPTON_MODE_PLAIN) {
-        const MlpDecide dec{(float)cfg.dt, cfg.gamma_fp64_threshold, nullptr, nullptr, false};
-        const bool fused = mode != COMPTON_MODE_MLP_FP32;
+    L.status = launch_serve(E, th, td, nt);
+    if (L.status == COMPTON_OK && mode != COMPTON_MODE_PLAIN)
         // the grids are sized for the list the host expects, at most a full one
-        const int64_t rows = (int64_t)std::min<double>(kServeListCap, 1.2 * cand + 4096.0);
-        compton_status st = launch_mlp_infer(E->ctx, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, rows,
-                                             (compton_mode)mode, E->list.r, s, false, false, fused ? &dec : nullptr,
-                                             &E->list);
-        if (st == COMPTON_OK && !fused) st = launch_decide(E->ctx, E->list, rows, s);
-        if (st != COMPTON_OK) E->fatal = st;
-        const int rgrid = (int)std::min<int64_t>((rows + 255) / 256, (int64_t)E->ctx->n_sm * 8);
-        k_serve_resolve<<<rgrid, 256, 0, s>>>(E->reqs_dev, E->list.accepted, E->ctl_dev, cfg.gamma_fp64_threshold,
-                                              c64sq);
+        L.net_status = launch_candidates(E, mode, (int64_t)std::min<double>(kServeListCap, 1.2 * cand + 4096.0));
+    if (L.status == COMPTON_OK) L.status = launch_results(E, L, nt);
+    if (L.status != COMPTON_OK) {
+        // no event to wait for: everything before has to end here
+        cudaStreamSynchronize(E->s_compute);
+        cudaGetLastError();
+        E->fatal = L.status;
+    } else if (L.net_status != COMPTON_OK) {
+        E->fatal = L.net_status;
     }
-    // the counters, and the tiles turned away
-    cudaMemcpyAsync(ch, E->ctl_dev, offsetof(ServeControl, rejected) + nt * sizeof(int32_t), cudaMemcpyDeviceToHost, s);
-    int hi = 0;
-    for (const auto& tr : L.tiles_per_req) hi = std::max(hi, E->reqs[tr.first].dslot);
-    cudaMemcpyAsync(E->scat_host + (size_t)E->ring * E->max_active, E->counters, sizeof(unsigned long long) * (hi + 1),
-                    cudaMemcpyDeviceToHost, s);
-    cudaEventCreateWithFlags(&L.ev, cudaEventDisableTiming);
-    cudaEventRecord(L.ev, s);
     E->inflight.push_back(std::move(L));
     E->ring = (E->ring + 1) % kTileRing;
 }
 
+// A request's end: its block and slot are given back, its result is ready.
+void finish(ServeEngine* E, ServeReq& R, compton_status status)
+{
+    R.state = 4;
+    R.status = status;
+    R.t_done = now_s();
+    if (R.dslot >= 0) {
+        pool_free(E, R.off, R.bytes);
+        E->free_slots.push_back(R.dslot);
+        R.dslot = -1;
+    } else {
+        R.t_admit = R.t_done;
+    }
+}
+
 void retire(ServeEngine* E)
 {
-    while (!E->inflight.empty() && cudaEventQuery(E->inflight.front().ev) == cudaSuccess) {
+    while (!E->inflight.empty()) {
         Launch& L = E->inflight.front();
+        const cudaError_t q = L.ev ? cudaEventQuery(L.ev) : cudaSuccess;
+        if (q == cudaErrorNotReady) break;
+        if (!note(E, q)) L.status = E->fatal;
+        const bool read = L.status == COMPTON_OK;  // the launch's counters are on the host
         ServeControl* ch = E->ctl_host + L.ring;
+        const uint32_t n_rejected = read ? ch->n_rejected : 0;
         const TileDev* th = E->tiles_host + (size_t)L.ring * kMaxTilesPerLaunch;
         std::unordered_map<int, int64_t> turned_away;  // slot -> tiles
-        for (uint32_t i = 0; i < ch->n_rejected; ++i) ++turned_away[th[ch->rejected[i]].req];
+        for (uint32_t i = 0; i < n_rejected; ++i) ++turned_away[th[ch->rejected[i]].req];
         for (auto& tr : L.tiles_per_req) {
             ServeReq& R = E->reqs[tr.first];
+            const compton_status st = L.status == COMPTON_OK && R.req.mode != COMPTON_MODE_PLAIN ? L.net_status : L.status;
+            if (R.status == COMPTON_OK) R.status = st;
             const auto it = turned_away.find(R.dslot);
             const int64_t away = it == turned_away.end() ? 0 : it->second;
+            R.flying -= tr.second;
             R.done_tiles += tr.second - away;
             if (away) {
                 if (R.launched == R.tiles && R.again.empty()) E->active.push_back(R.ticket);
-                for (uint32_t i = 0; i < ch->n_rejected; ++i)
+                for (uint32_t i = 0; i < n_rejected; ++i)
                     if (th[ch->rejected[i]].req == R.dslot) R.again.push_back(th[ch->rejected[i]]);
             }
             if (R.done_tiles == R.tiles) {
-                R.state = 4;
-                R.t_done = now_s();
-                const unsigned long long count = E->scat_host[(size_t)L.ring * E->max_active + R.dslot];
-                R.scatters = count - E->scat_base[R.dslot];
-                E->scat_base[R.dslot] = count;
-                pool_free(E, R.off, R.bytes);
-                E->free_slots.push_back(R.dslot);
-                R.dslot = -1;
+                if (read) {
+                    const unsigned long long count = E->scat_host[(size_t)L.ring * E->max_active + R.dslot];
+                    R.scatters = count - E->scat_base[R.dslot];
+                    E->scat_base[R.dslot] = count;
+                }
+                finish(E, R, R.status);
             }
         }
-        cudaEventDestroy(L.ev);
+        if (L.ev) cudaEventDestroy(L.ev);
         E->inflight.pop_front();
     }
+    if (E->fatal == COMPTON_OK) return;
+    // nothing more is launched: the other requests end as well, those with
+    // tiles in flight when these are retired
+    for (const uint64_t ticket : E->queued) finish(E, E->reqs[ticket], E->fatal);
+    E->queued.clear();
+    std::deque<uint64_t> rest;
+    for (const uint64_t ticket : E->active) {
+        ServeReq& R = E->reqs[ticket];
+        if (R.flying > 0) rest.push_back(ticket);
+        else finish(E, R, R.status != COMPTON_OK ? R.status : E->fatal);
+    }
+    E->active.swap(rest);
 }
 
 void engine_loop(ServeEngine* E)
@@ -615,11 +702,6 @@ void engine_loop(ServeEngine* E)
         retire(E);
         admit(E);
         if (E->inflight.size() < 2) launch_tiles(E);
-        cudaError_t err = cudaGetLastError();
-        if (err != cudaSuccess) {
-            set_cuda_error(E->ctx, err, "serve engine");
-            E->fatal = COMPTON_ECUDA;
-        }
         const bool busy = !E->inflight.empty() || !E->queued.empty() || !E->active.empty();
         if (busy) {
             lk.unlock();
@@ -689,7 +771,8 @@ void serve_stop_free(ServeEngine* E)
     if (E->ctl_dev) cudaFree(E->ctl_dev);
     if (E->ctl_host) cudaFreeHost(E->ctl_host);
     if (E->s_compute) cudaStreamDestroy(E->s_compute);
-    for (auto& L : E->inflight) cudaEventDestroy(L.ev);
+    for (auto& L : E->inflight)
+        if (L.ev) cudaEventDestroy(L.ev);
     delete E;
 }
 
@@ -739,13 +822,14 @@ compton_status serve_poll(compton_ctx* ctx, uint64_t ticket, compton_result* out
     auto it = E->reqs.find(ticket);
     if (it == E->reqs.end()) return COMPTON_EINVAL;
     ServeReq& R = it->second;
-    if (R.state != 4) return E->fatal != COMPTON_OK ? E->fatal : COMPTON_ENOTREADY;
-    out->status = R.status;
+    if (R.state != 4) return COMPTON_ENOTREADY;
+    const compton_status st = R.status;
+    out->status = st;
     out->scatters = R.scatters;
     out->latency_s = R.t_done - R.t_submit;
     out->queue_s = R.t_admit - R.t_submit;
     E->reqs.erase(it);
-    return COMPTON_OK;
+    return st;
 }
 
 compton_status serve_info(compton_ctx* ctx, uint64_t* in_use, uint64_t* peak, uint64_t* pool)
