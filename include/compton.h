@@ -447,8 +447,10 @@ typedef struct compton_result {
  * once, with 29 MB of the engine's own lists.  EINVAL if already started. */
 compton_status compton_serve_start(struct compton_ctx* ctx, uint64_t pool_bytes, int32_t max_active);
 
-/* Stop the engine after the work in flight; requests not yet done are
- * dropped.  compton_destroy calls it. */
+/* Stop the engine.  Requests whose work has begun are finished first; the
+ * others are dropped, their arrays as they were (an in-place request is either
+ * done or untouched, unless the engine failed, see compton_poll).  No ticket
+ * can be polled afterwards.  compton_destroy calls it. */
 compton_status compton_serve_stop(struct compton_ctx* ctx);
 
 /* Queue a request; returns at once with a ticket.  The engine admits it when

@@ -14,7 +14,9 @@
 //                     blocks freed.  Up to two launches are in flight.  After
 //                     a launch that failed nothing more is launched: its
 //                     requests and the unfinished others end with the error,
-//                     each once nothing of it is in flight.
+//                     each once nothing of it is in flight.  When the engine
+//                     is stopped, a request with tiles launched is finished (its
+//                     outputs are partly written), the others are dropped.
 //   compton_poll      returns ENOTREADY or the request's result.
 //
 // A launch is k_serve over its tiles, then, for the surrogate requests' candidates,
@@ -698,9 +700,18 @@ void engine_loop(ServeEngine* E)
     cudaSetDevice(E->device);
     prctl(PR_SET_TIMERSLACK, 1000);  // the 20 us sleeps below: wake within a microsecond of them
     std::unique_lock<std::mutex> lk(E->mu);
-    while (!E->stop) {
+    for (;;) {
         retire(E);
-        admit(E);
+        if (E->stop) {
+            E->queued.clear();
+            std::deque<uint64_t> begun;
+            for (const uint64_t ticket : E->active)
+                if (E->reqs[ticket].launched > 0) begun.push_back(ticket);
+            E->active.swap(begun);
+            if (E->inflight.empty() && E->active.empty()) break;
+        } else {
+            admit(E);
+        }
         if (E->inflight.size() < 2) launch_tiles(E);
         const bool busy = !E->inflight.empty() || !E->queued.empty() || !E->active.empty();
         if (busy) {

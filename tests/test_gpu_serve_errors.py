@@ -1,6 +1,7 @@
 """Serving when a launch of the engine fails (injected on the host, nothing is
 done to the device): no request of it is reported OK, the engine refuses work
-until it is started again, and then gives the direct call's results."""
+until it is started again, and then gives the direct call's results.  And the
+engine stopped with requests unfinished: each of them is done or untouched."""
 import time
 
 import pytest
@@ -112,5 +113,33 @@ def test_the_other_requests_end_too():
             if st == 0:
                 assert torch.equal(uo, ref[0]) and torch.equal(ko, ref[1])
         assert cg.compton_serve_info(ctx)["in_use"] == 0
+    finally:
+        cg.compton_destroy(ctx)
+
+
+@pytest.mark.parametrize("pause", [0.0, 2e-4, 5e-4, 1e-3, 2e-3])
+def test_stop_leaves_in_place_requests_done_or_untouched(pause):
+    """Requests of several launches each (every pair a candidate, more of them
+    than a launch's list holds), in place; more than the pool admits at once."""
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    cg.build()
+    n, dens = 700001, 200.0
+    ctx = _ctx(cg, n)
+    try:
+        jobs = []
+        for i in range(5):
+            u, k = _pairs(torch, n if i < 3 else 60013, 90 + i)
+            mode = (2, 3, 1, 0, 2)[i]
+            jobs.append((u, k, u.clone(), k.clone(), mode, _direct(cg, torch, ctx, u, k, dens, 60 + i, mode)))
+        cg.compton_serve_start(ctx, 3 * 32 * 720000, 16)
+        for i, (u, k, _, _, mode, _) in enumerate(jobs):
+            cg.compton_submit(ctx, u, k, u, k, dens, 60 + i, 2, mode)
+        time.sleep(pause)
+        cg.compton_serve_stop(ctx)
+        torch.cuda.synchronize()
+        for i, (u, k, u0, k0, _, (ur, kr)) in enumerate(jobs):
+            done = torch.equal(u, ur) and torch.equal(k, kr)
+            assert done or (torch.equal(u, u0) and torch.equal(k, k0)), i
     finally:
         cg.compton_destroy(ctx)
