@@ -61,3 +61,26 @@ def test_silu_f32():
     low = z64 <= -87.0
     assert np.all(np.abs(out[low] - exact[low])[z64[low] > -1e20] <= 1e-30)
     assert np.isnan(out[-1]) and out[-4] == 0.0
+
+
+def test_silu_f32_at_the_ends_of_its_range():
+    """Infinities, the largest numbers and NaN: z itself above 87 (sigma is 1 to
+    FP32), a value between SiLU(-87) = -1.4e-36 and 0 below -87."""
+    torch_cuda()
+    nvcc = shutil.which("nvcc") or "/usr/local/cuda/bin/nvcc"
+    build = os.path.join(HERE, "_build")
+    os.makedirs(build, exist_ok=True)
+    so = os.path.join(build, "libsilu_f32_ends.so")
+    subprocess.check_call([nvcc, "-gencode", "arch=compute_103a,code=sm_103a", "-O3", "-std=c++17", "-shared",
+                           "-Xcompiler", "-fPIC", "-o", so, os.path.join(HERE, "silu_f32_eval.cu")])
+    L = ctypes.CDLL(so)
+    L.silu_f32_eval.argtypes = [ctypes.c_void_p, ctypes.c_int64, ctypes.c_void_p]
+    top = np.finfo(np.float32).max
+    ends = np.concatenate([np.geomspace(87.0, top, 3001), [top, np.inf]]).astype(np.float32)
+    z = np.concatenate([ends, -ends, [np.nan]]).astype(np.float32)
+    out = np.empty_like(z)
+    assert L.silu_f32_eval(z.ctypes.data, z.size, out.ctypes.data) == 0
+    high, low = out[:ends.size], out[ends.size:-1]
+    assert np.isinf(high[-1]) and high[-1] > 0 and np.all(np.abs(high[:-1].astype(np.float64) / ends[:-1] - 1.0) <= 5e-7)
+    assert np.all(low <= 0.0) and np.all(low >= -1.5e-36)
+    assert np.isnan(out[-1])
