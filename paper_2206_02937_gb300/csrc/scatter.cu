@@ -606,9 +606,8 @@ __device__ __forceinline__ int32_t ntc_count(const NtcArgs& a, int32_t c, int ne
 }
 
 // Cells with at least this many candidates are listed and taken first, one at
-// a time; the others in runs of kNtcCells.
+// a time; the others in runs of 8 or 32 cells (launch_scatter_ntc).
 constexpr int kNtcBig = 64;
-constexpr int kNtcCells = 8;
 
 __device__ __forceinline__ int pick_index(uint32_t w, int n) { return (int)(((uint64_t)w * (uint64_t)n) >> 32); }
 
@@ -713,8 +712,10 @@ __device__ __forceinline__ int ntc_resolve(const NtcArgs& a, NtcWarp& W, int n)
     return left;
 }
 
+template <int kNtcCells>
 __global__ void __launch_bounds__(32 * kNtcWarps, 3) k_ntc(NtcArgs a)
 {
+    static_assert(kNtcCells == 8 || kNtcCells == 32, "a lane per cell of a run, a power of two");
     __shared__ NtcWarp s_warp[kNtcWarps];
     NtcWarp& W = s_warp[threadIdx.x >> 5];
     const int lane = (int)(threadIdx.x & 31u);
@@ -1141,20 +1142,32 @@ compton_status launch_scatter_ntc(compton_ctx* ctx, compton_species* e, compton_
     a.n_big = a.next + 2;
     a.big = ctx->count[0];
     COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(a.next, 0, 3 * sizeof(uint32_t), stream));
-    // persistent: the CTAs resident at once (work is taken cell by cell)
+    // persistent: the CTAs resident at once (work is taken run by run)
     int per_sm = 0;
-    COMPTON_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ntc, 32 * kNtcWarps, 0));
+    COMPTON_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ntc<8>, 32 * kNtcWarps, 0));
     if (per_sm < 1) per_sm = 1;
     int64_t blocks = (int64_t)ctx->n_sm * per_sm;
+    // runs of 32 cells where every resident warp gets one, or where 32 cells
+    // have no more candidates than a batch; else runs of 8, which spread the
+    // cells better.  A run costs its warp an atomic and a chain of loads however
+    // few candidates it has.  16 + 16 particles a cell with 0.5 candidates, runs
+    // of 8 and of 32: 100,000 cells 40 and 35 us, 262,144 cells 59 and 44;
+    // 2 million cells of 8 + 8 with one 303 and 161; 262,144 cells of 64 + 64
+    // with 4 113 and 105, with 10 135 and 144.
+    const double mean = (double)e->n / (double)pairs->n_cells * (double)g->n / (double)pairs->n_cells * a.w_over_v *
+                        2.0 * a.dt;
+    const bool many = mean < 1.0 || pairs->n_cells >= 32 * kNtcWarps * blocks;
+    const int cells = many ? 32 : 8;
     // a warp per run of cells at most
-    const int64_t need = (pairs->n_cells + kNtcCells * kNtcWarps - 1) / (kNtcCells * kNtcWarps);
+    const int64_t need = (pairs->n_cells + cells * kNtcWarps - 1) / (cells * kNtcWarps);
     if (blocks > need) blocks = need;
     {
         TimedScope ts_(ctx, COMPTON_K_NTC, stream);
         int64_t sb = (pairs->n_cells + 255) / 256;
         if (sb > (int64_t)ctx->n_sm * 8) sb = (int64_t)ctx->n_sm * 8;
         k_ntc_scan<<<(unsigned)sb, 256, 0, stream>>>(a);
-        k_ntc<<<(unsigned)blocks, 32 * kNtcWarps, 0, stream>>>(a);
+        if (many) k_ntc<32><<<(unsigned)blocks, 32 * kNtcWarps, 0, stream>>>(a);
+        else k_ntc<8><<<(unsigned)blocks, 32 * kNtcWarps, 0, stream>>>(a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_ntc");
     return COMPTON_OK;

@@ -40,3 +40,21 @@ def test_ragged_and_empty_cells():
 def test_candidates_that_all_share_two_particles():
     # two electrons and two photons a cell, dozens of candidates: most are held back
     _compare(_workload([2] * 40, 2.0, 4.0, 300), step=2)
+
+
+@pytest.mark.parametrize("cells", [1, 31, 32, 33, 1000, 4097])
+def test_runs_of_32_cells(cells):
+    # less than a candidate a cell in the mean, some cells empty, one listed
+    rng = np.random.default_rng(cells)
+    sizes = rng.poisson(4, cells)
+    if cells > 1:
+        sizes[cells // 2] = 130
+    w = _workload(list(sizes), 1.0 / 64.0, 0.25, 400 + cells)
+    assert (sizes.sum() / cells) ** 2 / 128.0 < 1.0
+    _compare(w, step=7)
+
+
+def test_runs_of_32_cells_among_many_cells():
+    # above a run of 32 for every resident warp, 1.6 candidates a cell
+    sizes = np.random.default_rng(9).integers(1, 4, 150001)
+    _compare(_workload(list(sizes), 0.4, 0.5, 500), step=8)
