@@ -167,6 +167,7 @@ __device__ __forceinline__ float analytic_P(const ScatterArgs& a, float ux, floa
 // accepted list.  Candidates above the FP64 gamma threshold are set aside and
 // decided after the warp's last chunk.
 constexpr int kProbWarps = kProbThreads / 32;
+constexpr int kResolveWarps = 2;                   // warps of a CTA that resolves its own collisions
 constexpr int kChunkPairs = 32 * kPairsPerThread;  // pairs of one warp step
 constexpr int kWarpCells = 64;                     // cells of a pair tile a warp stages
 constexpr int kQueueCap = 160;                     // queued candidates per warp (31 + one chunk's 128)
@@ -197,13 +198,19 @@ struct Batch {
 // (one atomic per batch) instead of being evaluated.
 // kResolve (a small call): every warp resolves its own accepted pairs at the
 // end, which saves the collision kernel's launch; where warps have many pairs
-// the collisions' registers and the idle lanes cost more than the launch.
+// the collisions' registers and the idle lanes cost more than the launch.  Its
+// CTAs have two warps, so that a small call's collisions reach all SMs (with
+// eight, 32 tiles share 32 SMs' FP64 units).  Plain step of 512 cells of 64 + 64
+// with n dt = 0.05 / 1 / 5, two launches, CTAs of eight and of two warps: 67.6 / 71.9
+// / 79.1, 43.7 / 56.4 / 77.2 and 42.6 / 52.2 / 67.5 us.
 template <bool kBinned, bool kWeighted, bool kCandOut = false, bool kResolve = false>
-__global__ void __launch_bounds__(kProbThreads, kResolve ? 2 : 4) k_pair_prob(ScatterArgs a)
+__global__ void __launch_bounds__(kResolve ? 32 * kResolveWarps : kProbThreads, kResolve ? 2 : 4)
+    k_pair_prob(ScatterArgs a)
 {
     chain_start();
-    __shared__ WarpWindow s_win[kProbWarps];
-    __shared__ WarpQueue s_queue[kProbWarps];
+    constexpr int kWarps = kResolve ? kResolveWarps : kProbWarps;
+    __shared__ WarpWindow s_win[kWarps];
+    __shared__ WarpQueue s_queue[kWarps];
     const unsigned lane = threadIdx.x & 31u;
     const unsigned lt_mask = (1u << lane) - 1u;
     const int w = threadIdx.x >> 5;
@@ -215,8 +222,8 @@ __global__ void __launch_bounds__(kProbThreads, kResolve ? 2 : 4) k_pair_prob(Sc
     const pidx total = kBinned ? (pidx)*a.n_pairs : (pidx)a.p_end;
     const pidx pbase = kBinned ? 0 : (pidx)a.p_begin;
     const int64_t n_chunks = total > pbase ? ((int64_t)total - pbase + kChunkPairs - 1) / kChunkPairs : 0;
-    const int64_t n_warps = (int64_t)gridDim.x * kProbWarps;
-    const int64_t gw = (int64_t)blockIdx.x * kProbWarps + w;
+    const int64_t n_warps = (int64_t)gridDim.x * kWarps;
+    const int64_t gw = (int64_t)blockIdx.x * kWarps + w;
     const int ch_begin = (int)(n_chunks * gw / n_warps), ch_end = (int)(n_chunks * (gw + 1) / n_warps);
     const bool all = a.prob_out != nullptr;
     unsigned n_pairs = 0;
@@ -966,8 +973,9 @@ compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, cu
 }
 
 // Pair tiles up to which a plain step resolves its collisions in the
-// probability kernel: one chunk of 128 pairs per warp, about four collisions,
-// which take less than the 6 us of the collision kernel's launch.
+// probability kernel: one chunk of 128 pairs per warp, so at most four rounds of
+// collisions after its own evaluation; the collision kernel's launch takes 6 us
+// and spreads them no further (the figures are at k_pair_prob, up to n dt = 5).
 constexpr unsigned kResolveTiles = 32;
 
 // The step after the pair list is known: probability and trial of every
@@ -982,7 +990,8 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         const unsigned grid = prob_grid(ctx, tiles);
         if (tiles <= kResolveTiles) {
             TimedScope ts_(ctx, COMPTON_K_PROB, stream);
-            launch_chained(k_pair_prob<kBinned, kWeighted, false, true>, grid, kProbThreads, 0, stream, a);
+            launch_chained(k_pair_prob<kBinned, kWeighted, false, true>, grid * (kProbWarps / kResolveWarps),
+                           32 * kResolveWarps, 0, stream, a);
             COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
             return COMPTON_OK;
         }
