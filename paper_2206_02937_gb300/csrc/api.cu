@@ -101,10 +101,10 @@ compton_status compton_init(const compton_config* cfg, compton_ctx** out)
     ctx->max_pair_tiles = (P + compton::kPairsPerTile - 1) / compton::kPairsPerTile + 1;
 
     Carver cv;
-    // both histograms and the two order flags in one block, cleared by one
+    // both histograms and the four order counts in one block, cleared by one
     // memset per binning call; the second histogram starts 256-byte aligned
     const size_t C_pad = align_up((size_t)C, 64);
-    const size_t o_count = cv.take<int32_t>(2 * C_pad + 2);
+    const size_t o_count = cv.take<int32_t>(2 * C_pad + 4);
     size_t o_off[2], o_rec[2], o_stile[2];
     for (int s = 0; s < 2; ++s) {
         o_off[s] = cv.take<int32_t>(C + 1);

@@ -46,6 +46,9 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // unsorted[s] counts the positions at which the cell index descends, plus one
 // per warp that saw an index outside [0, C): only if it is not zero does the
 // placement run, and by its size the placement takes its form (sort_source).
+// In large input each warp also looks at its last 128 positions: unsorted[2 + s]
+// counts the positions of the warps in whose stretch neighbours in the input are
+// not neighbours in the cells (scattered).
 //
 // What bounds it: instruction issue (113 instructions per 128 positions of input
 // in cell order; 140 when every position was looked at as first and last of its
@@ -65,13 +68,33 @@ __device__ __forceinline__ int4 load_cells4(const int32_t* __restrict__ cell, Id
     return v;
 }
 
+// Particles of a species from which the placement looks at scattered: below,
+// the input stays in the L2 while the sort gathers from it.
+constexpr int64_t kScatterLook = (int64_t)1 << 22;
+
+// Whether most of 128 consecutive positions lie far from their neighbours in the
+// cells (v: four per lane): more than max_runs runs of equal cells (a 32-byte
+// sector holds eight words), and 64 positions on another cell than such input in cell order, or some
+// two dozen ordered runs of it, would have there (one cell per n / C positions).
+__device__ __forceinline__ bool scattered(const int4& v, int64_t n, int64_t C, unsigned max_runs)
+{
+    const unsigned lane = lane_id();
+    const int32_t left = __shfl_up_sync(0xffffffffu, v.w, 1), on = __shfl_down_sync(0xffffffffu, v.x, 16);
+    const unsigned begins = __reduce_add_sync(0xffffffffu, (unsigned)(lane == 0 || v.x != left) + (v.y != v.x) +
+                                                               (v.z != v.y) + (v.w != v.z));
+    const uint32_t near = (uint32_t)(24.0f * 64.0f * (float)C / (float)n) + 8u;
+    const unsigned far = __ballot_sync(0xffffffffu, lane < 16u && (uint32_t)on - (uint32_t)v.x > near);
+    return begins > max_runs && __popc(far) > 8;
+}
+
 // Positions in Idx: 32-bit when every position the grid visits fits (the
 // launch checks), else 64-bit.
 template <typename Idx>
 __global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_count(const int32_t* __restrict__ cell_e, int64_t n_e,
                                                         const int32_t* __restrict__ cell_g, int64_t n_g, int64_t C,
                                                         int32_t* __restrict__ count_e, int32_t* __restrict__ count_g,
-                                                        uint32_t* __restrict__ unsorted, DeviceStats* stats)
+                                                        uint32_t* __restrict__ unsorted, unsigned max_runs,
+                                                        DeviceStats* stats)
 {
     chain_start();
     const int s = blockIdx.y;
@@ -96,10 +119,11 @@ __global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_cou
         if (vec && at + 128 <= n) return *reinterpret_cast<const int4*>(cell + at + 4 * (Idx)lane);
         return load_cells4(cell, (Idx)(at + 4 * (Idx)lane), n, vec);
     };
-    int4 q = make_int4(-1, -1, -1, -1);
+    int4 q = make_int4(-1, -1, -1, -1), v = q;
+    const Idx begin = base;
     if (base < stop) q = load(base);
     for (; base < stop; base += 128) {
-        const int4 v = q;
+        v = q;
         if (base + 128 < stop) q = load(base + 128);
         const int32_t left = __shfl_up_sync(0xffffffffu, v.w, 1), prev = lane == 0 ? before : left;
         // the lane's positions at which a run begins
@@ -130,9 +154,13 @@ __global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_cou
     }
     const bool any_bad = __any_sync(0xffffffffu, bad);
     descents = __reduce_add_sync(0xffffffffu, descents);
+    // (where a quarter of the stretch descends the order is settled)
+    const bool apart = (int64_t)n > kScatterLook && begin < stop && stop <= n &&
+                       (int64_t)descents * 4 < (int64_t)(stop - begin) && scattered(v, (int64_t)n, C, max_runs);
     if (lane == 0) {
         if (any_bad) atomicOr(&stats->error_flags, (unsigned long long)kErrCellRange);
         if (descents + any_bad) atomicAdd(&unsorted[s], descents + any_bad);
+        if (apart) atomicAdd(&unsorted[2 + s], (uint32_t)(stop - begin));
     }
 }
 
@@ -142,15 +170,21 @@ __global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_cou
 // after another) most of a cell's particles are neighbours in the input: the
 // placement writes each particle's index (4 bytes) and the sort gathers
 // through it.  Above that (particles in no order: half the positions descend)
-// a gather would fetch a 32-byte sector per word, and whole records are placed.
+// a gather would fetch a 32-byte sector per word, and whole records are placed;
+// so too where few positions descend but most are scattered (cell i mod C for
+// particle i; short runs of equal cells in no order).
 // 512^2 cells, 64 + 64 per cell, a tenth of them moved: the placement takes
-// 0.087 ms by index and 0.368 ms by record, the sort after it 0.34 ms each.
+// 0.087 ms by index and 0.368 ms by record, the sort after it 0.34 ms each.  The
+// same cells with particle i in cell i mod C: 0.278 and 0.784 by index, 0.523 and 0.322 by
+// record; runs of three in no order 0.224 and 0.916 against 0.498 and 0.338.
 enum SortSource : int { kInPlace = 0, kByIndex = 1, kRecords = 2 };
 constexpr uint32_t kIndexPlaced = 0xFFFFFFFFu;  // k_bin_small has placed indices, whatever the order
-__device__ __forceinline__ SortSource sort_source(uint32_t unsorted, int64_t n)
+__device__ __forceinline__ SortSource sort_source(const uint32_t* __restrict__ unsorted, int s, int64_t n)
 {
-    if (unsorted == 0) return kInPlace;
-    return unsorted == kIndexPlaced || (int64_t)unsorted * 4 < n ? kByIndex : kRecords;
+    const uint32_t descents = unsorted[s], apart = unsorted[2 + s];
+    if (descents == 0) return kInPlace;
+    if (descents == kIndexPlaced) return kByIndex;
+    return (int64_t)descents * 4 < n && (int64_t)apart * 2 < n ? kByIndex : kRecords;
 }
 
 // ---------------------------------------------------------------------------
@@ -602,7 +636,7 @@ __global__ void __launch_bounds__(kPlaceThreads, 2048 / kPlaceThreads) k_place(c
     if (kChained) chain_start();
     const int s = blockIdx.y;
     const int64_t n = a.n[s];
-    const SortSource source = sort_source(a.unsorted[s], n);
+    const SortSource source = sort_source(a.unsorted, s, n);
     if (source == kInPlace) return;
     const int32_t* __restrict__ cell = a.cell[s];
     const int32_t* __restrict__ off = a.off[s];
@@ -634,11 +668,12 @@ __global__ void __launch_bounds__(kPlaceThreads, 2048 / kPlaceThreads) k_place(c
         return;
     }
     // whole records.  Particles in no order among many cells seldom share one
-    // within a warp: each takes its own place, with no search for peers
+    // within a warp: each takes its own place, with no search for peers (scattered
+    // input with few descents may hold short runs of equal cells)
     const uint32_t* __restrict__ id = a.id[s];
     const float* __restrict__ wt = a.w[s];
     SortRec* __restrict__ rec = a.rec[s];
-    const bool alone = a.C >= kPlaceAloneCells;
+    const bool alone = a.C >= kPlaceAloneCells && (int64_t)a.unsorted[s] * 4 >= n;
     for (int64_t r0 = warp * 32; r0 < n; r0 += n_warps * 32) {
         const int64_t i = r0 + lane;
         const int c = load_cell(i);
@@ -1020,7 +1055,7 @@ __global__ void __launch_bounds__(kSortThreads, 10) k_sort_gather(const __grid_c
     if (R <= 0) return;
 
     SortSrc t;
-    const SortSource source = sort_source(g.unsorted[s], g.n[s]);
+    const SortSource source = sort_source(g.unsorted, s, g.n[s]);
     t.rec = source == kRecords ? g.rec[s] : nullptr;
     t.idx = source == kByIndex ? reinterpret_cast<const int32_t*>(g.rec[s]) : nullptr;
     t.id = g.in_id[s];
@@ -1123,20 +1158,22 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
     } else {
         // count[0], count[1] and unsorted lie in one block of the workspace
         COMPTON_CUDA_TRY(ctx, cudaMemsetAsync(ctx->count[0], 0,
-                                              reinterpret_cast<char*>(ctx->unsorted + 2) -
+                                              reinterpret_cast<char*>(ctx->unsorted + 4) -
                                                   reinterpret_cast<char*>(ctx->count[0]),
                                               stream));
         const dim3 cgrid(grid_for((nmax + 3) / 4, kCountThreads, ctx->n_sm * kCountCtasPerSm), 2);  // four per thread
         {
             TimedScope ts_(ctx, COMPTON_K_COUNT, stream);
+            // a sixth of the positions begin a run, an eighth with the weight as one word more to gather
+            const unsigned max_runs = weighted ? 16u : 24u;
             // 32-bit positions when the grid's last visited position fits
             const int64_t span = (nmax + 127) / 128 * 128 + (int64_t)cgrid.x * kCountThreads * 4;
             if (span < ((int64_t)1 << 31))
                 launch_chained(k_count<int32_t>, cgrid, kCountThreads, 0, stream, e_in->cell_dev, ne, g_in->cell_dev,
-                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, ctx->stats);
+                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, max_runs, ctx->stats);
             else
                 launch_chained(k_count<int64_t>, cgrid, kCountThreads, 0, stream, e_in->cell_dev, ne, g_in->cell_dev,
-                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, ctx->stats);
+                               ng, C, ctx->count[0], ctx->count[1], ctx->unsorted, max_runs, ctx->stats);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_count");
         TimedScope scan_scope(ctx, COMPTON_K_SCAN, stream);

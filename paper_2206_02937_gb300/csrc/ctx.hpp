@@ -192,7 +192,8 @@ struct compton_ctx {
     int32_t* count[2] = {nullptr, nullptr};      // [C] histogram, then insertion cursor
     int32_t* off[2] = {nullptr, nullptr};        // [C+1]
     compton::SortRec* rec[2] = {nullptr, nullptr};  // [max_particles] placed records
-    uint32_t* unsorted = nullptr;                // [2] descents (and warps with a bad index) of a species' cells
+    uint32_t* unsorted = nullptr;                // [2] descents (and warps with a bad index) of a species' cells,
+                                                 // [2] positions in scattered stretches of them
     int32_t* stile[2] = {nullptr, nullptr};      // [max_sort_tiles+1] first cell of each sort tile
     int64_t* block_sums = nullptr;               // [3 * max_scan_tiles]
     compton::CellInfo* cinfo = nullptr;          // [C]
