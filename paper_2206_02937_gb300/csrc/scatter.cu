@@ -959,13 +959,19 @@ void fill_common(ScatterArgs& a, compton_ctx* ctx, uint64_t seed, uint64_t step,
     a.weighted = false;
 }
 
-// The collisions of the accepted pairs.
-compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, cudaStream_t stream)
+// The collisions of the accepted pairs.  after_tc: the decisions were made in a
+// tensor-core network, whose CTAs fill their SMs: CTAs placed early then pack,
+// eight to an SM, into the SMs that come free first and are bound by these SMs'
+// FP64 units, so they are chained up to two per SM only.  Step of 2048 cells of
+// 64 + 64 with the BF16 network, 512 CTAs: 92.3 us chained, 67.5 us after the
+// network's end; 1024 cells, 256 CTAs: 64.2 and 68.5.
+compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, bool after_tc, cudaStream_t stream)
 {
     {
         TimedScope ts_(ctx, COMPTON_K_COLLIDE, stream);
         const unsigned grid = (unsigned)collide_grid(rows);
-        if (grid <= kChainBlocks) launch_chained(k_collide<true>, grid, 256, 0, stream, a);
+        const int64_t chained = after_tc ? 2 * (int64_t)ctx->n_sm : kChainBlocks;
+        if (grid <= chained) launch_chained(k_collide<true>, grid, 256, 0, stream, a);
         else k_collide<false><<<grid, 256, 0, stream>>>(a);
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_collide");
@@ -1025,7 +1031,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         if (mode == COMPTON_MODE_PNET) {
             const compton_status sp = launch_pnet_decide(ctx, rows, dec, a.w_e, a.w_g, stream);
             if (sp != COMPTON_OK) return sp;
-            return launch_collide(ctx, a, rows, stream);
+            return launch_collide(ctx, a, rows, false, stream);
         }
         const bool fused = mode != COMPTON_MODE_MLP_FP32;
         compton_status st = launch_mlp_infer(ctx, a.u[0], a.u[1], a.u[2], a.k[0], a.k[1], a.k[2], rows, mode,
@@ -1037,7 +1043,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
         }
     }
     COMPTON_LAUNCH_CHECK(ctx, "k_pair_prob");
-    return launch_collide(ctx, a, rows, stream);
+    return launch_collide(ctx, a, rows, mode != COMPTON_MODE_MLP_FP32, stream);
 }
 
 }  // namespace
