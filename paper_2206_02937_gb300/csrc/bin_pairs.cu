@@ -1209,7 +1209,7 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
         pa.draw = key_draw;
         {
             TimedScope ts_(ctx, COMPTON_K_PLACE, stream);
-            if ((int64_t)pgrid.x * pgrid.y <= kChainBlocks)
+            if ((int64_t)pgrid.x * pgrid.y <= chain_blocks(ctx))
                 launch_chained(k_place<true>, pgrid, kPlaceThreads, 0, stream, pa);
             else
                 k_place<false><<<pgrid, kPlaceThreads, 0, stream>>>(pa);
@@ -1241,7 +1241,7 @@ compton_status launch_bin_pairs(compton_ctx* ctx, const compton_species* e_in, c
         sg.nb_e = nb_e;
         const int smem = (int)kSortSmem;
         TimedScope ts_(ctx, COMPTON_K_SORT, stream);
-        if (nb_e + nb_g <= kChainBlocks)
+        if (nb_e + nb_g <= chain_blocks(ctx))
             launch_chained(k_sort_gather<true>, (unsigned)(nb_e + nb_g), kSortThreads, smem, stream, sg);
         else
             k_sort_gather<false><<<(unsigned)(nb_e + nb_g), kSortThreads, smem, stream>>>(sg);

@@ -263,13 +263,17 @@ inline compton_status set_cuda_error(compton_ctx* ctx, cudaError_t e, const char
 // Launch of a kernel that begins with chain_start(): its blocks may be placed,
 // and wait there, while the stream's previous kernel drains, so that a call's
 // launches follow one another without the launch latency in between (1 to 2 us
-// each).  A block pays about a microsecond for the wait, so the kernels of many
-// short blocks have a form without it, taken above kChainBlocks (a 512^2 step
-// of 65536 + 65536 sort blocks: 585 us without it, 608 with it; 131072 of 128^3
-// cells: 1175 and 1326; up to four blocks per SM all start together and the
-// wait is paid once).  The No-Time-Counter kernels gain nothing from it (270 us
-// either way) and are launched as usual.
-constexpr int64_t kChainBlocks = 608;
+// each).  A block pays about a microsecond for the wait where its launch does
+// not start all at once: the sort, the placement and the collisions have a form
+// without it, taken above four blocks per SM (a 512^2 step of 65536 + 65536 sort
+// blocks: 585 us without it, 608 with it; 131072 of 128^3 cells: 1175 and 1326;
+// up to four blocks per SM all start together and the wait is paid once).  The
+// others are always chained: the scans gain from it at any size (128^3 cells,
+// 2048 blocks: step 635 against 641 us; 256^3, 16384 blocks: 1215 and 1222), the
+// decisions and the paper's network run equally long either way at their
+// largest (32 and 8 blocks per SM).  The No-Time-Counter kernels gain nothing
+// from it and are launched as usual.
+inline int64_t chain_blocks(const compton_ctx* ctx) { return 4 * (int64_t)ctx->n_sm; }
 template <typename... KArgs, typename... Args>
 inline void launch_chained(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, Args&&... args)
 {

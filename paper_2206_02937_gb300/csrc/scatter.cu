@@ -970,7 +970,7 @@ compton_status launch_collide(compton_ctx* ctx, ScatterArgs& a, int64_t rows, bo
     {
         TimedScope ts_(ctx, COMPTON_K_COLLIDE, stream);
         const unsigned grid = (unsigned)collide_grid(rows);
-        const int64_t chained = after_tc ? 2 * (int64_t)ctx->n_sm : kChainBlocks;
+        const int64_t chained = after_tc ? 2 * (int64_t)ctx->n_sm : chain_blocks(ctx);
         if (grid <= chained) launch_chained(k_collide<true>, grid, 256, 0, stream, a);
         else k_collide<false><<<grid, 256, 0, stream>>>(a);
     }
@@ -1011,7 +1011,7 @@ compton_status launch_step(compton_ctx* ctx, ScatterArgs& a, compton_mode mode, 
             TimedScope ts_(ctx, COMPTON_K_COLLIDE, stream);
             // kCollideWarps warps per region, four to a CTA
             const unsigned cgrid = (unsigned)(kCollideWarps * prob_warps + 3) / 4;
-            if (cgrid <= kChainBlocks) launch_chained(k_collide_regions<true>, cgrid, 128, 0, stream, a, prob_warps);
+            if (cgrid <= chain_blocks(ctx)) launch_chained(k_collide_regions<true>, cgrid, 128, 0, stream, a, prob_warps);
             else k_collide_regions<false><<<cgrid, 128, 0, stream>>>(a, prob_warps);
         }
         COMPTON_LAUNCH_CHECK(ctx, "k_collide_regions");
