@@ -444,7 +444,8 @@ typedef struct compton_result {
 /* Start the serving engine: a device pool of pool_bytes (the memory budget;
  * each admitted request holds 28 bytes per pair, 32 in surrogate modes) and
  * at most max_active requests admitted at once.  The pool is allocated here,
- * once, with 29 MB of the engine's own lists.  EINVAL if already started. */
+ * once, with the engine's own lists beside it (100 bytes for each 64 of the
+ * pool, at least 29 MB and at most 213 MB).  EINVAL if already started. */
 compton_status compton_serve_start(struct compton_ctx* ctx, uint64_t pool_bytes, int32_t max_active);
 
 /* Stop the engine.  Requests whose work has begun are finished first; the

@@ -59,7 +59,7 @@ constexpr int kServeCandCap = kPairsPerTile + kServeThreads;  // queued candidat
 constexpr int kServeHitCap = 2 * kServeThreads;               // queued collisions: a batch's and a remainder
 constexpr int kMaxTilesPerLaunch = 32768;                     // 33.5M pairs
 constexpr int kTileRing = 4;
-constexpr uint32_t kServeListCap = 1u << 18;                  // surrogate candidates of a launch
+constexpr uint32_t kServeListMin = 1u << 18, kServeListMax = 1u << 21;  // surrogate candidates of a launch
 constexpr int kServeRejects = kMaxTilesPerLaunch;
 
 struct ReqDev {
@@ -86,6 +86,7 @@ struct TileDev {
 struct ServeControl {
     uint32_t n_cand, n_accepted, n_rejected;
     uint32_t n_reserved;  // candidates of all tiles, those turned away too
+    uint32_t n_unseen;    // tiles turned away before their candidates were counted
     int32_t rejected[kServeRejects];
 };
 
@@ -151,11 +152,12 @@ __device__ __forceinline__ void quad_transpose(uint32_t (&w)[4])
 // on explicit pairs (same device functions).
 __global__ void __launch_bounds__(kServeThreads, 3)
     k_serve(const ReqDev* __restrict__ reqs, const TileDev* __restrict__ tiles, int n_tiles, float dt, float gamma64,
-            float c64sq, DeviceStats* stats, CandPair* __restrict__ cand, ServeControl* __restrict__ ctl)
+            float c64sq, DeviceStats* stats, CandPair* __restrict__ cand, uint32_t cand_cap,
+            ServeControl* __restrict__ ctl)
 {
     __shared__ CQEntry cq[kServeCandCap];
     __shared__ SQEntry sq[kServeHitCap];
-    __shared__ int cn, sn, listed;
+    __shared__ int cn, sn, listed, full;
     __shared__ uint32_t list_base;
     const int tid = threadIdx.x;
     if (tid == 0) cn = sn = 0;
@@ -185,6 +187,7 @@ __global__ void __launch_bounds__(kServeThreads, 3)
     };
 
     for (int t = blockIdx.x; t < n_tiles; t += gridDim.x) {
+        const uint32_t reserved = tid == 0 ? __ldcg(&ctl->n_reserved) : 0u;
         const TileDev T = tiles[t];
         const ReqDev& R = reqs[T.req];
         const bool plain = R.mode == COMPTON_MODE_PLAIN;
@@ -200,8 +203,19 @@ __global__ void __launch_bounds__(kServeThreads, 3)
         const uint32_t thr0 = cand_threshold(R.dens_scalar, dt);
         float u[4][3], k[4][3], dens[4];
         int slot[4];
-        if (tid == 0) listed = 0;
+        if (tid == 0) {
+            listed = 0;
+            full = !plain && reserved > cand_cap;
+            if (full) {  // no room for any candidate
+                ctl->rejected[atomicAdd(&ctl->n_rejected, 1u)] = t;
+                atomicAdd(&ctl->n_unseen, 1u);
+            }
+        }
         __syncthreads();
+        if (full) {
+            __syncthreads();
+            continue;
+        }
 #pragma unroll
         for (int rr = 0; rr < kServePairsPerThread; ++rr) {
             const int local = rr * kServeThreads + tid;
@@ -236,7 +250,7 @@ __global__ void __launch_bounds__(kServeThreads, 3)
             if (tid == 0) {
                 // the reservations that fit are the first ones: what they hold has no gaps
                 uint32_t at = want > 0 ? atomicAdd(&ctl->n_reserved, (uint32_t)want) : 0u;
-                if (at + (uint32_t)want > kServeListCap) {
+                if (at + (uint32_t)want > cand_cap) {
                     at = 0xFFFFFFFFu;
                     ctl->rejected[atomicAdd(&ctl->n_rejected, 1u)] = t;
                 } else if (want > 0) {
@@ -327,6 +341,7 @@ struct ServeReq {
     compton_request req{};
     int64_t tiles = 0, launched = 0, done_tiles = 0;
     int64_t flying = 0;  // tiles in launches that are not retired
+    double share = 0.0;  // candidates among its pairs, roughly
     std::vector<TileDev> again;  // tiles a full candidate list turned away
     int state = 0;  // 0 queued, 1 admitted, 4 done
     size_t off = 0, bytes = 0;
@@ -341,6 +356,7 @@ struct Launch {
     int ring = 0;
     compton_status status = COMPTON_OK;      // of every request in it
     compton_status net_status = COMPTON_OK;  // of its surrogate requests
+    double known = 0.0, open_pairs = 0.0;    // candidates expected of its scalar densities, surrogate pairs of the others
     std::vector<std::pair<uint64_t, int64_t>> tiles_per_req;  // ticket, tiles in this launch
 };
 
@@ -361,7 +377,8 @@ struct ServeEngine {
     std::vector<int> free_slots;
     TileDev* tiles_dev = nullptr;
     TileDev* tiles_host = nullptr;      // pinned, kTileRing x kMaxTilesPerLaunch
-    CandList list{};                    // surrogate candidates of a launch, kServeListCap
+    CandList list{};                    // surrogate candidates of a launch
+    uint32_t list_cap = 0;
     ServeControl* ctl_dev = nullptr;
     ServeControl* ctl_host = nullptr;   // pinned, kTileRing
     int ring = 0;
@@ -502,12 +519,15 @@ void admit(ServeEngine* E)
     }
 }
 
-// Pairs of a request that are candidates, roughly (a launch takes no more
-// surrogate tiles than its list will hold; what it turns away is launched again).
-double expected_candidates(const compton_request& r, double dt, double pairs)
+// The share of a request's pairs that are candidates, roughly (a launch takes no
+// more surrogate tiles than its list will hold; what it turns away is launched
+// again).  Densities per pair are on the device: a quarter, until the first
+// launch of the request has counted them (retire).
+double candidate_share(const compton_request& r, double dt)
 {
-    const double share = r.n_dens_dev ? 0.25 : 1.0 - std::exp(-2.001 * (double)r.n_dens * dt);
-    return pairs * (share < 1.0 ? share : 1.0);
+    if (r.n_dens_dev) return 0.25;
+    const double share = 1.0 - std::exp(-2.001 * (double)r.n_dens * dt);
+    return share < 1.0 ? share : 1.0;
 }
 
 // The launch's table, tiles and k_serve.
@@ -526,7 +546,7 @@ compton_status launch_serve(ServeEngine* E, const TileDev* th, TileDev* td, int 
     const int grid = std::min(nt, ctx->n_sm * 3);
     k_serve<<<grid, kServeThreads, 0, s>>>(E->reqs_dev, td, nt, (float)cfg.dt, cfg.gamma_fp64_threshold,
                                            cfg.collide_fp64_threshold * cfg.collide_fp64_threshold, ctx->stats,
-                                           E->list.cand, E->ctl_dev);
+                                           E->list.cand, E->list_cap, E->ctl_dev);
     COMPTON_LAUNCH_CHECK(ctx, "k_serve");
     return COMPTON_OK;
 }
@@ -545,7 +565,7 @@ compton_status launch_candidates(ServeEngine* E, int mode, int64_t rows)
                                          &E->list);
     if (st == COMPTON_OK && !fused) st = launch_decide(ctx, E->list, rows, s);
     if (st != COMPTON_OK) return st;
-    const int rgrid = (int)std::min<int64_t>((rows + 255) / 256, (int64_t)ctx->n_sm * 8);
+    const int rgrid = (int)std::min<int64_t>((rows + 255) / 256, (int64_t)ctx->n_sm * 32);
     k_serve_resolve<<<rgrid, 256, 0, s>>>(E->reqs_dev, E->list.accepted, E->ctl_dev, cfg.gamma_fp64_threshold,
                                           cfg.collide_fp64_threshold * cfg.collide_fp64_threshold);
     COMPTON_LAUNCH_CHECK(ctx, "k_serve_resolve");
@@ -572,7 +592,6 @@ compton_status launch_results(ServeEngine* E, Launch& L, int nt)
 void launch_tiles(ServeEngine* E)
 {
     if (E->active.empty() || E->fatal != COMPTON_OK) return;
-    const compton_config& cfg = E->ctx->cfg;
     TileDev* th = E->tiles_host + (size_t)E->ring * kMaxTilesPerLaunch;
     TileDev* td = E->tiles_dev + (size_t)E->ring * kMaxTilesPerLaunch;
     int nt = 0;
@@ -590,9 +609,11 @@ void launch_tiles(ServeEngine* E)
         if (!surrogate || mode == (int)R.req.mode) {
             while ((R.launched < R.tiles || !R.again.empty()) && nt < kMaxTilesPerLaunch) {
                 if (surrogate) {
-                    const double c = expected_candidates(R.req, cfg.dt, kPairsPerTile);
-                    if (cand > 0.0 && cand + c > 0.9 * kServeListCap) break;
+                    const double c = R.share * kPairsPerTile;
+                    if (cand > 0.0 && cand + c > 0.95 * E->list_cap) break;
                     cand += c;
+                    if (R.req.n_dens_dev) L.open_pairs += kPairsPerTile;
+                    else L.known += c;
                 }
                 if (!R.again.empty()) {
                     th[nt++] = R.again.back();
@@ -614,7 +635,7 @@ void launch_tiles(ServeEngine* E)
     L.status = launch_serve(E, th, td, nt);
     if (L.status == COMPTON_OK && mode != COMPTON_MODE_PLAIN)
         // the grids are sized for the list the host expects, at most a full one
-        L.net_status = launch_candidates(E, mode, (int64_t)std::min<double>(kServeListCap, 1.2 * cand + 4096.0));
+        L.net_status = launch_candidates(E, mode, (int64_t)std::min<double>(E->list_cap, 1.2 * cand + 4096.0));
     if (L.status == COMPTON_OK) L.status = launch_results(E, L, nt);
     if (L.status != COMPTON_OK) {
         // no event to wait for: everything before has to end here
@@ -654,6 +675,10 @@ void retire(ServeEngine* E)
         ServeControl* ch = E->ctl_host + L.ring;
         const uint32_t n_rejected = read ? ch->n_rejected : 0;
         const TileDev* th = E->tiles_host + (size_t)L.ring * kMaxTilesPerLaunch;
+        // candidates among the pairs whose densities are on the device
+        double share = 0.0;
+        const double seen = L.open_pairs - (read ? (double)ch->n_unseen * kPairsPerTile : 0.0);
+        if (read && seen > 0.0) share = std::min(1.0, std::max(1e-3, ((double)ch->n_reserved - L.known) / seen));
         std::unordered_map<int, int64_t> turned_away;  // slot -> tiles
         for (uint32_t i = 0; i < n_rejected; ++i) ++turned_away[th[ch->rejected[i]].req];
         for (auto& tr : L.tiles_per_req) {
@@ -663,6 +688,7 @@ void retire(ServeEngine* E)
             const auto it = turned_away.find(R.dslot);
             const int64_t away = it == turned_away.end() ? 0 : it->second;
             R.flying -= tr.second;
+            if (share > 0.0 && R.req.n_dens_dev) R.share = share;
             R.done_tiles += tr.second - away;
             if (away) {
                 if (R.launched == R.tiles && R.again.empty()) E->active.push_back(R.ticket);
@@ -737,6 +763,13 @@ compton_status serve_start(compton_ctx* ctx, uint64_t pool_bytes, int32_t max_ac
     E->device = ctx->cfg.device;
     E->pool_bytes = pool_bytes;
     E->max_active = max_active;
+    // one candidate for two pairs that the pool admits, within the bounds: a
+    // launch has fixed costs of about 30 us and a last wave of collisions.  8
+    // million pairs of densities 200 (all candidates) for the BF16 network, known
+    // to the host / per pair on the device: 4119 and 4361 us with 2^18 and no
+    // count of the candidates seen, 3966 and 4060 with the count, 2742 and 2883
+    // with 2^21 and no work spent on tiles that find the list full.
+    E->list_cap = (uint32_t)std::min<uint64_t>(kServeListMax, std::max<uint64_t>(kServeListMin, pool_bytes / 64));
     cudaError_t e = inject_fault() ? cudaErrorMemoryAllocation : cudaMalloc(&E->pool, pool_bytes);
     if (e == cudaSuccess) e = cudaMalloc(&E->reqs_dev, sizeof(ReqDev) * max_active);
     if (e == cudaSuccess) e = cudaMalloc(&E->counters, sizeof(unsigned long long) * max_active);
@@ -744,9 +777,9 @@ compton_status serve_start(compton_ctx* ctx, uint64_t pool_bytes, int32_t max_ac
     if (e == cudaSuccess) e = cudaMallocHost(&E->reqs_host, sizeof(ReqDev) * max_active);
     if (e == cudaSuccess) e = cudaMallocHost(&E->tiles_host, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
     if (e == cudaSuccess) e = cudaMallocHost(&E->scat_host, sizeof(unsigned long long) * max_active * kTileRing);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.cand, sizeof(CandPair) * kServeListCap);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.accepted, sizeof(AcceptedPair) * kServeListCap);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.r, sizeof(float) * kServeListCap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.cand, sizeof(CandPair) * E->list_cap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.accepted, sizeof(AcceptedPair) * E->list_cap);
+    if (e == cudaSuccess) e = cudaMalloc(&E->list.r, sizeof(float) * E->list_cap);
     if (e == cudaSuccess) e = cudaMalloc(&E->ctl_dev, sizeof(ServeControl));
     if (e == cudaSuccess) e = cudaMallocHost(&E->ctl_host, sizeof(ServeControl) * kTileRing);
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&E->s_compute, cudaStreamNonBlocking);
@@ -817,6 +850,7 @@ compton_status serve_submit(compton_ctx* ctx, const compton_request* r, uint64_t
     R.req = *r;
     R.tiles = (r->n + kPairsPerTile - 1) / kPairsPerTile;
     R.bytes = bytes;
+    R.share = candidate_share(*r, ctx->cfg.dt);
     R.t_submit = now_s();
     *ticket = R.ticket;
     E->reqs.emplace(R.ticket, R);

@@ -94,3 +94,55 @@ def test_more_candidates_than_the_list_holds(per_pair):
         assert st["pairs_tested"] == 2 * sum(j[1].shape[1] for j in jobs)
     finally:
         cg.compton_destroy(ctx)
+
+
+@pytest.mark.parametrize("n,launches", [(1000003, 2), (5000003, 6)])
+def test_dense_densities_per_pair_take_few_launches(n, launches):
+    """Every pair a candidate, which the host cannot know: the list follows the
+    pool (2^21 candidates here), and what a launch turns away is taken in full
+    lists once its candidates are counted (three full lists for 5 million, two
+    launches before the count)."""
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    cg.build()
+    ctx = _ctx(cg, n)
+    try:
+        u, k = _pairs(torch, n, 31)
+        dens = torch.full((n,), 200.0, device="cuda")
+        ref = _direct(cg, torch, ctx, u, k, dens, 6, 1, 2)
+        cg.compton_serve_start(ctx, 1 << 28, 8)
+        cg.compton_kernel_timing(ctx, True)
+        uo, ko = torch.empty_like(u), torch.empty_like(k)
+        t = cg.compton_submit(ctx, u, k, uo, ko, dens, 6, 1, 2)
+        res = _wait(cg, ctx, [t])
+        torch.cuda.synchronize()
+        assert torch.equal(uo, ref[0]) and torch.equal(ko, ref[1]) and res[t]["scatters"] == ref[2]
+        assert cg.compton_kernel_times(ctx)["k_mlp"]["launches"] <= launches
+    finally:
+        cg.compton_destroy(ctx)
+
+
+def test_more_candidates_than_a_small_pools_list_holds():
+    # 2^18 candidates a launch; requests of mixed modes, scalar and per-pair densities
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    cg.build()
+    ctx = _ctx(cg, 400003)
+    try:
+        cg.compton_serve_start(ctx, 1 << 24, 64)
+        jobs = []
+        for i, (n, mode) in enumerate(((400003, 2), (150000, 1), (300001, 3), (5000, 0), (400003, 1), (200001, 2))):
+            u, k = _pairs(torch, n, 80 + i)
+            dens = torch.rand(n, device="cuda") * 200 if i % 2 == 0 else 200.0
+            ref = _direct(cg, torch, ctx, u, k, dens, 3 + i, 1, mode)
+            uo, ko = torch.empty_like(u), torch.empty_like(k)
+            jobs.append((cg.compton_submit(ctx, u, k, uo, ko, dens, 3 + i, 1, mode), uo, ko, ref, u, k, dens))
+        res = _wait(cg, ctx, [j[0] for j in jobs])
+        torch.cuda.synchronize()
+        for t, uo, ko, (ur, kr, hits), *_ in jobs:
+            assert torch.equal(uo, ur) and torch.equal(ko, kr)
+            assert res[t]["scatters"] == hits
+        assert cg.compton_get_stats(ctx, reset=True)["pairs_tested"] == 2 * sum(j[1].shape[1] for j in jobs)
+        assert cg.compton_serve_info(ctx)["in_use"] == 0
+    finally:
+        cg.compton_destroy(ctx)
