@@ -84,3 +84,38 @@ def test_silu_f32_at_the_ends_of_its_range():
     assert np.isinf(high[-1]) and high[-1] > 0 and np.all(np.abs(high[:-1].astype(np.float64) / ends[:-1] - 1.0) <= 5e-7)
     assert np.all(low <= 0.0) and np.all(low >= -1.5e-36)
     assert np.isnan(out[-1])
+
+
+@pytest.mark.parametrize("n", [1, 31, 32, 33, 1000, 4097])
+def test_calibration_sees_the_samples_alone(n):
+    """The FP8 scales are 448 over the largest |input| of each hidden layer over
+    the n samples, whatever fills the rest of a tile: against the FP64 maxima, to
+    the FP32 forward's 64-term sums (relative 2e-5; biases apart from zero, so that
+    a sample of zeros would show)."""
+    import paper_2206_02937_gb300 as cg
+    torch = torch_cuda()
+    cg.build()
+    th = _theta(7, gain=1.5)
+    off = [384, 4544, 8704, 12864]  # the hidden layers' biases
+    rng = np.random.default_rng(8)
+    for o in off:
+        th[o:o + 64] = rng.uniform(1.0, 2.0, 64)
+    th = th.astype(np.float32)
+    u, k = wl.c3(n, seed=41)
+    t = th.astype(np.float64)
+    h, want = omlp.features(u, k).T, []
+    for l, (o, i) in enumerate(((64, 6), (64, 64), (64, 64))):
+        at = (0, 448, 4608)[l]
+        want.append(np.abs(h).max())
+        z = h @ t[at:at + o * i].reshape(o, i).T + t[at + o * i:at + o * i + o]
+        h = z / (1.0 + np.exp(-z))
+    want.append(np.abs(h).max())
+    ctx = cg.compton_init(1, 1, 1.0, 0.05, 1)
+    try:
+        cg.compton_mlp_set_params(ctx, th)
+        cg.compton_mlp_calibrate(ctx, torch.from_numpy(u).cuda(), torch.from_numpy(k).cuda())
+        torch.cuda.synchronize()
+        scales = np.frombuffer(cg.compton_mlp_save(ctx)[40:56], np.float32)
+    finally:
+        cg.compton_destroy(ctx)
+    assert np.allclose(scales, 448.0 / np.array(want), rtol=2e-5, atol=0.0)
