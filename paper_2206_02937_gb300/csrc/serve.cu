@@ -364,6 +364,8 @@ struct ServeEngine {
     compton_ctx* ctx = nullptr;
     int device = 0;
     void* pool = nullptr;
+    void* dev = nullptr;   // the lists below on the device
+    void* host = nullptr;  // and those on the host, pinned
     size_t pool_bytes = 0;
     std::map<size_t, size_t> free_blocks;  // offset -> size
     size_t in_use = 0, peak_in_use = 0;
@@ -771,20 +773,44 @@ compton_status serve_start(compton_ctx* ctx, uint64_t pool_bytes, int32_t max_ac
     // with 2^21 and no work spent on tiles that find the list full.
     E->list_cap = (uint32_t)std::min<uint64_t>(kServeListMax, std::max<uint64_t>(kServeListMin, pool_bytes / 64));
     cudaError_t e = inject_fault() ? cudaErrorMemoryAllocation : cudaMalloc(&E->pool, pool_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&E->reqs_dev, sizeof(ReqDev) * max_active);
-    if (e == cudaSuccess) e = cudaMalloc(&E->counters, sizeof(unsigned long long) * max_active);
-    if (e == cudaSuccess) e = cudaMalloc(&E->tiles_dev, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
-    if (e == cudaSuccess) e = cudaMallocHost(&E->reqs_host, sizeof(ReqDev) * max_active);
-    if (e == cudaSuccess) e = cudaMallocHost(&E->tiles_host, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
-    if (e == cudaSuccess) e = cudaMallocHost(&E->scat_host, sizeof(unsigned long long) * max_active * kTileRing);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.cand, sizeof(CandPair) * E->list_cap);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.accepted, sizeof(AcceptedPair) * E->list_cap);
-    if (e == cudaSuccess) e = cudaMalloc(&E->list.r, sizeof(float) * E->list_cap);
-    if (e == cudaSuccess) e = cudaMalloc(&E->ctl_dev, sizeof(ServeControl));
-    if (e == cudaSuccess) e = cudaMallocHost(&E->ctl_host, sizeof(ServeControl) * kTileRing);
+    // one allocation each for the device's and the host's (pinned) lists
+    const size_t slots = (size_t)max_active;
+    size_t dev_bytes = 0, host_bytes = 0;
+    const auto take = [](size_t& used, size_t bytes) {
+        const size_t at = used;
+        used += align256(bytes);
+        return at;
+    };
+    const size_t d_cand = take(dev_bytes, sizeof(CandPair) * E->list_cap);
+    const size_t d_acc = take(dev_bytes, sizeof(AcceptedPair) * E->list_cap);
+    const size_t d_r = take(dev_bytes, sizeof(float) * E->list_cap);
+    const size_t d_tiles = take(dev_bytes, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
+    const size_t d_reqs = take(dev_bytes, sizeof(ReqDev) * slots);
+    const size_t d_counters = take(dev_bytes, sizeof(unsigned long long) * slots);
+    const size_t d_ctl = take(dev_bytes, sizeof(ServeControl));
+    const size_t h_tiles = take(host_bytes, sizeof(TileDev) * kMaxTilesPerLaunch * kTileRing);
+    const size_t h_reqs = take(host_bytes, sizeof(ReqDev) * slots);
+    const size_t h_scat = take(host_bytes, sizeof(unsigned long long) * slots * kTileRing);
+    const size_t h_ctl = take(host_bytes, sizeof(ServeControl) * kTileRing);
+    if (e == cudaSuccess) e = cudaMalloc(&E->dev, dev_bytes);
+    if (e == cudaSuccess) e = cudaMallocHost(&E->host, host_bytes);
+    if (e == cudaSuccess) {
+        char* d = static_cast<char*>(E->dev);
+        char* h = static_cast<char*>(E->host);
+        E->list.cand = reinterpret_cast<CandPair*>(d + d_cand);
+        E->list.accepted = reinterpret_cast<AcceptedPair*>(d + d_acc);
+        E->list.r = reinterpret_cast<float*>(d + d_r);
+        E->tiles_dev = reinterpret_cast<TileDev*>(d + d_tiles);
+        E->reqs_dev = reinterpret_cast<ReqDev*>(d + d_reqs);
+        E->counters = reinterpret_cast<unsigned long long*>(d + d_counters);
+        E->ctl_dev = reinterpret_cast<ServeControl*>(d + d_ctl);
+        E->tiles_host = reinterpret_cast<TileDev*>(h + h_tiles);
+        E->reqs_host = reinterpret_cast<ReqDev*>(h + h_reqs);
+        E->scat_host = reinterpret_cast<unsigned long long*>(h + h_scat);
+        E->ctl_host = reinterpret_cast<ServeControl*>(h + h_ctl);
+    }
     if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&E->s_compute, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMemset(E->counters, 0, sizeof(unsigned long long) * max_active);
-    if (e == cudaSuccess) e = cudaDeviceSynchronize();
+    if (e == cudaSuccess) e = cudaMemsetAsync(E->counters, 0, sizeof(unsigned long long) * slots, E->s_compute);
     if (e != cudaSuccess) {
         cudaGetLastError();
         serve_stop_free(E);
@@ -803,17 +829,8 @@ compton_status serve_start(compton_ctx* ctx, uint64_t pool_bytes, int32_t max_ac
 void serve_stop_free(ServeEngine* E)
 {
     if (E->pool) cudaFree(E->pool);
-    if (E->reqs_dev) cudaFree(E->reqs_dev);
-    if (E->counters) cudaFree(E->counters);
-    if (E->tiles_dev) cudaFree(E->tiles_dev);
-    if (E->reqs_host) cudaFreeHost(E->reqs_host);
-    if (E->tiles_host) cudaFreeHost(E->tiles_host);
-    if (E->scat_host) cudaFreeHost(E->scat_host);
-    if (E->list.cand) cudaFree(E->list.cand);
-    if (E->list.accepted) cudaFree(E->list.accepted);
-    if (E->list.r) cudaFree(E->list.r);
-    if (E->ctl_dev) cudaFree(E->ctl_dev);
-    if (E->ctl_host) cudaFreeHost(E->ctl_host);
+    if (E->dev) cudaFree(E->dev);
+    if (E->host) cudaFreeHost(E->host);
     if (E->s_compute) cudaStreamDestroy(E->s_compute);
     for (auto& L : E->inflight)
         if (L.ev) cudaEventDestroy(L.ev);
