@@ -1162,16 +1162,17 @@ compton_status launch_scatter_ntc(compton_ctx* ctx, compton_species* e, compton_
     COMPTON_CUDA_TRY(ctx, cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_ntc<8>, 32 * kNtcWarps, 0));
     if (per_sm < 1) per_sm = 1;
     int64_t blocks = (int64_t)ctx->n_sm * per_sm;
-    // runs of 32 cells where every resident warp gets one, or where 32 cells
-    // have no more candidates than a batch; else runs of 8, which spread the
-    // cells better.  A run costs its warp an atomic and a chain of loads however
-    // few candidates it has.  16 + 16 particles a cell with 0.5 candidates, runs
-    // of 8 and of 32: 100,000 cells 40 and 35 us, 262,144 cells 59 and 44;
-    // 2 million cells of 8 + 8 with one 303 and 161; 262,144 cells of 64 + 64
-    // with 4 113 and 105, with 10 135 and 144.
+    // runs of 32 cells where 32 cells have no more candidates than a batch, or
+    // where a resident warp gets half as many such runs as a cell has candidates;
+    // else runs of 8, which spread the cells better.  A run costs its warp an atomic
+    // and a chain of loads however few candidates it has.  k_ntc's step in us with
+    // runs of 8 and of 32: 262,144 cells of 16 + 16 with 0.5 candidates each 59 and
+    // 43, of 64 + 64 with 4 108 and 104, with 10 136 and 144; a million cells of 16
+    // + 16 with 10 408 and 390, with 40 1497 and 1527; 2 million cells of 8 + 8 with
+    // one 300 and 161.
     const double mean = (double)e->n / (double)pairs->n_cells * (double)g->n / (double)pairs->n_cells * a.w_over_v *
                         2.0 * a.dt;
-    const bool many = mean < 1.0 || pairs->n_cells >= 32 * kNtcWarps * blocks;
+    const bool many = mean < 1.0 || (double)pairs->n_cells >= 16.0 * mean * (double)(kNtcWarps * blocks);
     const int cells = many ? 32 : 8;
     // a warp per run of cells at most
     const int64_t need = (pairs->n_cells + cells * kNtcWarps - 1) / (cells * kNtcWarps);
