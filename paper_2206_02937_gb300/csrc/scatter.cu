@@ -387,7 +387,17 @@ __global__ void __launch_bounds__(kResolve ? 32 * kResolveWarps : kProbThreads, 
                     thr = kWeighted ? cand_threshold(dens, a.dt) : W.thr[cr];
                 } else if (kBinned) {
                     // a tile of more cells than the window: cells in global memory
-                    while (ci + 1 < nw && cw[ci + 1].pair_off <= p) ++ci;
+                    if (kResolve) {
+                        // few pairs among many cells: past the next cell by bisection
+                        int lo = ci, hi = ci + 1 < nw && cw[ci + 1].pair_off <= p ? nw - 1 : ci;
+                        while (lo < hi) {
+                            const int mid = (lo + hi + 1) >> 1;
+                            if (cw[mid].pair_off <= p) lo = mid; else hi = mid - 1;
+                        }
+                        ci = lo;
+                    } else {
+                        while (ci + 1 < nw && cw[ci + 1].pair_off <= p) ++ci;
+                    }
                     if (ci != cur) {
                         cur = ci;
                         const CellInfo c = cw[ci];
