@@ -304,7 +304,7 @@ compton_status compton_mlp_train_step(struct compton_ctx* ctx, const float* ux_d
 /* Arithmetic of the following compton_mlp_train_step calls (Sec. 3.2
  * trains the network; the precision is this library's choice).
  * COMPTON_MODE_MLP_FP32 (the default): forward and backward in FP32 on the
- * CUDA cores, one sample per thread.  COMPTON_MODE_MLP_BF16: every
+ * CUDA cores, tiles of 64 samples.  COMPTON_MODE_MLP_BF16: every
  * contraction (forward z = a W^T, backward delta W and the weight gradients
  * delta^T a) on the tcgen05 tensor cores with BF16 operands and FP32
  * accumulation in tensor memory, 128-sample tiles, one CTA per SM holding all
@@ -442,8 +442,9 @@ typedef struct compton_result {
 } compton_result;
 
 /* Start the serving engine: a device pool of pool_bytes (the memory budget;
- * each admitted request holds 28 bytes per pair, 32 in surrogate modes) and
- * at most max_active requests admitted at once.  The pool is allocated here,
+ * each admitted request is charged 28 bytes per pair, 32 in surrogate modes,
+ * and its inputs are staged there if its outputs overlap them other than pair
+ * by pair) and at most max_active requests admitted at once.  The pool is allocated here,
  * once, with the engine's own lists beside it (100 bytes for each 64 of the
  * pool, at least 29 MB and at most 213 MB).  EINVAL if already started. */
 compton_status compton_serve_start(struct compton_ctx* ctx, uint64_t pool_bytes, int32_t max_active);
@@ -507,11 +508,15 @@ compton_status compton_cell_offsets_noalloc(const int32_t* cell_dev, int64_t n, 
 
 /* Kernel slots of compton_kernel_times. */
 typedef enum compton_kernel_slot {
-    COMPTON_K_COUNT = 0,   /* histogram and order check                    */
+    COMPTON_K_COUNT = 0,   /* histogram and order check; in a small call (at most
+                              4096 cells, and 16384 particles of both species
+                              together) all of the binning before the sort, and
+                              the next two slots record nothing            */
     COMPTON_K_SCAN = 1,    /* the scan kernels together                    */
     COMPTON_K_PLACE = 2,   /* keyed placement (shuffled input)             */
     COMPTON_K_SORT = 3,    /* per-cell sort and sorted copy                */
-    COMPTON_K_PROB = 4,    /* probability and Bernoulli trial of all pairs */
+    COMPTON_K_PROB = 4,    /* probability and Bernoulli trial of all pairs; up to
+                              32768 pairs of a plain step the collisions too */
     COMPTON_K_COLLIDE = 5, /* collisions of the accepted pairs             */
     COMPTON_K_MLP = 6,     /* surrogate network forward                    */
     COMPTON_K_NTC = 7,     /* No-Time-Counter candidates and collisions    */

@@ -84,16 +84,6 @@ __device__ __forceinline__ float pair_density(const ScatterArgs& a, float cell_d
     return cell_dens * fmaxf(we, wg);
 }
 
-__device__ __forceinline__ int find_cell(const CellInfo* win, int nwin, int64_t p)
-{
-    int lo = 0, hi = nwin - 1;
-    while (lo < hi) {
-        const int mid = (lo + hi + 1) >> 1;
-        if ((int64_t)win[mid].pair_off <= p) lo = mid; else hi = mid - 1;
-    }
-    return lo;
-}
-
 // The collision of one accepted pair, written back in place.
 __device__ __forceinline__ void resolve(const ScatterArgs& a, const AcceptedPair& e)
 {

@@ -27,8 +27,8 @@
 // otherwise than output on its own input.  Only candidates (pairs whose uniform
 // lies below the bound of every probability) are evaluated, and only they pass
 // through the network, all requests' together.  24 requests of 1,155 to 866,000
-// pairs, half of them for the BF16 network: 2264 us with a staged copy of every
-// array each way and a network pass per request, 430 us so.
+// pairs, half of them for the BF16 network: 2274 us with a staged copy of every
+// array each way and a network pass per request, 414 us so.
 //
 // Every pair of request r uses Philox counter (pair index within r, step_r)
 // under key seed_r, so a request's result does not depend on what it shares
