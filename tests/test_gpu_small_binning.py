@@ -68,3 +68,19 @@ def test_one_species_empty():
     w = _random_workload(41, n_cells=50, ppc_e=20, ppc_g=20)
     w.g = {k: v[:0] for k, v in w.g.items()}
     compare_with_oracle(w)
+
+
+@pytest.mark.parametrize("cells", [65, 4096, 6000])
+@pytest.mark.parametrize("n_e", [1, 10, 200, 3000])
+def test_few_pairs_among_many_cells(n_e, cells):
+    """Pairs whose cells lie far apart, more cells than a warp's window holds
+    between two of them (the cell of a pair is then found by bisection)."""
+    from paper_2206_02937_gb300 import workloads as wl
+    from tests.test_gpu_parity import compare_with_oracle
+    rng = wl.rng_for(cells + n_e)
+    n_g = 12000
+    ce, cg = rng.integers(0, cells, n_e), rng.integers(0, cells, n_g)
+    ce[0] = cells - 1
+    u = 3.0 * wl.isotropic(rng, n_e)
+    k = 10 ** rng.uniform(-4, 0, n_g) * wl.isotropic(rng, n_g)
+    compare_with_oracle(wl.Workload("few pairs", cells, 0.1, 1.0, 17, 1, wl._species(u, ce), wl._species(k, cg)), step=4)
