@@ -46,9 +46,9 @@ __device__ __forceinline__ unsigned lane_id() { return threadIdx.x & 31u; }
 // unsorted[s] counts the positions at which the cell index descends, plus one
 // per warp that saw an index outside [0, C): only if it is not zero does the
 // placement run, and by its size the placement takes its form (sort_source).
-// In large input each warp also looks at its last 128 positions: unsorted[2 + s]
-// counts the positions of the warps in whose stretch neighbours in the input are
-// not neighbours in the cells (scattered).
+// In large input every fourth warp also looks at its last 128 positions:
+// unsorted[2 + s] counts the positions (four times a stretch) of those in whose
+// stretch neighbours in the input are not neighbours in the cells (scattered).
 //
 // What bounds it: instruction issue (113 instructions per 128 positions of input
 // in cell order; 140 when every position was looked at as first and last of its
@@ -154,13 +154,13 @@ __global__ void __launch_bounds__(kCountThreads, sizeof(Idx) == 4 ? 2 : 1) k_cou
     }
     const bool any_bad = __any_sync(0xffffffffu, bad);
     descents = __reduce_add_sync(0xffffffffu, descents);
-    // (where a quarter of the stretch descends the order is settled)
-    const bool apart = (int64_t)n > kScatterLook && begin < stop && stop <= n &&
+    // every fourth warp, for four (where a quarter of the stretch descends the order is settled)
+    const bool apart = (int64_t)n > kScatterLook && (w & 3) == 0 && begin < stop && stop <= n &&
                        (int64_t)descents * 4 < (int64_t)(stop - begin) && scattered(v, (int64_t)n, C, max_runs);
     if (lane == 0) {
         if (any_bad) atomicOr(&stats->error_flags, (unsigned long long)kErrCellRange);
         if (descents + any_bad) atomicAdd(&unsorted[s], descents + any_bad);
-        if (apart) atomicAdd(&unsorted[2 + s], (uint32_t)(stop - begin));
+        if (apart) atomicAdd(&unsorted[2 + s], 4u * (uint32_t)(stop - begin));
     }
 }
 
